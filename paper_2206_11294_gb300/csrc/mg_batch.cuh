@@ -124,12 +124,13 @@ __global__ void __launch_bounds__(kBatchThreads) kb_restrict(const BLevel *__res
         const int gx = (Cc.n0 + kBX - 1) / kBX, gy = (Cc.n1 + kBY - 1) / kBY;
         int bx, by, bz;
         block_coords(e.y, gx, gy, bx, by, bz);
-        if (red) residual_restrict_block<R, DIM, true, true>(F, Cc, bx, by, bz);
-        else residual_restrict_block<R, DIM, true, false>(F, Cc, bx, by, bz);
+        if (red) residual_restrict_block<R, DIM, true, true>(F, Cc, 1, bx, by, bz);
+        else residual_restrict_block<R, DIM, true, false>(F, Cc, 0, bx, by, bz);
     }
 }
 
-template <typename R, int DIM>
+// BLACK: red-black sweeps follow, the black cells only (prolong_add_block), over the colour sweeps' table.
+template <typename R, int DIM, bool BLACK>
 __global__ void __launch_bounds__(kBatchThreads) kb_prolong(const BLevel *__restrict__ lv,
                                                             const BState *__restrict__ st,
                                                             const int2 *__restrict__ tab, int n) {
@@ -140,10 +141,10 @@ __global__ void __launch_bounds__(kBatchThreads) kb_prolong(const BLevel *__rest
         const Level<R> F = pick<R>(B);
         const Level<R> Cc = pick<R>(lv[e.x + 1]);
         const BcFlags bc = B.bc;
-        const int gx = (F.n0 + kBX - 1) / kBX, gy = (F.n1 + kBY - 1) / kBY;
+        const int gx = ((BLACK ? (F.n0 + 1) / 2 : F.n0) + kBX - 1) / kBX, gy = (F.n1 + kBY - 1) / kBY;
         int bx, by, bz;
         block_coords(e.y, gx, gy, bx, by, bz);
-        prolong_add_block<R, DIM>(Cc, F, bc, bx, by, bz);
+        prolong_add_block<R, DIM, true, BLACK>(Cc, F, bc, bx, by, bz);
     }
 }
 
@@ -472,7 +473,7 @@ template <int DIM>
 __global__ void __launch_bounds__(kBatchThreads) kb_residual64(const BLevel *__restrict__ lv,
                                                                const BProb *__restrict__ pr, BState *__restrict__ st,
                                                                const int2 *__restrict__ tab, int n, int initial,
-                                                               double rtol, int max_cycles,
+                                                               int red_start, double rtol, int max_cycles,
                                                                int *__restrict__ active_count) {
     for (int v = blockIdx.x; v < n; v += gridDim.x) {
         __syncthreads();
@@ -487,7 +488,7 @@ __global__ void __launch_bounds__(kBatchThreads) kb_residual64(const BLevel *__r
         // form r0 - A delta
         if (!initial) L.x = B.delta;
         const double2 s = residual64_to32_block<DIM>(L, B.f.b, B.f.bt, B.f.x, initial ? L.b : nullptr,
-                                                     initial ? B.delta : nullptr, bx, by, bz);
+                                                     initial ? B.delta : nullptr, red_start, bx, by, bz);
         batch_finish(pr[p], st[p], e.y, s, initial, rtol, max_cycles, active_count);
     }
 }
@@ -593,8 +594,9 @@ void b_fused_pair(mg_batch *b, cudaStream_t s, int d, int t) {
     kb_rbgs_fused2d<R, TX, TY><<<batch_grid(b, nf), kBlock, 0, s>>>(b->lv, b->st, ft, nf, 0);
 }
 
+// red_done: the guess is zero with the first red half-sweep applied (enqueue_sweeps).
 template <typename R, int DIM>
-void b_smooth(mg_batch *b, cudaStream_t s, int d, int sweeps) {
+void b_smooth(mg_batch *b, cudaStream_t s, int d, int sweeps, bool red_done = false) {
     const int2 *ct = b->tabs + b->colour[d].first;
     const int nc = b->colour[d].second;
     int q = 0;
@@ -607,18 +609,19 @@ void b_smooth(mg_batch *b, cudaStream_t s, int d, int sweeps) {
             b->launches += 2;
         }
     }
-    for (; q < sweeps; q++) {
-        kb_rbgs_colour<R, DIM><<<batch_grid(b, nc), kBlock, 0, s>>>(b->lv, b->st, ct, nc, 0);
-        kb_rbgs_colour<R, DIM><<<batch_grid(b, nc), kBlock, 0, s>>>(b->lv, b->st, ct, nc, 1);
-        b->launches += 2;
-    }
+    for (; q < sweeps; q++)
+        for (int colour = red_done && q == 0 ? 1 : 0; colour < 2; colour++) {
+            kb_rbgs_colour<R, DIM><<<batch_grid(b, nc), kBlock, 0, s>>>(b->lv, b->st, ct, nc, colour);
+            b->launches++;
+        }
 }
 
+// red_done: the finest level's guess is zero with the first red half-sweep applied.
 template <typename R, int DIM>
-void b_vcycle(mg_batch *b, cudaStream_t s) {
+void b_vcycle(mg_batch *b, cudaStream_t s, bool red_done = false) {
     for (int d = 0; d + 1 < b->dmax; d++) {
         if (b->colour[d].second == 0) continue;
-        b_smooth<R, DIM>(b, s, d, b->opt.nu1);
+        b_smooth<R, DIM>(b, s, d, b->opt.nu1, d > 0 || red_done);
         const int nr = b->restr[d].second;
         kb_restrict<R, DIM><<<batch_grid(b, nr), kBlock, 0, s>>>(b->lv, b->st, b->tabs + b->restr[d].first, nr,
                                                               b->opt.nu1 > 0);
@@ -637,8 +640,13 @@ void b_vcycle(mg_batch *b, cudaStream_t s) {
     }
     for (int d = b->dmax - 2; d >= 0; d--) {
         if (b->colour[d].second == 0) continue;
-        const int np = b->prolong[d].second;
-        kb_prolong<R, DIM><<<batch_grid(b, np), kBlock, 0, s>>>(b->lv, b->st, b->tabs + b->prolong[d].first, np);
+        if (b->opt.nu2 > 0) {
+            const int np = b->colour[d].second;
+            kb_prolong<R, DIM, true><<<batch_grid(b, np), kBlock, 0, s>>>(b->lv, b->st, b->tabs + b->colour[d].first, np);
+        } else {
+            const int np = b->prolong[d].second;
+            kb_prolong<R, DIM, false><<<batch_grid(b, np), kBlock, 0, s>>>(b->lv, b->st, b->tabs + b->prolong[d].first, np);
+        }
         b->launches++;
         b_smooth<R, DIM>(b, s, d, b->opt.nu2);
     }
@@ -654,7 +662,8 @@ void b_norm(mg_batch *b, cudaStream_t s, int initial) {
                                                       b->active_count);
     else
         kb_residual64<DIM><<<batch_grid(b, n), kBlock, 0, s>>>(b->lv, b->pr, b->st, b->tabs + b->norm.first, n, initial,
-                                                            b->opt.rtol, b->opt.max_cycles, b->active_count);
+                                                            b->opt.nu1 > 0, b->opt.rtol, b->opt.max_cycles,
+                                                            b->active_count);
     b->launches++;
     cudaMemcpyAsync(b->active_h, b->active_count, sizeof(int), cudaMemcpyDeviceToHost, s);
 }
@@ -755,7 +764,7 @@ void b_step(mg_batch *b, cudaStream_t s) {
     if (b->opt.precision == MG_FP64) {
         b_vcycle<double, DIM>(b, s);
     } else {
-        for (int q = 0; q < b->opt.inner_cycles; q++) b_vcycle<float, DIM>(b, s);
+        for (int q = 0; q < b->opt.inner_cycles; q++) b_vcycle<float, DIM>(b, s, q == 0);
         const int n = b->cells0.second;
         kb_add_correction<<<batch_grid(b, n), kBatchThreads, 0, s>>>(b->lv, b->st, b->tabs + b->cells0.first, n);
         b->launches++;

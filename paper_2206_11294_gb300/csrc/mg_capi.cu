@@ -610,8 +610,12 @@ void launch_fused_tma(const mg_handle *h, int l, int tile, const Level<R> &v, cu
 // sweep (and every non-fused sweep) runs as two colour launches in place.
 // alt: the values start in xalt (only after fused pairs).  Returns whether
 // they end in xalt.  The values are the same, bit for bit, for every choice.
+// red_done: x already is the state after the first red half-sweep (from a zero
+// guess, see residual_restrict_block): colour sweeps start with the black one;
+// the fused kinds recompute the red values they are given.
 template <typename R, int DIM>
-bool enqueue_sweeps(const mg_handle *h, cudaStream_t s, int l, int sweeps, int kind, int tile, bool alt = false) {
+bool enqueue_sweeps(const mg_handle *h, cudaStream_t s, int l, int sweeps, int kind, int tile, bool alt = false,
+                    bool red_done = false) {
     using V2 = typename Vec<R>::v2;
     const LevelBuf &lb = h->L[l];
     Level<R> v = view<R>(lb);
@@ -648,21 +652,21 @@ bool enqueue_sweeps(const mg_handle *h, cudaStream_t s, int l, int sweeps, int k
     if (kind == MG_SWEEP_COLOUR2) {
         const dim3 g2(gr.x, (unsigned)((lb.n[1] + 2 * kBY - 1) / (2 * kBY)), gr.z);
         for (; q < sweeps; q++) {
-            launch_k(h, k_rbgs_colour2<R, DIM>, g2, kBlock, 0, s, 0, v, 0);
-            launch_k(h, k_rbgs_colour2<R, DIM>, g2, kBlock, 0, s, 0, v, 1);
-            counted(h, 2);
+            const int first = red_done && q == 0 ? 1 : 0;
+            for (int colour = first; colour < 2; colour++) launch_k(h, k_rbgs_colour2<R, DIM>, g2, kBlock, 0, s, 0, v, colour);
+            counted(h, 2 - first);
         }
     }
     for (; q < sweeps; q++) {
-        if (h->persistent) {
-            const unsigned gw = wave((const void *)k_rbgs_colour<R, DIM, true>, tiles_of(gr));
-            launch_k(h, k_rbgs_colour<R, DIM, true>, gw, kBlock, 0, s, 0, v, 0);
-            launch_k(h, k_rbgs_colour<R, DIM, true>, gw, kBlock, 0, s, 0, v, 1);
-        } else {
-            launch_k(h, k_rbgs_colour<R, DIM, false>, gr, kBlock, 0, s, 0, v, 0);
-            launch_k(h, k_rbgs_colour<R, DIM, false>, gr, kBlock, 0, s, 0, v, 1);
+        const int first = red_done && q == 0 ? 1 : 0;
+        for (int colour = first; colour < 2; colour++) {
+            if (h->persistent)
+                launch_k(h, k_rbgs_colour<R, DIM, true>, wave((const void *)k_rbgs_colour<R, DIM, true>, tiles_of(gr)),
+                         kBlock, 0, s, 0, v, colour);
+            else
+                launch_k(h, k_rbgs_colour<R, DIM, false>, gr, kBlock, 0, s, 0, v, colour);
         }
-        counted(h, 2);
+        counted(h, 2 - first);
     }
     return v.x != xm;
 }
@@ -691,12 +695,12 @@ void enqueue_wjac(const mg_handle *h, cudaStream_t s, int l, int sweeps) {
 // Returns whether the level's values end in xalt (fused pairs only; alt:
 // they start there).
 template <typename R, int DIM>
-bool enqueue_smooth(const mg_handle *h, cudaStream_t s, int l, int sweeps, bool alt = false) {
+bool enqueue_smooth(const mg_handle *h, cudaStream_t s, int l, int sweeps, bool alt = false, bool red_done = false) {
     if (h->opt.smoother == MG_SMOOTH_WJAC) {
         enqueue_wjac<R, DIM>(h, s, l, sweeps);
         return false;
     }
-    return enqueue_sweeps<R, DIM>(h, s, l, sweeps, h->sweep[l], h->tile[l], alt);
+    return enqueue_sweeps<R, DIM>(h, s, l, sweeps, h->sweep[l], h->tile[l], alt, red_done);
 }
 
 // Fused pairs leave a level's values in xalt after an odd number of pairs;
@@ -709,6 +713,17 @@ bool fused2_ok(const mg_options &o, int dim) {
 // so the restriction after pre-smoothing evaluates the red children only and
 // the norm after post-smoothing the red cells only; Jacobi leaves no such zeros.
 bool red_only_after_sweeps(const mg_handle *h) { return h->opt.smoother == MG_SMOOTH_RBGS; }
+
+// A level whose guess is zero starts from the state after the first red
+// half-sweep (red_start of the kernels that write the guess).
+int red_start(const mg_handle *h) { return h->opt.smoother == MG_SMOOTH_RBGS && h->opt.nu1 > 0 ? 1 : 0; }
+
+// Whether the timed pre-smoothing of the finest level begins after its first
+// sweep: with that state as its start, the sweep is one launch, not two.
+bool timed_after_first(const mg_handle *h) {
+    return h->opt.precision == MG_MIXED && h->opt.inner_cycles == 1 && red_start(h) && h->opt.nu1 > 1 &&
+           (h->sweep[0] == MG_SWEEP_COLOUR || h->sweep[0] == MG_SWEEP_COLOUR2);
+}
 
 // The tail kernel runs red-black V-cycles.
 bool tail_runs(const mg_handle *h) { return h->opt.cycle == MG_CYCLE_V && h->opt.smoother == MG_SMOOTH_RBGS; }
@@ -756,14 +771,15 @@ void enqueue_tail(const mg_handle *h, cudaStream_t s) {
 }
 
 template <typename R, int DIM>
-void enqueue_vcycle(const mg_handle *h, cudaStream_t s, int l, int type);
+void enqueue_vcycle(const mg_handle *h, cudaStream_t s, int l, int type, bool red_done = false);
 
 template <typename R, int DIM>
 // One cycle from level l: V, or (type) W / F, whose coarse-grid correction
 // visits level l + 1 twice (W then W, F then V), the second visit continuing
 // from the first one's coarse solution, except at the exactly solved coarsest
 // level.  The tail kernel runs V-cycles only, so W and F cycles never use it.
-void enqueue_vcycle(const mg_handle *h, cudaStream_t s, int l, int type) {
+// red_done: the level's guess is zero with the first red half-sweep applied.
+void enqueue_vcycle(const mg_handle *h, cudaStream_t s, int l, int type, bool red_done) {
     const LevelBuf &lb = h->L[l];
     if (l == h->tail_lev && tail_runs(h)) {
         // the coarsest inverse is computed on the aux stream after each set-up
@@ -800,36 +816,45 @@ void enqueue_vcycle(const mg_handle *h, cudaStream_t s, int l, int type) {
     // per cycle, not four: each costs the step a little)
     const bool tm_pre = h->timing && !h->cond_body && l == 0 && h->opt.nu1 > 0;
     const bool tm_post = h->timing && !h->cond_body && l == 0 && h->opt.nu1 == 0;
+    int nu1 = h->opt.nu1;
+    if (tm_pre && red_done && timed_after_first(h)) {
+        enqueue_smooth<R, DIM>(h, s, l, 1, false, true);
+        nu1--;
+        red_done = false;
+    }
     if (tm_pre) cudaEventRecordWithFlags(h->ev[0], s, cudaEventRecordExternal);
-    const bool alt = enqueue_smooth<R, DIM>(h, s, l, h->opt.nu1);
+    const bool alt = enqueue_smooth<R, DIM>(h, s, l, nu1, false, red_done);
     if (tm_pre) cudaEventRecordWithFlags(h->ev[1], s, cudaEventRecordExternal);
     // the level's values, where the smoothing left them
     Level<R> vl = view<R>(lb);
     if (alt) vl.x = xalt_of<R>(lb);
     const dim3 rg = cell_grid(cb, DIM, cb.n[0]);
-    if (h->opt.nu1 > 0 && red_only_after_sweeps(h)) {
+    auto restrict_with = [&](auto tile, auto wave_of) {
         if (h->persistent)
-            launch_k(h, k_residual_restrict<R, DIM, true, true>, wave((const void *)k_residual_restrict<R, DIM, true, true>, tiles_of(rg)), kBlock, 0, s, 0, vl,
-                                                                                                          view<R>(cb));
+            launch_k(h, wave_of, wave((const void *)wave_of, tiles_of(rg)), kBlock, 0, s, 0, vl, view<R>(cb), red_start(h));
         else
-            launch_k(h, k_residual_restrict<R, DIM, true, false>, rg, kBlock, 0, s, 0, vl, view<R>(cb));
-    } else {
-        if (h->persistent)
-            launch_k(h, k_residual_restrict<R, DIM, false, true>, wave((const void *)k_residual_restrict<R, DIM, false, true>, tiles_of(rg)), kBlock, 0, s, 0, 
-                    vl, view<R>(cb));
-        else
-            launch_k(h, k_residual_restrict<R, DIM, false, false>, rg, kBlock, 0, s, 0, vl, view<R>(cb));
-    }
+            launch_k(h, tile, rg, kBlock, 0, s, 0, vl, view<R>(cb), red_start(h));
+    };
+    if (h->opt.nu1 > 0 && red_only_after_sweeps(h))
+        restrict_with(k_residual_restrict<R, DIM, true, false>, k_residual_restrict<R, DIM, true, true>);
+    else
+        restrict_with(k_residual_restrict<R, DIM, false, false>, k_residual_restrict<R, DIM, false, true>);
     counted(h);
-    enqueue_vcycle<R, DIM>(h, s, l + 1, type);
+    enqueue_vcycle<R, DIM>(h, s, l + 1, type, red_start(h) != 0);
     if (type != MG_CYCLE_V && l + 1 < h->nlev - 1)
         enqueue_vcycle<R, DIM>(h, s, l + 1, type == MG_CYCLE_W ? MG_CYCLE_W : MG_CYCLE_V);
-    const dim3 pg = cell_grid(lb, DIM, lb.n[0]);
-    if (h->persistent)
-        launch_k(h, k_prolong_add<R, DIM, true>, wave((const void *)k_prolong_add<R, DIM, true>, tiles_of(pg)), kBlock, 0, s, 0, 
-            view<R>(cb), vl, bc_flags(h->grid));
-    else
-        launch_k(h, k_prolong_add<R, DIM, false>, pg, kBlock, 0, s, 0, view<R>(cb), vl, bc_flags(h->grid));
+    // a red-black sweep next: the black cells only
+    const bool black = h->opt.nu2 > 0 && h->opt.smoother == MG_SMOOTH_RBGS;
+    const dim3 pg = cell_grid(lb, DIM, black ? (lb.n[0] + 1) / 2 : lb.n[0]);
+    auto prolong_with = [&](auto tile, auto wave_of) {
+        if (h->persistent)
+            launch_k(h, wave_of, wave((const void *)wave_of, tiles_of(pg)), kBlock, 0, s, 0, view<R>(cb), vl,
+                     bc_flags(h->grid));
+        else
+            launch_k(h, tile, pg, kBlock, 0, s, 0, view<R>(cb), vl, bc_flags(h->grid));
+    };
+    if (black) prolong_with(k_prolong_add<R, DIM, true, false>, k_prolong_add<R, DIM, true, true>);
+    else prolong_with(k_prolong_add<R, DIM, false, false>, k_prolong_add<R, DIM, false, true>);
     counted(h);
     if (tm_post) cudaEventRecordWithFlags(h->ev[0], s, cudaEventRecordExternal);
     const bool alt_end = enqueue_smooth<R, DIM>(h, s, l, h->opt.nu2, alt);
@@ -881,10 +906,10 @@ void enqueue_residual_to32(const mg_handle *h, cudaStream_t s, bool initial = fa
     double2 *r_out2 = initial ? delta : nullptr;
     if (h->persistent)
         launch_k(h, k_residual64_to32<DIM, true>, wave((const void *)k_residual64_to32<DIM, true>, tiles_of(ng)), kBlock, 0, s, 0, 
-            v, f.b32, f.bt32, f.x32, r_out, r_out2, h->partial, h->ticket, h->norms_d);
+            v, f.b32, f.bt32, f.x32, r_out, r_out2, red_start(h), h->partial, h->ticket, h->norms_d);
     else
-        launch_k(h, k_residual64_to32<DIM, false>, ng, kBlock, 0, s, 0, v, f.b32, f.bt32, f.x32, r_out, r_out2, h->partial,
-                                                             h->ticket, h->norms_d);
+        launch_k(h, k_residual64_to32<DIM, false>, ng, kBlock, 0, s, 0, v, f.b32, f.bt32, f.x32, r_out, r_out2,
+                 red_start(h), h->partial, h->ticket, h->norms_d);
     counted(h);
 }
 
@@ -894,7 +919,8 @@ void warm_waves_r() {
     wave((const void *)k_rbgs_colour<R, DIM, true>, 1);
     wave((const void *)k_residual_restrict<R, DIM, true, true>, 1);
     wave((const void *)k_residual_restrict<R, DIM, false, true>, 1);
-    wave((const void *)k_prolong_add<R, DIM, true>, 1);
+    wave((const void *)k_prolong_add<R, DIM, true, true>, 1);
+    wave((const void *)k_prolong_add<R, DIM, false, true>, 1);
 }
 
 template <int DIM>
@@ -917,7 +943,8 @@ void enqueue_cycle64(const mg_handle *h, cudaStream_t s) {
 // Mixed: FP32 V-cycles on the correction, FP64 update, FP64 residual + norm.
 template <int DIM>
 void enqueue_step32(const mg_handle *h, cudaStream_t s) {
-    for (int q = 0; q < h->opt.inner_cycles; q++) enqueue_vcycle<float, DIM>(h, s, 0, h->opt.cycle);
+    for (int q = 0; q < h->opt.inner_cycles; q++)
+        enqueue_vcycle<float, DIM>(h, s, 0, h->opt.cycle, q == 0 && red_start(h));
     const LevelBuf &f = h->L[0];
     launch_k(h, k_add_correction, lin_blocks(f.N), 256, 0, s, 0, mixed_delta(h), f.x32, f.N);
     counted(h);
@@ -1023,7 +1050,7 @@ mg_status accumulate_timing(mg_handle *h) {
     CK(cudaEventElapsedTime(&a, h->ev[0], h->ev[1]));
     h->smooth_ms += (double)a;
     long long l1, s1;
-    const int sw = h->opt.nu1 > 0 ? h->opt.nu1 : h->opt.nu2;
+    const int sw = h->opt.nu1 > 0 ? h->opt.nu1 - (timed_after_first(h) ? 1 : 0) : h->opt.nu2;
     if (h->opt.smoother == MG_SMOOTH_WJAC) {
         l1 = sw;                 // one Jacobi kernel per sweep
         s1 = sw;
@@ -1412,7 +1439,8 @@ mg_status enqueue_correction(mg_handle *h, cudaStream_t s, const double2 *rhs) {
     enqueue_prep<DIM>(h, rhs, s);
     if (h->opt.precision == MG_MIXED) {
         enqueue_residual_to32<DIM>(h, s, true);        // x = 0: b32 = b, bt32 = Dinv b, e32 = 0
-        for (int q = 0; q < h->opt.max_cycles; q++) enqueue_vcycle<float, DIM>(h, s, 0, h->opt.cycle);
+        for (int q = 0; q < h->opt.max_cycles; q++)
+        enqueue_vcycle<float, DIM>(h, s, 0, h->opt.cycle, q == 0 && red_start(h));
         launch_k(h, k_add_correction, lin_blocks(f.N), 256, 0, s, 0, f.x, f.x32, f.N);
         counted(h);
     } else {
@@ -1472,7 +1500,8 @@ mg_status capture_async(mg_handle *h) {
         const long long b0 = h->enq;
         h->cond_body = true;
         if (mixed) {
-            for (int q = 0; q < h->opt.inner_cycles; q++) enqueue_vcycle<float, DIM>(h, h->cap2, 0, h->opt.cycle);
+            for (int q = 0; q < h->opt.inner_cycles; q++)
+                enqueue_vcycle<float, DIM>(h, h->cap2, 0, h->opt.cycle, q == 0 && red_start(h));
             const LevelBuf &f = h->L[0];
             launch_k(h, k_add_correction, lin_blocks(f.N), 256, 0, h->cap2, 0, mixed_delta(h), f.x32, f.N);
             counted(h);

@@ -161,7 +161,8 @@ __device__ __forceinline__ void tail_colour(const TailCta<R> &C, const TailLevel
 // Restriction of the residual from F to its coarse level Cl over the coarse
 // cells this CTA owns (residual_restrict_block's arithmetic).
 template <typename R, int DIM, bool CL, bool RED>
-__device__ __forceinline__ void tail_restrict(const TailCta<R> &C, const TailLevel<R> &F, const TailLevel<R> &Cl) {
+__device__ __forceinline__ void tail_restrict(const TailCta<R> &C, const TailLevel<R> &F, const TailLevel<R> &Cl,
+                                              int red_start) {
     using V2 = typename Vec<R>::v2;
     const Level<R> &FL = F.g, &CG = Cl.g;
     int s0, s1;
@@ -192,24 +193,27 @@ __device__ __forceinline__ void tail_restrict(const TailCta<R> &C, const TailLev
         const R bT = aT * wgt, bp = ap * wgt;
         *tail_at<R, DIM, CL>(C, Cl, 1, I, J, K) = mk2<R>(bT, bp);
         const auto Di = ldgq(CG.Dinv + cc);
-        *tail_at<R, DIM, CL>(C, Cl, 2, I, J, K) = mk2<R>(Di.a * bT + Di.b * bp, Di.c * bT + Di.d * bp);
-        *tail_at<R, DIM, CL>(C, Cl, 0, I, J, K) = mk2<R>(R(0), R(0));
+        const V2 z = mk2<R>(Di.a * bT + Di.b * bp, Di.c * bT + Di.d * bp);
+        *tail_at<R, DIM, CL>(C, Cl, 2, I, J, K) = z;
+        *tail_at<R, DIM, CL>(C, Cl, 0, I, J, K) = red_start && !((I + J + K) & 1) ? z : mk2<R>(R(0), R(0));
     }
 }
 
-// Prolongation of Cl's x into F's owned cells (prolong_add_block's arithmetic).
+// Prolongation of Cl's x into F's owned cells (prolong_add_block's arithmetic; black: the black cells only).
 template <typename R, int DIM, bool CL>
 __device__ __forceinline__ void tail_prolong(const TailCta<R> &C, const TailLevel<R> &Cl, const TailLevel<R> &F,
-                                             const BcFlags &bc) {
+                                             const BcFlags &bc, bool black) {
     using V2 = typename Vec<R>::v2;
     const Level<R> &FL = F.g, &CG = Cl.g;
     int s0, s1;
     tail_owned(C, F, s0, s1);
-    for (int q = threadIdx.x + kBX * threadIdx.y; q < (s1 - s0) * F.slab; q += kTailThreads) {
-        const int sl = q / F.slab, w = q - sl * F.slab;
-        const int i = w % FL.n0;
-        const int j = DIM == 3 ? w / FL.n0 : s0 + sl;
+    const int row = black ? (FL.n0 + 1) / 2 : FL.n0, per = (DIM == 3 ? FL.n1 : 1) * row;
+    for (int q = threadIdx.x + kBX * threadIdx.y; q < (s1 - s0) * per; q += kTailThreads) {
+        const int sl = q / per, w = q - sl * per;
+        const int j = DIM == 3 ? w / row : s0 + sl;
         const int k = DIM == 3 ? s0 + sl : 0;
+        const int i = black ? 2 * (w % row) + ((j + k + 1) & 1) : w % row;
+        if (i >= FL.n0) continue;
         const int P[3] = {i >> 1, j >> 1, k >> 1};
         const int s[3] = {(i & 1) ? 1 : -1, (j & 1) ? 1 : -1, (k & 1) ? 1 : -1};
         const int nC[3] = {CG.n0, CG.n1, CG.n2};
@@ -261,20 +265,21 @@ __global__ void __launch_bounds__(kTailThreads) k_vcycle_tail(const __grid_const
         tail_owned(C, T, s0, s1);
         const long long g0 = (long long)s0 * T.slab;
         for (int q = tid; q < (s1 - s0) * T.slab; q += kTailThreads) {
-            C.sm[T.off + q] = mk2<R>(R(0), R(0));
+            const V2 z = __ldcg(T.g.bt + g0 + q);
+            const int j = q / T.g.n0, par = (q - j * T.g.n0) + (DIM == 3 ? j % T.g.n1 + s0 + j / T.g.n1 : s0 + j);
+            C.sm[T.off + q] = A.nu1 > 0 && !(par & 1) ? z : mk2<R>(R(0), R(0));   // the first red half-sweep from zero
             C.sm[T.off + T.cap + q] = __ldcg(T.g.b + g0 + q);
-            C.sm[T.off + 2 * T.cap + q] = __ldcg(T.g.bt + g0 + q);
+            C.sm[T.off + 2 * T.cap + q] = z;
         }
     }
     tail_sync<CL>();                    // every CTA resident and loaded before any remote read
     for (int l = 0; l + 1 < A.nlev; l++) {
-        for (int q = 0; q < A.nu1; q++)
-            for (int colour = 0; colour < 2; colour++) {
-                tail_colour<R, DIM, CL>(C, A.L[l], colour);
-                tail_sync<CL>();
-            }
-        if (A.nu1 > 0) tail_restrict<R, DIM, CL, true>(C, A.L[l], A.L[l + 1]);
-        else tail_restrict<R, DIM, CL, false>(C, A.L[l], A.L[l + 1]);
+        for (int q = 1; q < 2 * A.nu1; q++) {          // the first red half-sweep is in the guess
+            tail_colour<R, DIM, CL>(C, A.L[l], q & 1);
+            tail_sync<CL>();
+        }
+        if (A.nu1 > 0) tail_restrict<R, DIM, CL, true>(C, A.L[l], A.L[l + 1], 1);
+        else tail_restrict<R, DIM, CL, false>(C, A.L[l], A.L[l + 1], 0);
         tail_sync<CL>();
     }
     {   // coarsest: x = Minv b for the unknowns of the owned cells, one warp per row
@@ -305,7 +310,7 @@ __global__ void __launch_bounds__(kTailThreads) k_vcycle_tail(const __grid_const
         tail_sync<CL>();
     }
     for (int l = A.nlev - 2; l >= 0; l--) {
-        tail_prolong<R, DIM, CL>(C, A.L[l + 1], A.L[l], A.bc);
+        tail_prolong<R, DIM, CL>(C, A.L[l + 1], A.L[l], A.bc, A.nu2 > 0);
         tail_sync<CL>();
         for (int q = 0; q < A.nu2; q++)
             for (int colour = 0; colour < 2; colour++) {
