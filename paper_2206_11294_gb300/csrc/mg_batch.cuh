@@ -33,7 +33,8 @@ struct BProb {                  // one problem, device side
     unsigned int *ticket;
     const double *Minv;
     const float *Minv32;
-    const double *Lb, *Uc;      // the coarsest level's factors, when its solve uses them (k_coarse_lu)
+    const double *Lb, *Uc;      // the coarsest level's factors, when its solve uses them (coarse_solve_cluster)
+    CoarseProb cp;              // the coarsest matrix on the cluster paths (mg_coarse.cuh)
     const int *piv;
     const double *dinv;
     const int *err;
@@ -172,21 +173,55 @@ __global__ void __launch_bounds__(kBatchThreads) kb_coarse(const BLevel *__restr
     }
 }
 
-// Coarsest solves of the problems that keep the factors (ids): one block each.
+// Coarsest solves of the problems that keep the factors (ids): one cluster each (blockIdx.y).
 template <typename R>
-__global__ void __launch_bounds__(kLuSolveThreads) kb_coarse_lu(const BLevel *__restrict__ lv,
-                                                                const BProb *__restrict__ pr,
-                                                                const BState *__restrict__ st,
-                                                                const int *__restrict__ ids) {
+__global__ void __launch_bounds__(kBcrThreads) kb_coarse_solve(const BLevel *__restrict__ lv,
+                                                              const BProb *__restrict__ pr,
+                                                              const BState *__restrict__ st,
+                                                              const int *__restrict__ ids) {
     extern __shared__ double blusm[];
-    const int p = ids[blockIdx.x];
+    const int p = ids[blockIdx.y];
     if (!st[p].active) return;
     const BProb &P = pr[p];
     const Level<R> C = pick<R>(lv[P.coarse]);
-    coarse_lu_solve_block<R>(P.Lb, P.Uc, P.piv, P.dinv, P.nc, P.kl, P.kl, reinterpret_cast<const R *>(C.b),
-                             reinterpret_cast<R *>(C.x), P.err, blusm);
+    coarse_solve_cluster<R>(P.cp, P.Lb, P.Uc, P.piv, P.dinv, P.kl, reinterpret_cast<const R *>(C.b),
+                            reinterpret_cast<R *>(C.x), blusm);
 }
 
+// The cluster paths of mg_coarse.cuh over the problems ids[blockIdx.y] (inverses: nc <= kBandSmemMax; the other
+// kernels: block cyclic reduction, stage s).  Problems with fewer blocks or stages than the largest return early.
+__global__ void __launch_bounds__(kGjThreads) kb_coarse_invert(const BProb *__restrict__ pr, const int *__restrict__ ids) {
+    extern __shared__ double bgsm[];
+    coarse_invert(pr[ids[blockIdx.y]].cp, bgsm);
+}
+
+__global__ void __launch_bounds__(kGjThreads) kb_bcr_invert(const BProb *__restrict__ pr, const int *__restrict__ ids, int s) {
+    extern __shared__ double bgsm[];
+    bcr_invert(pr[ids[blockIdx.y]].cp, s, blockIdx.x / kGjCtas, bgsm);
+}
+
+__global__ void __launch_bounds__(256) kb_bcr_couplings(const BProb *__restrict__ pr, const int *__restrict__ ids) {
+    bcr_couplings(pr[ids[blockIdx.y]].cp, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+}
+
+__global__ void __launch_bounds__(256) kb_bcr_update0(const BProb *__restrict__ pr, const int *__restrict__ ids) {
+    bcr_update0(pr[ids[blockIdx.z]].cp, blockIdx.y, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+}
+
+__global__ void __launch_bounds__(256) kb_bcr_products1(const BProb *__restrict__ pr, const int *__restrict__ ids, int s) {
+    extern __shared__ double bgsm[];
+    if (s + 1 < pr[ids[blockIdx.z]].cp.stages) bcr_products1(pr[ids[blockIdx.z]].cp, s, blockIdx.y, blockIdx.x, bgsm);
+}
+
+__global__ void __launch_bounds__(256) kb_bcr_products2(const BProb *__restrict__ pr, const int *__restrict__ ids, int s) {
+    extern __shared__ double bgsm[];
+    if (s + 1 < pr[ids[blockIdx.z]].cp.stages) bcr_products2(pr[ids[blockIdx.z]].cp, s, blockIdx.y, blockIdx.x, bgsm);
+}
+
+__global__ void __launch_bounds__(kBcrThreads) kb_bcr_check(const BProb *__restrict__ pr, const int *__restrict__ ids) {
+    extern __shared__ double bgsm[];
+    bcr_check(pr[ids[blockIdx.y]].cp, bgsm);
+}
 
 template <int DIM>
 __global__ void __launch_bounds__(kBatchThreads) kb_setup_fine(const BSetupLevel *__restrict__ sl,
@@ -305,8 +340,9 @@ __global__ void __launch_bounds__(kBatchThreads) kb_coarse_assemble(const BCoars
 // factors (the factors in the problem's work array: Lb, then Uc); a 2D grid
 // of warp groups (x: column groups, y: problem) computes the inverse.
 __global__ void __launch_bounds__(kWinThreads) kb_band_lu_window(const BCoarse *__restrict__ co,
-                                                                  const int *__restrict__ ids) {
+                                                                  const int *__restrict__ ids, int fallback) {
     const BCoarse &C = co[ids[blockIdx.x]];
+    if (fallback && coarse_done(C.err + 3)) return;
     band_lu_window_block(C.M, C.nc, C.kl, C.kl, C.piv, C.dinv, C.Mwork, C.Mwork + (long long)C.nc * C.kl, C.err);
 }
 
@@ -314,15 +350,17 @@ __global__ void __launch_bounds__(kWinThreads) kb_band_lu_window(const BCoarse *
 // problem's entries, y: problem).
 __global__ void __launch_bounds__(256) kb_scale_uc(const BCoarse *__restrict__ co, const int *__restrict__ ids) {
     const BCoarse &C = co[ids[blockIdx.y]];
+    if (coarse_done(C.err + 3)) return;
     scale_uc(C.Mwork + (long long)C.nc * C.kl, C.dinv, C.nc, C.kl, C.kl, C.err,
              blockIdx.x * (long long)blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
 }
 
 // The blocked LU on one cluster per problem (band_lu_blocked_block): cluster c factors problem ids[c].
 __global__ void __launch_bounds__(kLuBlockedThreads) kb_band_lu_blocked(const BCoarse *__restrict__ co,
-                                                                        const int *__restrict__ ids) {
+                                                                        const int *__restrict__ ids, int fallback) {
     extern __shared__ double bbsm[];
     const BCoarse &C = co[ids[blockIdx.x / kLuClusterCtas]];
+    if (fallback && coarse_done(C.err + 3)) return;
     band_lu_blocked_block(C.M, C.nc, C.kl, C.kl, C.piv, C.dinv, C.Mwork, C.Mwork + (long long)C.nc * C.kl, C.err,
                           bbsm);
 }
@@ -340,13 +378,14 @@ __global__ void __launch_bounds__(256) kb_band_inv_block(const BCoarse *__restri
 __global__ void __launch_bounds__(kLUThreads) kb_band_lu_warp(const BCoarse *__restrict__ co,
                                                                const int *__restrict__ ids) {
     const BCoarse &C = co[ids[blockIdx.x]];
+    if (coarse_done(C.err + 3)) return;
     band_lu_warp_block(C.M, C.nc, C.kl, C.kl, C.piv, C.dinv, C.err);
 }
 
 __global__ void __launch_bounds__(32 * kInvRows) kb_band_inv_cols_warp(const BCoarse *__restrict__ co,
                                                                       const int *__restrict__ ids) {
     const BCoarse &C = co[ids[blockIdx.y]];
-    if ((int)blockIdx.x * 32 >= C.nc) return;
+    if ((int)blockIdx.x * 32 >= C.nc || coarse_done(C.err + 3)) return;
     band_inv_cols_warp_block(C.M, C.piv, C.dinv, C.nc, C.kl, C.kl, C.Minv, C.Minv32, blockIdx.x, C.err);
 }
 
@@ -562,7 +601,9 @@ struct mg_batch {
     int *win_ids;                     // problems on the windowed banded path (device)
     std::vector<int> win_coarse;      // their indices
     bool win_factors = false;         // the windowed-path problems solve from their factors (no inverse)
-    size_t lu_smem = 0;               // shared memory of kb_coarse_lu
+    size_t lu_smem = 0;               // shared memory of kb_coarse_solve
+    int bcr_q = 0, bcr_m = 0, bcr_stages = 0;   // largest block, block count and stages of the reductions (0: none)
+    size_t bcr_smem = 0;              // shared memory of kb_bcr_check
     int max_nc_win = 0;
     size_t win_smem = 0, win_inv_smem = 0;
     int win_warps = 8;
@@ -633,9 +674,8 @@ void b_vcycle(mg_batch *b, cudaStream_t s, bool red_done = false) {
         b->launches++;
     }
     if (b->win_factors) {
-        raise_smem_limit((const void *)kb_coarse_lu<R>, (int)b->lu_smem);
-        kb_coarse_lu<R><<<(unsigned)b->win_coarse.size(), kLuSolveThreads, b->lu_smem, s>>>(b->lv, b->pr, b->st,
-                                                                                            b->win_ids);
+        launch_clusters(kb_coarse_solve<R>, s, 1, (int)b->win_coarse.size(), kBcrThreads, b->lu_smem,
+                        (const BLevel *)b->lv, (const BProb *)b->pr, (const BState *)b->st, (const int *)b->win_ids);
         b->launches++;
     }
     for (int d = b->dmax - 2; d >= 0; d--) {
@@ -850,6 +890,7 @@ mg_status mg_batch_create(int count, mg_handle *const *handles, mg_batch **out) 
         pr[p].piv = h->piv;
         pr[p].dinv = h->dinv;
         pr[p].err = h->err_d;
+        pr[p].cp = h->cprob;
         pr[p].kl = h->coarse_kl;
         pr[p].nc = h->nc;
         pr[p].coarse = base[p] + h->nlev - 1;
@@ -965,7 +1006,13 @@ mg_status mg_batch_create(int count, mg_handle *const *handles, mg_batch **out) 
         } else if (window_path(h->nc, C.kl)) {
             b->win_coarse.push_back(p);
             b->win_factors = h->coarse_factors;      // one coarse_solve option for the whole batch
-            b->lu_smem = std::max(b->lu_smem, (size_t)coarse_lu_smem(h->nc, C.kl, C.kl));
+            b->lu_smem = std::max(b->lu_smem, coarse_solve_smem(h->nc, C.kl));
+            if (h->cprob.q > 0) {
+                b->bcr_q = std::max(b->bcr_q, h->cprob.q);
+                b->bcr_m = std::max(b->bcr_m, h->cprob.m);
+                b->bcr_stages = std::max(b->bcr_stages, h->cprob.stages);
+            }
+            b->bcr_smem = std::max(b->bcr_smem, bcr_solve_smem(h->nc));
             b->max_nc_win = std::max(b->max_nc_win, h->nc);
             b->win_smem = std::max(b->win_smem, (size_t)band_window_smem(C.kl, C.kl));
             b->win_warps = std::min(b->win_warps, inv_block_warps(h->nc, C.kl));
@@ -1218,6 +1265,9 @@ mg_status mg_batch_set_coeffs(mg_batch *b, const double *const *lambda, const do
     else kb_coarse_assemble<3><<<dim3(4, gy), kBatchThreads, 0, s>>>(b->co, b->count);
     b->launches += 2;
     if (b->n_inv_smem > 0) {
+        CK(launch_clusters(kb_coarse_invert, s, 1, b->n_inv_smem, kGjThreads, gj_smem(b->max_nc_small),
+                           (const BProb *)b->pr, (const int *)b->inv_ids));
+        b->launches++;
         CK(raise_smem_limit((const void *)kb_band_lu_warp, (int)(sizeof(double) * kBandSmemMax * kBandSmemMax)));
         kb_band_lu_warp<<<b->n_inv_smem, kLUThreads, b->inv_smem_bytes, s>>>(b->co, b->inv_ids);
         CK(raise_smem_limit((const void *)kb_band_inv_cols_warp, (int)b->inv_cols_smem_bytes));
@@ -1229,6 +1279,34 @@ mg_status mg_batch_set_coeffs(mg_batch *b, const double *const *lambda, const do
         const unsigned nw = (unsigned)b->win_coarse.size();
         CK(raise_smem_limit((const void *)kb_band_lu_window, (int)b->win_smem));
         CK(raise_smem_limit((const void *)kb_band_inv_block, (int)b->win_inv_smem));
+        const int fallback = b->win_factors ? 1 : 0;
+        if (b->win_factors) {               // block cyclic reduction of all of them, stage by stage
+            const BProb *pr = b->pr;
+            const int *ids = b->win_ids;
+            const int nt = (b->bcr_q + kBcrTile - 1) / kBcrTile;
+            const size_t gsm = bcr_gemm_smem(b->bcr_q);
+            CK(raise_smem_limit((const void *)kb_bcr_products1, (int)gsm));
+            CK(raise_smem_limit((const void *)kb_bcr_products2, (int)gsm));
+            kb_bcr_couplings<<<dim3(4, nw), 256, 0, s>>>(pr, ids);
+            b->launches++;
+            for (int st = 0; st < b->bcr_stages; st++) {
+                const int E = bcr_eliminated(b->bcr_m, st), left = b->bcr_m >> (st + 1);
+                CK(launch_clusters(kb_bcr_invert, s, E, (int)nw, kGjThreads, gj_smem(b->bcr_q), pr, ids, st));
+                b->launches++;
+                if (st + 1 == b->bcr_stages) break;
+                if (st == 0) {
+                    kb_bcr_update0<<<dim3((unsigned)((b->bcr_q * b->bcr_q / 4 + 255) / 256), (unsigned)(2 * E + left), nw),
+                                     256, 0, s>>>(pr, ids);
+                    b->launches++;
+                } else {
+                    kb_bcr_products1<<<dim3((unsigned)(nt * nt), (unsigned)(4 * E), nw), 256, gsm, s>>>(pr, ids, st);
+                    kb_bcr_products2<<<dim3((unsigned)(nt * nt), (unsigned)(2 * E + left), nw), 256, gsm, s>>>(pr, ids, st);
+                    b->launches += 2;
+                }
+            }
+            CK(launch_clusters(kb_bcr_check, s, 1, (int)nw, kBcrThreads, b->bcr_smem, pr, ids));
+            b->launches++;
+        }
         {   // blocked over one cluster per problem where every problem's shared memory fits and all the clusters
             // run at once (one SM per CTA), else one block each: a second wave of clusters would cost more than
             // the blocked LU saves over all problems factoring side by side
@@ -1240,13 +1318,13 @@ mg_status mg_batch_set_coeffs(mg_batch *b, const double *const *lambda, const do
                 bsm = std::max(bsm, (size_t)band_blocked_smem(hp->nc, hp->coarse_kl, hp->coarse_kl));
             }
             if (blocked)
-                CK(launch_cluster(kb_band_lu_blocked, s, (int)nw, kLuBlockedThreads, bsm, (const BCoarse *)b->co,
-                                  (const int *)b->win_ids));
+                CK(launch_clusters(kb_band_lu_blocked, s, (int)nw, 1, kLuBlockedThreads, bsm, (const BCoarse *)b->co,
+                                   (const int *)b->win_ids, fallback));
             else
-                kb_band_lu_window<<<nw, kWinThreads, b->win_smem, s>>>(b->co, b->win_ids);
+                kb_band_lu_window<<<nw, kWinThreads, b->win_smem, s>>>(b->co, b->win_ids, fallback);
         }
         b->launches++;
-        if (b->win_factors)                 // the cycles solve from Lb and the scaled Uc (kb_coarse_lu)
+        if (b->win_factors)                 // the cycles solve from Lb and the scaled Uc (kb_coarse_solve)
             kb_scale_uc<<<dim3(64, nw), 256, 0, s>>>(b->co, b->win_ids);
         else
             kb_band_inv_block<<<dim3((unsigned)((b->max_nc_win + b->win_warps - 1) / b->win_warps), nw),

@@ -22,6 +22,7 @@
 #include "coupledmg.h"
 #include "mg_host.h"
 #include "mg_kernels.cuh"
+#include "mg_coarse.cuh"
 #include "mg_tail.cuh"
 #include "mg_async.cuh"
 #include "mg_assemble.cuh"
@@ -139,7 +140,10 @@ struct mg_handle {
     TmaLevel *tmaps;       // tensor maps per (level, precision, tile), built on first use (host memory)
     unsigned char *tmap_ok;
     double *Minv, *Mtmp;   // coarse inverse (NULL when the cycles solve from the factors); assembled matrix
-    bool coarse_factors;   // the cycles solve the coarsest level from its LU factors (k_coarse_lu)
+    bool coarse_factors;   // the cycles solve the coarsest level from its factors (k_coarse_solve)
+    CoarseProb cprob;      // the coarsest matrix on the cluster paths (mg_coarse.cuh); q > 0: block cyclic reduction
+    cudaGraphExec_t gcoarse;   // its factorisation or inverse, replayed on the aux stream after each set-up
+    long long coarse_kernels;
     int coarse_kl;         // the coarsest matrix's lower (= upper) bandwidth
     double *Mwork;         // coarse inverse: columns before the transpose (banded path); the window path's factors
     int *piv;              // coarse inverse: pivot rows (banded path)
@@ -331,7 +335,18 @@ void plan(mg_handle *h, char *base, size_t *bytes) {
     h->Minv = h->coarse_factors ? nullptr : P.take<double>((long long)h->nc * h->nc);
     h->Mtmp = P.take<double>((long long)h->nc * h->nc);
     const bool big = h->nc > kBandSmemMax;
-    h->Mwork = big ? P.take<double>((long long)h->nc * h->nc) : nullptr;
+    CoarseProb &cp = h->cprob;
+    std::memset(&cp, 0, sizeof(cp));
+    cp.nc = h->nc;
+    for (int a = 0; a < 3; a++) cp.n[a] = c.n[a];
+    if (h->coarse_factors) {
+        bcr_shape(cp);
+        if (cp.q > kGjMax || cp.stages > kBcrMaxStages) cp.q = cp.m = 0;
+    }
+    cp.M = h->Mtmp;
+    // the reduction's arrays and the banded LU's (its fallback, run once they are discarded) share one area
+    h->Mwork = big ? P.take<double>(std::max((long long)h->nc * h->nc, bcr_work_doubles(cp.q, cp.m))) : nullptr;
+    cp.work = h->Mwork;
     h->piv = P.take<int>(h->nc);
     h->dinv = P.take<double>(h->nc);
     h->Minv32 = mixed && !h->coarse_factors ? P.take<float>((long long)h->nc * h->nc) : nullptr;
@@ -340,8 +355,12 @@ void plan(mg_handle *h, char *base, size_t *bytes) {
     h->partial = P.take<double2>(h->npartial);
     h->norms_d = P.take<double>(8);
     h->ticket = P.take<unsigned int>(1);
-    h->err_d = P.take<int>(4);            // [0] set-up flags, [1] bounded waits that gave up (per solve), [2] jump cells
+    h->err_d = P.take<int>(4);            // [0] set-up flags, [1] bounded waits that gave up (per solve), [2] jump cells,
+                                          // [3] the coarsest factors of mg_coarse.cuh are good
     if (h->L[0].jflag) h->L[0].jcount = h->err_d + 2;
+    cp.Minv = h->Minv;
+    cp.Minv32 = h->Minv32;
+    cp.err = h->err_d;
     h->astat_d = P.take<AsyncStat>(1);
     *bytes = P.off + kAlign;
 }
@@ -464,6 +483,11 @@ void launch_k(const mg_handle *h, void (*kern)(KArgs...), dim3 grid, dim3 block,
     cfg.attrs = attr;
     cfg.numAttrs = (unsigned)na;
     cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+}
+
+// Shared memory of k_coarse_solve (bytes): the reduction's solve or the LU's.
+size_t coarse_solve_smem(int nc, int kl) {
+    return std::max(bcr_solve_smem(nc), (size_t)coarse_lu_smem(nc, kl, kl));
 }
 
 template <typename R> typename Vec<R>::v2 *xalt_of(const LevelBuf &l);
@@ -794,12 +818,11 @@ void enqueue_vcycle(const mg_handle *h, cudaStream_t s, int l, int type, bool re
         // the coarsest inverse (or factors) is computed on the aux stream after each set-up
         if (!h->cond_body) cudaStreamWaitEvent(s, h->ev_inv, cudaEventWaitExternal);
         if (h->coarse_factors) {
-            const long long sm = coarse_lu_smem(h->nc, h->coarse_kl, h->coarse_kl);
-            raise_smem_limit((const void *)k_coarse_lu<R>, (int)sm);
-            launch_k(h, k_coarse_lu<R>, 1, kLuSolveThreads, (size_t)sm, s, 0, h->Mwork, h->Mwork + (long long)h->nc * h->coarse_kl, h->piv,
-                                                     h->dinv, h->nc, h->coarse_kl, h->coarse_kl,
-                                                     reinterpret_cast<const R *>(v.b), reinterpret_cast<R *>(v.x),
-                                                     h->err_d);
+            const size_t sm = coarse_solve_smem(h->nc, h->coarse_kl);
+            raise_smem_limit((const void *)k_coarse_solve<R>, (int)sm);
+            launch_k(h, k_coarse_solve<R>, kGjCtas, kBcrThreads, sm, s, kGjCtas, h->cprob, h->Mwork,
+                     h->Mwork + (long long)h->nc * h->coarse_kl, h->piv, h->dinv, h->coarse_kl,
+                     reinterpret_cast<const R *>(v.b), reinterpret_cast<R *>(v.x));
             counted(h);
             return;
         }
@@ -1092,15 +1115,16 @@ bool window_path(int n, int kl) {
 // memory fits.
 bool lu_blocked_ok(int n, int kl) { return band_blocked_smem(n, kl, kl) <= kWinSmemMax; }
 
-// Launches kern on `clusters` clusters of kLuClusterCtas CTAs of `threads` threads.
+// Launches kern on `clusters` x `rows` clusters (grid x, y) of kLuClusterCtas CTAs of `threads` threads.
+static_assert(kLuClusterCtas == kGjCtas, "one cluster shape");
 template <typename... Args>
-cudaError_t launch_cluster(void (*kern)(Args...), cudaStream_t s, int clusters, int threads, size_t smem,
-                           Args... args) {
+cudaError_t launch_clusters(void (*kern)(Args...), cudaStream_t s, int clusters, int rows, int threads, size_t smem,
+                            Args... args) {
     cudaError_t e = raise_smem_limit((const void *)kern, (int)smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg;
     std::memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3((unsigned)(kLuClusterCtas * clusters), 1, 1);
+    cfg.gridDim = dim3((unsigned)(kLuClusterCtas * clusters), (unsigned)rows, 1);
     cfg.blockDim = dim3((unsigned)threads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
@@ -1115,9 +1139,91 @@ cudaError_t launch_cluster(void (*kern)(Args...), cudaStream_t s, int clusters, 
 }
 
 cudaError_t launch_lu_blocked(cudaStream_t s, const double *M, int n, int kl, int *piv, double *dinv, double *Lb,
-                              double *Uc, int *err) {
-    return launch_cluster(k_band_lu_blocked, s, 1, kLuBlockedThreads, (size_t)band_blocked_smem(n, kl, kl), M, n, kl,
-                          kl, piv, dinv, Lb, Uc, err);
+                              double *Uc, int *err, const int *done) {
+    return launch_clusters(k_band_lu_blocked, s, 1, 1, kLuBlockedThreads, (size_t)band_blocked_smem(n, kl, kl), M, n,
+                           kl, kl, piv, dinv, Lb, Uc, err, done);
+}
+
+// Blocks eliminated at stage s, and left after it (host side of bcr_count, bcr_left).
+int bcr_eliminated(int m, int s) {
+    const int f = (1 << s) - 1;
+    return m > f ? (m - f + (2 << s) - 1) >> (s + 1) : 0;
+}
+
+// The factorisation or inverse of the coarsest matrix on stream a: the cluster
+// paths of mg_coarse.cuh with the banded LU behind them as the fallback, or
+// the banded LU alone.
+mg_status enqueue_coarse(mg_handle *h, cudaStream_t a) {
+    const int n = h->nc, kl = h->coarse_kl;
+    float *inv32 = h->opt.precision == MG_MIXED ? h->Minv32 : nullptr;
+    const CoarseProb &P = h->cprob;
+    if (n <= kBandSmemMax) {
+        CK(launch_clusters(k_coarse_invert, a, 1, 1, kGjThreads, gj_smem(n), P));
+        const int *done = h->err_d + 3;
+        const size_t smem_lu = sizeof(double) * (size_t)n * n;
+        CK(raise_smem_limit((const void *)k_band_lu_warp, (int)(sizeof(double) * kBandSmemMax * kBandSmemMax)));
+        k_band_lu_warp<<<1, kLUThreads, smem_lu, a>>>(h->Mtmp, n, kl, kl, h->piv, h->dinv, h->err_d, done);
+        const int smem_inv = (int)(sizeof(double) * inv_smem_doubles(n, kl, kl));
+        CK(raise_smem_limit((const void *)k_band_inv_cols_warp,
+                            (int)(sizeof(double) * inv_smem_doubles(kBandSmemMax, kBandSmemMax - 1, kBandSmemMax - 1))));
+        k_band_inv_cols_warp<<<(n + 31) / 32, dim3(32, kInvRows), smem_inv, a>>>(h->Mtmp, h->piv, h->dinv, n, kl, kl,
+                                                                                h->Minv, inv32, h->err_d, done);
+        counted(h, 3);
+    } else if (window_path(n, kl)) {
+        const int *done = nullptr;
+        if (P.q > 0) {
+            const int nt = (P.q + kBcrTile - 1) / kBcrTile;
+            const size_t gsm = bcr_gemm_smem(P.q);
+            raise_smem_limit((const void *)k_bcr_products1, (int)gsm);
+            raise_smem_limit((const void *)k_bcr_products2, (int)gsm);
+            k_bcr_couplings<<<(unsigned)((P.q * P.m + 255) / 256), 256, 0, a>>>(P);
+            counted(h);
+            for (int st = 0; st < P.stages; st++) {
+                const int E = bcr_eliminated(P.m, st), left = P.m >> (st + 1);
+                CK(launch_clusters(k_bcr_invert, a, E, 1, kGjThreads, gj_smem(P.q), P, st));
+                counted(h);
+                if (st + 1 == P.stages) break;
+                if (st == 0) {
+                    const unsigned gx = (unsigned)((P.q * P.q / 4 + 255) / 256);
+                    k_bcr_update0<<<dim3(gx, (unsigned)(2 * E + left)), 256, 0, a>>>(P);
+                    counted(h);
+                } else {
+                    k_bcr_products1<<<dim3((unsigned)(nt * nt), (unsigned)(4 * E)), 256, gsm, a>>>(P, st);
+                    k_bcr_products2<<<dim3((unsigned)(nt * nt), (unsigned)(2 * E + left)), 256, gsm, a>>>(P, st);
+                    counted(h, 2);
+                }
+            }
+            CK(launch_clusters(k_bcr_check, a, 1, 1, kBcrThreads, bcr_solve_smem(n), P));
+            counted(h);
+            done = h->err_d + 3;
+        }
+        // the band's active window in shared memory, then (INVERSE) the columns of the inverse, a warp each
+        const long long wsm = band_window_smem(kl, kl);
+        const int warps = inv_block_warps(n, kl);
+        const long long ism = band_inv_block_smem(n, kl, kl, warps);
+        CK(raise_smem_limit((const void *)k_band_lu_window, (int)wsm));
+        CK(raise_smem_limit((const void *)k_band_inv_block, (int)ism));
+        double *Lb = h->Mwork, *Uc = h->Mwork + (long long)n * kl;
+        if (lu_blocked_ok(n, kl))
+            CK(launch_lu_blocked(a, h->Mtmp, n, kl, h->piv, h->dinv, Lb, Uc, h->err_d, done));
+        else
+            k_band_lu_window<<<1, kWinThreads, (size_t)wsm, a>>>(h->Mtmp, n, kl, kl, h->piv, h->dinv, Lb, Uc, h->err_d,
+                                                                 done);
+        if (h->coarse_factors)           // the cycles solve from Lb and the scaled Uc (k_coarse_solve)
+            k_scale_uc<<<lin_blocks((long long)n * 2 * kl), 256, 0, a>>>(Uc, h->dinv, n, kl, kl, h->err_d, done);
+        else
+            k_band_inv_block<<<(n + warps - 1) / warps, 32 * warps, (size_t)ism, a>>>(
+                Lb, Uc, h->piv, h->dinv, n, kl, kl, h->Minv, inv32, h->err_d);
+        counted(h, 2);
+    } else {
+        k_band_lu<<<1, dim3(32, 32, 1), 0, a>>>(h->Mtmp, n, kl, kl, h->piv, h->dinv, h->err_d);
+        k_band_inv_cols<<<(n + 127) / 128, 128, 0, a>>>(h->Mtmp, h->piv, h->dinv, n, kl, kl, h->Mwork, h->err_d);
+        k_transpose<<<lin_blocks((long long)n * n), 256, 0, a>>>(h->Mwork, h->Minv, n);
+        if (inv32) k_to_f32<<<lin_blocks((long long)n * n), 256, 0, a>>>(h->Minv, inv32, (long long)n * n);
+        counted(h, 4);
+    }
+    CK(cudaGetLastError());
+    return MG_OK;
 }
 
 // ---------------------------------------------------------------- set-up
@@ -1193,7 +1299,6 @@ mg_status setup_hierarchy(mg_handle *h, const double *lam, const double *const f
                           int on_device) {
     const mg_grid &g = h->grid;
     cudaStream_t s = h->stream;
-    const bool mixed = h->opt.precision == MG_MIXED;
     LevelBuf &f = h->L[0];
     // the previous set-up's coarsest inverse must be done before anything is overwritten
     CK(cudaStreamWaitEvent(s, h->ev_inv, 0));
@@ -1261,58 +1366,22 @@ mg_status setup_hierarchy(mg_handle *h, const double *lam, const double *const f
     }
     CK(cudaGraphLaunch(sg->exec, s));
     h->enq += sg->kernels;
-    const LevelBuf &c = h->L[h->nlev - 1];
     // The coarsest inverse runs on the aux stream, overlapping the caller's
     // next work and the start of the next solve (whose cycles wait for it
     // before their coarsest solve).  A singular coarsest matrix is reported by
     // mg_solve.
     CK(cudaEventRecord(h->ev_asm, s));
     CK(cudaStreamWaitEvent(h->aux, h->ev_asm, 0));
-    cudaStream_t a = h->aux;
-    // band of the coarsest matrix: the farthest neighbour cell is n0 (2D)
-    // or n0*n1 (3D) cells away, two unknowns per cell
-    const int off = DIM == 3 ? c.n[0] * c.n[1] : c.n[0];
-    const int kl = std::min(h->nc - 1, 2 * off + 1);
-    if (h->nc <= kBandSmemMax) {
-        const size_t smem_lu = sizeof(double) * (size_t)h->nc * h->nc;
-        CK(raise_smem_limit((const void *)k_band_lu_warp, (int)(sizeof(double) * kBandSmemMax * kBandSmemMax)));
-        k_band_lu_warp<<<1, kLUThreads, smem_lu, a>>>(h->Mtmp, h->nc, kl, kl, h->piv, h->dinv, h->err_d);
-        const int smem_inv = (int)(sizeof(double) * inv_smem_doubles(h->nc, kl, kl));
-        CK(raise_smem_limit((const void *)k_band_inv_cols_warp,
-                            (int)(sizeof(double) * inv_smem_doubles(kBandSmemMax, kBandSmemMax - 1, kBandSmemMax - 1))));
-        k_band_inv_cols_warp<<<(h->nc + 31) / 32, dim3(32, kInvRows), smem_inv,
-                               a>>>(h->Mtmp, h->piv, h->dinv, h->nc, kl, kl, h->Minv, mixed ? h->Minv32 : nullptr,
-                                    h->err_d);
-    } else if (window_path(h->nc, kl)) {
-        // the band's active window in shared memory, then the columns of the inverse, a warp each
-        const long long wsm = band_window_smem(kl, kl);
-        const int warps = inv_block_warps(h->nc, kl);
-        const long long ism = band_inv_block_smem(h->nc, kl, kl, warps);
-        CK(raise_smem_limit((const void *)k_band_lu_window, (int)wsm));
-        CK(raise_smem_limit((const void *)k_band_inv_block, (int)ism));
-        double *Lb = h->Mwork, *Uc = h->Mwork + (long long)h->nc * kl;
-        if (lu_blocked_ok(h->nc, kl))
-            CK(launch_lu_blocked(a, h->Mtmp, h->nc, kl, h->piv, h->dinv, Lb, Uc, h->err_d));
-        else
-            k_band_lu_window<<<1, kWinThreads, (size_t)wsm, a>>>(h->Mtmp, h->nc, kl, kl, h->piv, h->dinv, Lb, Uc,
-                                                                 h->err_d);
-        if (h->coarse_factors)           // the cycles solve from Lb and the scaled Uc (k_coarse_lu)
-            k_scale_uc<<<lin_blocks((long long)h->nc * 2 * kl), 256, 0, a>>>(Uc, h->dinv, h->nc, kl, kl, h->err_d);
-        else
-            k_band_inv_block<<<(h->nc + warps - 1) / warps, 32 * warps, (size_t)ism, a>>>(
-                Lb, Uc, h->piv, h->dinv, h->nc, kl, kl, h->Minv, mixed ? h->Minv32 : nullptr, h->err_d);
-    } else {
-        k_band_lu<<<1, dim3(32, 32, 1), 0, a>>>(h->Mtmp, h->nc, kl, kl, h->piv, h->dinv, h->err_d);
-        k_band_inv_cols<<<(h->nc + 127) / 128, 128, 0, a>>>(h->Mtmp, h->piv, h->dinv, h->nc, kl, kl, h->Mwork,
-                                                            h->err_d);
-        k_transpose<<<lin_blocks((long long)h->nc * h->nc), 256, 0, a>>>(h->Mwork, h->Minv, h->nc);
-        if (mixed)
-            k_to_f32<<<lin_blocks((long long)h->nc * h->nc), 256, 0, a>>>(h->Minv, h->Minv32,
-                                                                         (long long)h->nc * h->nc);
+    // its kernels are one graph per handle: their arguments never change
+    if (!h->gcoarse) {
+        mg_status ce = MG_OK;
+        const mg_status e = capture(h, &h->gcoarse, &h->coarse_kernels, [&](cudaStream_t cs) { ce = enqueue_coarse(h, cs); });
+        if (ce) return ce;
+        if (e) return e;
     }
-    CK(cudaGetLastError());
-    CK(cudaEventRecord(h->ev_inv, a));
-    counted(h, h->nc <= kBandSmemMax || window_path(h->nc, kl) ? 2 : 4);
+    CK(cudaGraphLaunch(h->gcoarse, h->aux));
+    h->enq += h->coarse_kernels;
+    CK(cudaEventRecord(h->ev_inv, h->aux));
     // flags 1 and 2 come from the level kernels, which precede this copy on
     // the stream (the inverse on the private stream keeps running)
     CK(cudaMemcpyAsync(h->errh, h->err_d, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -1804,11 +1873,14 @@ mg_status mg_create(const mg_grid *grid, const mg_options *opt, void *workspace,
     h->arena_bytes = need;
     size_t dummy;
     plan(h, aligned, &dummy);
+    int prio_low = 0, prio_high = 0;
     if (cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking) != cudaSuccess ||
         cudaStreamCreateWithFlags(&h->cap2, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreate(&h->ev_a0) != cudaSuccess || cudaEventCreate(&h->ev_a1) != cudaSuccess ||
         cudaMallocHost(&h->astat_h, sizeof(AsyncStat)) != cudaSuccess ||
-        cudaStreamCreateWithFlags(&h->aux, cudaStreamNonBlocking) != cudaSuccess ||
+        // high priority: the coarsest factors are a chain of small kernels beside the caller's finest-level ones
+        cudaDeviceGetStreamPriorityRange(&prio_low, &prio_high) != cudaSuccess ||
+        cudaStreamCreateWithPriority(&h->aux, cudaStreamNonBlocking, prio_high) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->ev_asm, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->ev_inv, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->ev_last, cudaEventDisableTiming) != cudaSuccess ||
@@ -2339,6 +2411,7 @@ mg_status mg_destroy(mg_handle *h) {
     if (h->g64) cudaGraphExecDestroy(h->g64);
     if (h->gasync) cudaGraphExecDestroy(h->gasync);
     if (h->gcorr) cudaGraphExecDestroy(h->gcorr);
+    if (h->gcoarse) cudaGraphExecDestroy(h->gcoarse);
     for (auto &sg : h->gsetup)
         if (sg.exec) cudaGraphExecDestroy(sg.exec);
     if (h->g32) cudaGraphExecDestroy(h->g32);

@@ -1327,9 +1327,14 @@ __device__ __forceinline__ void band_lu_warp_block(double *__restrict__ M, int n
     for (int q = tid; q < n * n; q += nthr) M[q] = a[q];
 }
 
+// The factorisation kernels below return at once when *done is set (mg_coarse.cuh: that path's factors are good and
+// these are its fallback); NULL: they always run.
+__device__ __forceinline__ bool coarse_done(const int *done) { return done && *(volatile const int *)done; }
+
 __global__ void __launch_bounds__(kLUThreads) k_band_lu_warp(double *__restrict__ M, int n, int kl, int ku,
                                                              int *__restrict__ piv, double *__restrict__ dinv,
-                                                             int *__restrict__ err) {
+                                                             int *__restrict__ err, const int *done) {
+    if (coarse_done(done)) return;
     band_lu_warp_block(M, n, kl, ku, piv, dinv, err);
 }
 
@@ -1423,7 +1428,8 @@ __global__ void __launch_bounds__(32 * kInvRows) k_band_inv_cols_warp(const doub
                                                                       const double *__restrict__ dinv, int n, int kl,
                                                                       int ku, double *__restrict__ Minv,
                                                                       float *__restrict__ Minv32,
-                                                                      const int *__restrict__ err) {
+                                                                      const int *__restrict__ err, const int *done) {
+    if (coarse_done(done)) return;
     band_inv_cols_warp_block(M, piv, dinv, n, kl, ku, Minv, Minv32, blockIdx.x, err);
 }
 
@@ -1730,7 +1736,8 @@ __device__ __forceinline__ void band_lu_window_block(const double *__restrict__ 
 __global__ void __launch_bounds__(kWinThreads) k_band_lu_window(const double *__restrict__ M, int n, int kl, int ku,
                                                                 int *__restrict__ piv, double *__restrict__ dinv,
                                                                 double *__restrict__ Lb, double *__restrict__ Uc,
-                                                                int *__restrict__ err) {
+                                                                int *__restrict__ err, const int *done) {
+    if (coarse_done(done)) return;
     band_lu_window_block(M, n, kl, ku, piv, dinv, Lb, Uc, err);
 }
 
@@ -1939,7 +1946,8 @@ __global__ void __launch_bounds__(kLuBlockedThreads) k_band_lu_blocked(const dou
                                                                        double *__restrict__ dinv,
                                                                        double *__restrict__ Lb,
                                                                        double *__restrict__ Uc,
-                                                                       int *__restrict__ err) {
+                                                                       int *__restrict__ err, const int *done) {
+    if (coarse_done(done)) return;
     extern __shared__ double lbsm[];
     band_lu_blocked_block(M, n, kl, ku, piv, dinv, Lb, Uc, err, lbsm);
 }
@@ -2084,7 +2092,8 @@ __device__ __forceinline__ void scale_uc(double *__restrict__ Uc, const double *
 }
 
 __global__ void k_scale_uc(double *__restrict__ Uc, const double *__restrict__ dinv, int n, int kl, int ku,
-                           const int *__restrict__ err) {
+                           const int *__restrict__ err, const int *done) {
+    if (coarse_done(done)) return;
     scale_uc(Uc, dinv, n, kl, ku, err, blockIdx.x * (long long)blockDim.x + threadIdx.x,
              (long long)gridDim.x * blockDim.x);
 }
@@ -2175,18 +2184,6 @@ __device__ void coarse_lu_solve_block(const double *__restrict__ Lb, const doubl
         }
     }
     for (int i = tid; i < n; i += nt) x[i] = (R)(y[i] * dinv[i]);
-}
-
-template <typename R>
-__global__ void __launch_bounds__(kLuSolveThreads) k_coarse_lu(const double *__restrict__ Lb,
-                                                               const double *__restrict__ Uc,
-                                                               const int *__restrict__ piv,
-                                                               const double *__restrict__ dinv, int n, int kl, int ku,
-                                                               const R *__restrict__ b, R *__restrict__ x,
-                                                               const int *__restrict__ err) {
-    pdl_entry();
-    extern __shared__ double lusm[];
-    coarse_lu_solve_block<R>(Lb, Uc, piv, dinv, n, kl, ku, b, x, err, lusm);
 }
 
 }  // namespace cmg
