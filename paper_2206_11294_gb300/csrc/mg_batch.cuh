@@ -149,27 +149,19 @@ __global__ void __launch_bounds__(kBatchThreads) kb_prolong(const BLevel *__rest
     }
 }
 
-// Coarsest solves of all problems: one warp per row of x = Minv b.
+// Coarsest solves of all problems: blocks of rows of x = Minv b.
 template <typename R>
 __global__ void __launch_bounds__(kBatchThreads) kb_coarse(const BLevel *__restrict__ lv,
                                                            const BProb *__restrict__ pr,
                                                            const BState *__restrict__ st,
                                                            const int2 *__restrict__ tab, int n) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int v = blockIdx.x; v < n; v += gridDim.x) {
         const int2 e = tab[v];
         if (!st[e.x].active) continue;
         const BProb &P = pr[e.x];
-        const int row = e.y * (kBatchThreads / 32) + warp;
-        if (row >= P.nc) continue;
         const Level<R> C = pick<R>(lv[P.coarse]);
         const R *Mi = (const R *)(sizeof(R) == 8 ? (const void *)P.Minv : (const void *)P.Minv32);
-        const R *b = reinterpret_cast<const R *>(C.b);
-        R acc = R(0);
-        for (int c = lane; c < P.nc; c += 32) acc += Mi[(long long)row * P.nc + c] * b[c];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-        if (lane == 0) reinterpret_cast<R *>(C.x)[row] = acc;
+        coarse_matvec_block<R>(Mi, reinterpret_cast<const R *>(C.b), reinterpret_cast<R *>(C.x), P.nc, e.y);
     }
 }
 
@@ -935,7 +927,7 @@ mg_status mg_batch_create(int count, mg_handle *const *handles, mg_batch **out) 
         const dim3 gn = norm_grid(h->L[0], dim);
         add_blocks(tnorm, base[p], (long long)gn.x * gn.y * gn.z);
         if (!h->coarse_factors)
-            for (int r = 0; r < (h->nc + 7) / 8; r++) tco.push_back(make_int2(p, r));
+            for (int r = 0; r * coarse_rows_per_block(h->nc) < h->nc; r++) tco.push_back(make_int2(p, r));
         add_blocks(tcell, base[p], (h->L[0].N + kBatchThreads - 1) / kBatchThreads);
     }
     b->cells0g = slice(tn);

@@ -36,7 +36,8 @@ constexpr int kMaxLevels = 32;
 constexpr int kMaxCoarseUnknowns = 2048;
 constexpr int kSetupGraphs = 4;
 constexpr size_t kAlign = 256;
-constexpr size_t kTailSmemMax = 200 * 1024;   // shared memory a tail CTA may use
+constexpr size_t kTailSmemMax = 200 * 1024;   // state of a tail CTA the tuning rules allow; its staging stays below it
+constexpr int kTailSmemTop = 220 * 1024;      // dynamic shared memory of the tail kernel at most (beside 4 KB of descriptors)
 
 thread_local std::string g_err;
 
@@ -771,11 +772,10 @@ TailArgs<R> tail_args(const mg_handle *h, int first, int ctas, size_t *smem) {
     std::memset(&A, 0, sizeof(A));
     A.nlev = h->nlev - first;
     for (int q = 0; q < A.nlev; q++) A.L[q].g = view<R>(h->L[first + q]);
-    const int pairs = tail_layout(A, h->grid.dim, ctas);
-    *smem = (size_t)pairs * sizeof(typename Vec<R>::v2);
+    A.nc = h->nc;
+    *smem = tail_layout(A, h->grid.dim, ctas, kTailSmemMax);
     A.bc = bc_flags(h->grid);
     A.Minv = coarse_inverse<R>(h);
-    A.nc = h->nc;
     A.nu1 = h->opt.nu1;
     A.nu2 = h->opt.nu2;
     return A;
@@ -786,12 +786,23 @@ void enqueue_tail(const mg_handle *h, cudaStream_t s) {
     size_t smem = 0;
     TailArgs<R> A = tail_args<R>(h, h->tail_lev, h->tail_ctas, &smem);
     if (h->tail_ctas == 1) {                  // one CTA, no cluster
-        raise_smem_limit((const void *)k_vcycle_tail<R, DIM, false>, (int)kTailSmemMax);
-        launch_k(h, k_vcycle_tail<R, DIM, false>, 1, kBlock, smem, s, 0, A);
+        raise_smem_limit((const void *)k_vcycle_tail<R, DIM, false>, kTailSmemTop);
+        launch_k(h, k_vcycle_tail<R, DIM, false>, 1, kTailThreads, smem, s, 0, A);
         return;
     }
-    raise_smem_limit((const void *)k_vcycle_tail<R, DIM, true>, (int)kTailSmemMax);
-    launch_k(h, k_vcycle_tail<R, DIM, true>, dim3((unsigned)h->tail_ctas, 1, 1), kBlock, smem, s, h->tail_ctas, A);
+    raise_smem_limit((const void *)k_vcycle_tail<R, DIM, true>, kTailSmemTop);
+    launch_k(h, k_vcycle_tail<R, DIM, true>, dim3((unsigned)h->tail_ctas, 1, 1), kTailThreads, smem, s, h->tail_ctas, A);
+}
+
+// Whether level l's visit is the tail's.  A tail the tuning rules allow whose
+// colour-split state (rows padded to an even length) exceeds a block's shared
+// memory runs as separate launches: the result is the same.
+template <typename R>
+bool tail_here(const mg_handle *h, int l) {
+    if (l != h->tail_lev || !tail_runs(h)) return false;
+    size_t smem = 0;
+    tail_args<R>(h, l, h->tail_ctas, &smem);
+    return smem <= (size_t)kTailSmemTop;
 }
 
 template <typename R, int DIM>
@@ -805,7 +816,7 @@ template <typename R, int DIM>
 // red_done: the level's guess is zero with the first red half-sweep applied.
 void enqueue_vcycle(const mg_handle *h, cudaStream_t s, int l, int type, bool red_done) {
     const LevelBuf &lb = h->L[l];
-    if (l == h->tail_lev && tail_runs(h)) {
+    if (tail_here<R>(h, l)) {
         // the coarsest inverse is computed on the aux stream after each set-up
         // (a conditional body may hold no event node: the async solve waits first)
         if (!h->cond_body) cudaStreamWaitEvent(s, h->ev_inv, cudaEventWaitExternal);
@@ -826,9 +837,8 @@ void enqueue_vcycle(const mg_handle *h, cudaStream_t s, int l, int type, bool re
             counted(h);
             return;
         }
-        const int threads = 256;
-        const unsigned blocks = (unsigned)((h->nc * 32LL + threads - 1) / threads);
-        launch_k(h, k_coarse_matvec<R>, blocks, threads, 0, s, 0, coarse_inverse<R>(h), reinterpret_cast<const R *>(v.b),
+        const int per = coarse_rows_per_block(h->nc);
+        launch_k(h, k_coarse_matvec<R>, (unsigned)((h->nc + per - 1) / per), kReduceThreads, 0, s, 0, coarse_inverse<R>(h), reinterpret_cast<const R *>(v.b),
                                                       reinterpret_cast<R *>(v.x), h->nc);
         counted(h);
         return;
@@ -1633,10 +1643,13 @@ mg_status check_handle(const mg_handle *h, bool need_coeffs) {
 bool tail_level_ok(const mg_handle *h, int l, int ctas = kTailCtas) {
     if (h->coarse_factors) return false;     // the tail multiplies by the coarsest inverse
     if (!(l >= 1 && h->nlev - l >= 2 && h->nlev - l <= kTailMaxLevels && h->L[l].N <= kTailMaxCells)) return false;
-    size_t smem = 0;
-    if (h->opt.precision == MG_MIXED) tail_args<float>(h, l, ctas, &smem);
-    else tail_args<double>(h, l, ctas, &smem);
-    return smem <= kTailSmemMax;
+    long long pairs = 0;                     // x, b and bt of the slabs a CTA owns
+    for (int q = l; q < h->nlev; q++) {
+        const int *n = h->L[q].n;
+        const int S = h->grid.dim == 3 ? n[2] : n[1];
+        pairs += 3LL * ((S + ctas - 1) / ctas) * (h->L[q].N / S);
+    }
+    return (size_t)pairs * (h->opt.precision == MG_MIXED ? sizeof(float2) : sizeof(double2)) <= kTailSmemMax;
 }
 
 // 8 CTAs is a portable cluster size; 16 needs the kernel's opt-in and a
@@ -1653,7 +1666,7 @@ bool tail_ctas_allowed(int ctas) {
     cudaLaunchConfig_t cfg;
     std::memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3(16, 1, 1);
-    cfg.blockDim = kBlock;
+    cfg.blockDim = dim3(kTailThreads, 1, 1);
     cudaLaunchAttribute a;
     a.id = cudaLaunchAttributeClusterDimension;
     a.val.clusterDim.x = 16;

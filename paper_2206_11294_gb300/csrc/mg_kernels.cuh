@@ -118,6 +118,10 @@ __device__ __forceinline__ typename Vec<R>::v2 gs_update(const Level<R> &L, long
     return mk2<R>(bt.x - W.a * sT - W.b * sp, bt.y - W.c * sT - W.d * sp);
 }
 
+// A row of Dinv times a right-hand side, contracted the same way wherever a coarse level's bt is formed.
+__device__ __forceinline__ double dinv_row(double a, double b, double x, double y) { return fma(a, x, b * y); }
+__device__ __forceinline__ float dinv_row(float a, float b, float x, float y) { return fmaf(a, x, b * y); }
+
 // ---------------------------------------------------------------------------
 // Smoothing: one colour of a red-black block Gauss-Seidel sweep.  Each thread
 // owns one cell of the colour (red: i+j+k even) and solves its two rows for
@@ -449,7 +453,7 @@ __device__ __forceinline__ void residual_restrict_block(const Level<R> &F, const
     const R bT = aT * w, bp = ap * w;
     C.b[cc] = mk2<R>(bT, bp);
     const auto Di = ldgq(C.Dinv + cc);
-    const V2 z = mk2<R>(Di.a * bT + Di.b * bp, Di.c * bT + Di.d * bp);
+    const V2 z = mk2<R>(dinv_row(Di.a, Di.b, bT, bp), dinv_row(Di.c, Di.d, bT, bp));
     C.bt[cc] = z;
     C.x[cc] = red_start && !((I + J + K) & 1) ? z : mk2<R>(R(0), R(0));
 }
@@ -530,20 +534,63 @@ __global__ void __launch_bounds__(kBX * kBY) k_prolong_add(Level<R> C, Level<R> 
 
 // ---------------------------------------------------------------------------
 // Coarsest level: x = Minv b with the dense inverse of the level's matrix
-// (unknown order: (T, p) per cell).  One warp per row, fixed summation order.
+// (unknown order: (T, p) per cell), each row in a fixed summation order: up to
+// kBandSmemMax unknowns four lanes of a warp sum a quarter of the row each (the
+// FP64 pipe would otherwise spend five warp-wide additions on reducing one or
+// two products per lane), above that a warp per row.
 // ---------------------------------------------------------------------------
-template <typename R>
-__global__ void k_coarse_matvec(const R *__restrict__ Minv, const R *__restrict__ b, R *__restrict__ x, int n) {
-    pdl_entry();
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (warp >= n) return;
-    const R *row = Minv + (long long)warp * n;
+constexpr int kBandSmemMax = 128;
+
+// part 0..3 in adjacent lanes, whole warps; the sum in every lane.  pitch: entries between a row's columns.
+template <typename R, typename B>
+__device__ __forceinline__ R coarse_dot4(const R *__restrict__ row, int pitch, int n, int part, B b) {
     R acc = R(0);
-    for (int c = lane; c < n; c += 32) acc += row[c] * b[c];
+    const int c1 = n * (part + 1) / 4;
+#pragma unroll 8
+    for (int c = n * part / 4; c < c1; c++) acc += row[(long long)c * pitch] * b(c);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+    return acc;
+}
+
+// One warp; the sum in lane 0.
+template <typename R, typename B>
+__device__ __forceinline__ R coarse_dot32(const R *__restrict__ row, int n, int lane, B b) {
+    R acc = R(0);
+    for (int c = lane; c < n; c += 32) acc += row[c] * b(c);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if (lane == 0) x[warp] = acc;
+    return acc;
+}
+
+// Rows per block of kReduceThreads threads.
+__host__ __device__ __forceinline__ int coarse_rows_per_block(int n) {
+    return n <= kBandSmemMax ? kReduceThreads / 4 : kReduceThreads / 32;
+}
+
+// Block `blk` of the rows (kReduceThreads threads).
+template <typename R>
+__device__ __forceinline__ void coarse_matvec_block(const R *__restrict__ Minv, const R *__restrict__ b,
+                                                    R *__restrict__ x, int n, int blk) {
+    auto get = [&](int c) { return b[c]; };
+    const int tid = threadIdx.x, row0 = blk * coarse_rows_per_block(n);
+    if (n <= kBandSmemMax) {
+        const int row = row0 + (tid >> 2);
+        const R v = coarse_dot4<R>(Minv + (long long)min(row, n - 1) * n, 1, n, tid & 3, get);
+        if ((tid & 3) == 0 && row < n) x[row] = v;
+    } else {
+        const int row = row0 + (tid >> 5);
+        if (row >= n) return;
+        const R v = coarse_dot32<R>(Minv + (long long)row * n, n, tid & 31, get);
+        if ((tid & 31) == 0) x[row] = v;
+    }
+}
+
+template <typename R>
+__global__ void __launch_bounds__(kReduceThreads) k_coarse_matvec(const R *__restrict__ Minv, const R *__restrict__ b,
+                                                                  R *__restrict__ x, int n) {
+    pdl_entry();
+    coarse_matvec_block<R>(Minv, b, x, n, blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -1245,8 +1292,6 @@ __global__ void k_coarse_assemble(int n0, int n1, int n2, const double2 *__restr
 //   per lane and row groups on threadIdx.y: L U x = P e_j with the vectors in
 //   shared memory (column-interleaved) and the factors read as broadcasts;
 //   writes Minv (and Minv32).
-constexpr int kBandSmemMax = 128;
-
 __device__ __forceinline__ long long abs_bits(double v) {
     return __double_as_longlong(v) & 0x7fffffffffffffffLL;
 }
