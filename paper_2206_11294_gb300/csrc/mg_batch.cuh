@@ -49,6 +49,7 @@ struct BSetupLevel {            // one (problem, level) of the batched set-up
     SetupGeom gm;
     SetupOut out;
     SetupFine fine;             // the level below (coarse levels only)
+    int from_lam;               // level 1 of a Cartesian grid: the level below as lambda (SetupFine::lam)
     int problem;
     int *err;                   // the problem's set-up error flags
 };
@@ -231,14 +232,17 @@ __global__ void __launch_bounds__(kBatchThreads) kb_setup_fine(const BSetupLevel
 
 template <int DIM>
 __global__ void __launch_bounds__(kBatchThreads) kb_setup_coarse(const BSetupLevel *__restrict__ sl,
+                                                                 const SetupIn *__restrict__ in,
                                                                  const int2 *__restrict__ tab, int n) {
     for (int v = blockIdx.x; v < n; v += gridDim.x) {
         const int2 e = tab[v];
         const BSetupLevel &L = sl[e.x];
+        SetupFine fine = L.fine;
+        if (L.from_lam) fine.lam = in[L.problem].lam;
         const int gx = (L.gm.n[0] + kBX - 1) / kBX, gy = (L.gm.n[1] + kBY - 1) / kBY;
         int bx, by, bz;
         block_coords(e.y, gx, gy, bx, by, bz);
-        setup_coarse_block<DIM>(L.gm, L.fine, L.out, L.err, bx, by, bz);
+        setup_coarse_block<DIM>(L.gm, fine, L.out, L.err, bx, by, bz);
     }
 }
 
@@ -493,8 +497,10 @@ __global__ void __launch_bounds__(kBatchThreads) kb_norm(const BLevel *__restric
         if (!initial && !st[p].active) continue;
         const Level<double> L = B.d;
         int bx, by, bz;
-        block_coords(e.y, norm_gx(L.n0), norm_gy(L.n1), bx, by, bz);
-        const double2 s = (red && !initial) ? norm_block<DIM, true>(L, bx, by, bz) : norm_block<DIM, false>(L, bx, by, bz);
+        const int rows = norm_rows(L.N);
+        block_coords(e.y, norm_gx(L.n0), norm_gy(L.n1, rows), bx, by, bz);
+        const double2 s = (red && !initial) ? norm_block<DIM, true>(L, rows, bx, by, bz)
+                                               : norm_block<DIM, false>(L, rows, bx, by, bz);
         batch_finish(pr[p], st[p], e.y, s, initial, rtol, max_cycles, active_count);
     }
 }
@@ -514,12 +520,13 @@ __global__ void __launch_bounds__(kBatchThreads) kb_residual64(const BLevel *__r
         if (!initial && !st[p].active) continue;
         Level<double> L = B.d;
         int bx, by, bz;
-        block_coords(e.y, norm_gx(L.n0), norm_gy(L.n1), bx, by, bz);
+        const int rows = norm_rows(L.N);
+        block_coords(e.y, norm_gx(L.n0), norm_gy(L.n1, rows), bx, by, bz);
         // defect correction: the initial call stores r0 = b - A x0 over b and sets delta = 0; later calls
         // form r0 - A delta
         if (!initial) L.x = B.delta;
         const double2 s = residual64_to32_block<DIM>(L, B.f.b, B.f.bt, B.f.x, initial ? L.b : nullptr,
-                                                     initial ? B.delta : nullptr, red_start, bx, by, bz);
+                                                     initial ? B.delta : nullptr, red_start, rows, bx, by, bz);
         batch_finish(pr[p], st[p], e.y, s, initial, rtol, max_cycles, active_count);
     }
 }
@@ -956,17 +963,19 @@ mg_status mg_batch_create(int count, mg_handle *const *handles, mg_batch **out) 
         for (int l = 0; l < h->nlev; l++) {
             BSetupLevel &S = sl[base[p] + l];
             std::memset(&S, 0, sizeof(S));
+            S.gm.ih2 = 1.0 / (hl * hl);
             for (int a = 0; a < 3; a++) {
                 S.gm.n[a] = h->L[l].n[a];
                 for (int sd = 0; sd < 2; sd++)
-                    S.gm.fac[a][sd] = (a < dim && h->grid.bc[a][sd] == MG_BC_DIRICHLET) ? 2.0 : 0.0;
+                    S.gm.wb[a][sd] = (a < dim && h->grid.bc[a][sd] == MG_BC_DIRICHLET) ? 2.0 * S.gm.ih2 : 0.0;
             }
             S.gm.axisym = h->grid.axisym;
             S.gm.r0 = h->grid.r0;
             S.gm.h = hl;
-            S.gm.ih2 = 1.0 / (hl * hl);
             S.out = setup_out(h->L[l], mixed);
             if (l > 0) S.fine = setup_fine_of(h->L[l - 1], hl / 2.0);
+            if (l == 0 && !S.gm.axisym) S.out.S = nullptr;
+            S.from_lam = l == 1 && !S.gm.axisym ? 1 : 0;
             S.problem = p;
             S.err = h->err_d;
             hl *= 2.0;
@@ -1247,8 +1256,8 @@ mg_status mg_batch_set_coeffs(mg_batch *b, const double *const *lambda, const do
     for (size_t d = 0; d < b->setup_tab.size(); d++) {
         const int n = b->setup_tab[d].second;
         if (n == 0) continue;
-        if (dim == 2) kb_setup_coarse<2><<<batch_grid(b, n), kBlock, 0, s>>>(b->sl, b->tabs + b->setup_tab[d].first, n);
-        else kb_setup_coarse<3><<<batch_grid(b, n), kBlock, 0, s>>>(b->sl, b->tabs + b->setup_tab[d].first, n);
+        if (dim == 2) kb_setup_coarse<2><<<batch_grid(b, n), kBlock, 0, s>>>(b->sl, b->sin, b->tabs + b->setup_tab[d].first, n);
+        else kb_setup_coarse<3><<<batch_grid(b, n), kBlock, 0, s>>>(b->sl, b->sin, b->tabs + b->setup_tab[d].first, n);
         b->launches++;
     }
     const unsigned gy = (unsigned)std::min(b->count, 65535);

@@ -16,6 +16,7 @@
 #include <map>
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -245,9 +246,18 @@ dim3 cell_grid(const LevelBuf &l, int dim, int xthreads) {
                 (unsigned)(dim == 3 ? l.n[2] : 1));
 }
 
-// Blocks of the norm / FP64-residual kernels (64 x 32 cells each).
+// Blocks of the norm / FP64-residual kernels (64 x (8 norm_rows) cells each).
 dim3 norm_grid(const LevelBuf &l, int dim) {
-    return dim3((unsigned)norm_gx(l.n[0]), (unsigned)norm_gy(l.n[1]), (unsigned)(dim == 3 ? l.n[2] : 1));
+    return dim3((unsigned)norm_gx(l.n[0]), (unsigned)norm_gy(l.n[1], norm_rows(l.N)), (unsigned)(dim == 3 ? l.n[2] : 1));
+}
+
+// body(std::integral_constant<int, norm_rows(N)>)
+template <typename F>
+void with_norm_rows(long long N, F &&body) {
+    const int rows = norm_rows(N);
+    if (rows == 1) body(std::integral_constant<int, 1>());
+    else if (rows == 2) body(std::integral_constant<int, 2>());
+    else body(std::integral_constant<int, 4>());
 }
 
 bool window_path(int n, int kl);
@@ -903,17 +913,18 @@ template <int DIM>
 void enqueue_norm(const mg_handle *h, cudaStream_t s, bool after_sweep) {
     const LevelBuf &f = h->L[0];
     const dim3 ng = norm_grid(f, DIM);
-    if (after_sweep) {
-        if (h->persistent)
-            launch_k(h, k_norm_partials<DIM, true, true>, wave((const void *)k_norm_partials<DIM, true, true>, tiles_of(ng)), kBlock, 0, s, 0, view<double>(f), h->partial, h->ticket, h->norms_d);
-        else
-            launch_k(h, k_norm_partials<DIM, true, false>, ng, kBlock, 0, s, 0, view<double>(f), h->partial, h->ticket, h->norms_d);
-    } else {
-        if (h->persistent)
-            launch_k(h, k_norm_partials<DIM, false, true>, wave((const void *)k_norm_partials<DIM, false, true>, tiles_of(ng)), kBlock, 0, s, 0, view<double>(f), h->partial, h->ticket, h->norms_d);
-        else
-            launch_k(h, k_norm_partials<DIM, false, false>, ng, kBlock, 0, s, 0, view<double>(f), h->partial, h->ticket, h->norms_d);
-    }
+    with_norm_rows(f.N, [&](auto rows) {
+        constexpr int R = decltype(rows)::value;
+        auto run = [&](auto tile, auto wave_of) {
+            if (h->persistent)
+                launch_k(h, wave_of, wave((const void *)wave_of, tiles_of(ng)), kBlock, 0, s, 0, view<double>(f), h->partial,
+                         h->ticket, h->norms_d);
+            else
+                launch_k(h, tile, ng, kBlock, 0, s, 0, view<double>(f), h->partial, h->ticket, h->norms_d);
+        };
+        if (after_sweep) run(k_norm_partials<DIM, true, false, R>, k_norm_partials<DIM, true, true, R>);
+        else run(k_norm_partials<DIM, false, false, R>, k_norm_partials<DIM, false, true, R>);
+    });
     counted(h);
 }
 
@@ -937,12 +948,17 @@ void enqueue_residual_to32(const mg_handle *h, cudaStream_t s, bool initial = fa
     if (!initial) v.x = delta;
     double2 *r_out = initial ? f.b : nullptr;
     double2 *r_out2 = initial ? delta : nullptr;
-    if (h->persistent)
-        launch_k(h, k_residual64_to32<DIM, true>, wave((const void *)k_residual64_to32<DIM, true>, tiles_of(ng)), kBlock, 0, s, 0, 
-            v, f.b32, f.bt32, f.x32, r_out, r_out2, red_start(h), h->partial, h->ticket, h->norms_d);
-    else
-        launch_k(h, k_residual64_to32<DIM, false>, ng, kBlock, 0, s, 0, v, f.b32, f.bt32, f.x32, r_out, r_out2,
-                 red_start(h), h->partial, h->ticket, h->norms_d);
+    with_norm_rows(f.N, [&](auto rows) {
+        constexpr int R = decltype(rows)::value;
+        auto run = [&](auto kern, dim3 grid) {
+            launch_k(h, kern, grid, kBlock, 0, s, 0, v, f.b32, f.bt32, f.x32, r_out, r_out2, red_start(h), h->partial,
+                     h->ticket, h->norms_d);
+        };
+        if (h->persistent)
+            run(k_residual64_to32<DIM, true, R>, dim3(wave((const void *)k_residual64_to32<DIM, true, R>, tiles_of(ng))));
+        else
+            run(k_residual64_to32<DIM, false, R>, ng);
+    });
     counted(h);
 }
 
@@ -960,9 +976,15 @@ template <int DIM>
 void warm_waves() {
     warm_waves_r<double, DIM>();
     warm_waves_r<float, DIM>();
-    wave((const void *)k_norm_partials<DIM, true, true>, 1);
-    wave((const void *)k_norm_partials<DIM, false, true>, 1);
-    wave((const void *)k_residual64_to32<DIM, true>, 1);
+    auto of = [](auto rows) {
+        constexpr int R = decltype(rows)::value;
+        wave((const void *)k_norm_partials<DIM, true, true, R>, 1);
+        wave((const void *)k_norm_partials<DIM, false, true, R>, 1);
+        wave((const void *)k_residual64_to32<DIM, true, R>, 1);
+    };
+    of(std::integral_constant<int, 1>());
+    of(std::integral_constant<int, 2>());
+    of(std::integral_constant<int, 4>());
 }
 
 // FP64: one V-cycle, then the stopping norm, copied to pinned host memory.
@@ -1268,6 +1290,7 @@ SetupFine setup_fine_of(const LevelBuf &F, double h) {
     SetupFine s;
     s.n0 = F.n[0];
     s.n1 = F.n[1];
+    s.lam = nullptr;
     s.S = F.S;
     s.l4 = F.l4;
     for (int a = 0; a < 3; a++) s.G[a] = F.G[a] ? F.G[a] : F.G[0];
@@ -1283,7 +1306,9 @@ void enqueue_setup_levels(mg_handle *h, cudaStream_t s, const SetupGeom &gm, con
     const LevelBuf &f = h->L[0];
     cudaMemsetAsync(h->err_d, 0, sizeof(int), s);
     if (f.jflag) cudaMemsetAsync(h->err_d + 2, 0, sizeof(int), s);
-    launch_k(h, k_setup_fine<DIM>, cell_grid(f, DIM, f.n[0]), kBlock, 0, s, 0, gm, in, setup_out(f, mixed), h->err_d);
+    SetupOut fine = setup_out(f, mixed);
+    if (!gm.axisym) fine.S = nullptr;        // level 1 reads lambda
+    launch_k(h, k_setup_fine<DIM>, cell_grid(f, DIM, f.n[0]), kBlock, 0, s, 0, gm, in, fine, h->err_d);
     counted(h);
     double hl = h->grid.h;
     for (int l = 1; l < h->nlev; l++) {
@@ -1292,8 +1317,10 @@ void enqueue_setup_levels(mg_handle *h, cudaStream_t s, const SetupGeom &gm, con
         SetupGeom cg = gm;
         for (int a = 0; a < 3; a++) cg.n[a] = C.n[a];
         cg.h = 2.0 * hl;
-        launch_k(h, k_setup_coarse<DIM>, cell_grid(C, DIM, C.n[0]), kBlock, 0, s, 0, cg, setup_fine_of(F, hl),
-                 setup_out(C, mixed), h->err_d);
+        SetupFine below = setup_fine_of(F, hl);
+        if (l == 1 && !gm.axisym) below.lam = in.lam;
+        launch_k(h, k_setup_coarse<DIM>, cell_grid(C, DIM, C.n[0]), kBlock, 0, s, 0, cg, below, setup_out(C, mixed),
+                 h->err_d);
         counted(h);
         hl *= 2.0;
     }
@@ -1335,15 +1362,15 @@ mg_status setup_hierarchy(mg_handle *h, const double *lam, const double *const f
     }
     SetupGeom gm;
     std::memset(&gm, 0, sizeof(gm));
+    gm.ih2 = 1.0 / (g.h * g.h);
     for (int a = 0; a < 3; a++) {
         gm.n[a] = f.n[a];
         for (int sd = 0; sd < 2; sd++)
-            gm.fac[a][sd] = (a < DIM && g.bc[a][sd] == MG_BC_DIRICHLET) ? 2.0 : 0.0;
+            gm.wb[a][sd] = (a < DIM && g.bc[a][sd] == MG_BC_DIRICHLET) ? 2.0 * gm.ih2 : 0.0;
     }
     gm.axisym = g.axisym;
     gm.r0 = g.r0;
     gm.h = g.h;
-    gm.ih2 = 1.0 / (g.h * g.h);
     SetupIn in;
     in.lam = lam_d;
     for (int a = 0; a < 3; a++) {

@@ -50,10 +50,19 @@ __device__ __forceinline__ void block_coords(int local, int gx, int gy, int &bx,
             }                                                                            \
         }                                                                                \
     } while (0)
+// A 2x2 block by one 256-bit access (sm_100 and later; 32-byte aligned): a
+// lane's block is one sector, which two 128-bit accesses would touch twice.
 __device__ __forceinline__ dq ldgq(const dq *p) {
-    const double2 *q = reinterpret_cast<const double2 *>(p);
-    double2 u = __ldg(q), v = __ldg(q + 1);
-    return dq{u.x, u.y, v.x, v.y};
+    dq q;
+    asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];\n"
+        : "=d"(q.a), "=d"(q.b), "=d"(q.c), "=d"(q.d)
+        : "l"(__cvta_generic_to_global(p)));
+    return q;
+}
+__device__ __forceinline__ void stq(dq *p, const dq &q) {
+    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};\n" ::"l"(__cvta_generic_to_global(p)), "d"(q.a), "d"(q.b),
+                 "d"(q.c), "d"(q.d)
+                 : "memory");
 }
 __device__ __forceinline__ fq ldgq(const fq *p) {
     float4 u = __ldg(reinterpret_cast<const float4 *>(p));
@@ -596,30 +605,32 @@ __global__ void __launch_bounds__(kReduceThreads) k_coarse_matvec(const R *__res
 // ---------------------------------------------------------------------------
 // Norms.  Per cell z = Dinv (b - offdiag(x)) - x = Dinv r: the block-Jacobi
 // scaled residual, invariant under the row scaling.  Each block writes its
-// partial sums of z_T^2 and z_p^2; k_reduce_norms sums them in a fixed order.
+// partial sums of z_T^2 and z_p^2; the last block sums them in index order.
 // ---------------------------------------------------------------------------
+// Sums of a and b over a block of kReduceThreads threads, in thread 0.  The FP64
+// pipe takes a warp-wide addition as a whole whatever its lanes hold, so shuffle
+// trees in every warp (ten additions each) would be the larger part of a small
+// tile's work: the values meet in shared memory, warp 0 sums a and warp 1 b, one
+// column of eight per lane and then one tree each.
 __device__ __forceinline__ void block_sum2(double &a, double &b) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_down_sync(0xffffffffu, a, o);
-        b += __shfl_down_sync(0xffffffffu, b, o);
-    }
-    __shared__ double sa[32], sb[32];
+    __shared__ double sv[2][kReduceThreads];
+    __shared__ double res[2];
     const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
-    const int nthr = blockDim.x * blockDim.y * blockDim.z;
-    const int lane = tid & 31, w = tid >> 5;
-    if (lane == 0) { sa[w] = a; sb[w] = b; }
+    sv[0][tid] = a;
+    sv[1][tid] = b;
     __syncthreads();
-    if (w == 0) {
-        const int nw = (nthr + 31) >> 5;
-        a = lane < nw ? sa[lane] : 0.0;
-        b = lane < nw ? sb[lane] : 0.0;
+    const int w = tid >> 5, lane = tid & 31;
+    if (w < 2) {
+        double v = sv[w][lane];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            a += __shfl_down_sync(0xffffffffu, a, o);
-            b += __shfl_down_sync(0xffffffffu, b, o);
-        }
+        for (int r = 1; r < kReduceThreads / 32; r++) v += sv[w][32 * r + lane];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if (lane == 0) res[w] = v;
     }
+    __syncthreads();
+    a = res[0];
+    b = res[1];
 }
 
 // Last-block completion: after a block stored its partial, the block that
@@ -650,17 +661,19 @@ __device__ __forceinline__ void finish_norms(double2 *partial, int nblocks, unsi
     }
 }
 
-// Norm and FP64-residual tiles cover 64 x 32 cells (x, y) of one z-plane,
-// eight per thread (four rows unrolled, for loads in flight).  The solo
-// kernels run one persistent wave: each thread
-// accumulates the squares of all its tiles' cells with FMAs and the block
-// reduces once, so the FP64 reduction tree (shuffles, then one warp) is spread
-// over many cells; on a part with few FP64 units per SM it would otherwise
-// cost as much as the cells themselves.  (The batched kernels reduce per tile.)
+// Norm and FP64-residual tiles cover 64 columns and kBY x ROWS rows of one
+// z-plane, 2 x ROWS cells per thread (unrolled, for loads in flight).  ROWS
+// (norm_rows) trades the block's reduction, 24 warp-wide FP64 additions per
+// tile, against filling the chip: 4 rows make 512 tiles of a 1024^2 grid, 3.4
+// per SM, and the SMs with 4 set the time (the FP64 pipe of an average SM was
+// busy 61% of it); 2 rows make 6.7 per SM.  On small grids 1 row spreads the
+// cells over more SMs (64^2: 8 tiles instead of 2, 15.4 -> 8.3 us).  Each thread
+// accumulates its cells' squares with FMAs; a persistent block reduces once.
+// (The batched kernels reduce per tile.)
 constexpr int kNormCols = 64;
-constexpr int kNormRows = 4;   // rows per thread: the tile spans kBY * kNormRows rows
+__host__ __device__ __forceinline__ int norm_rows(long long N) { return N >= (1LL << 22) ? 4 : N >= (1LL << 17) ? 2 : 1; }
 __host__ __device__ __forceinline__ int norm_gx(int n0) { return (n0 + kNormCols - 1) / kNormCols; }
-__host__ __device__ __forceinline__ int norm_gy(int n1) { return (n1 + kBY * kNormRows - 1) / (kBY * kNormRows); }
+__host__ __device__ __forceinline__ int norm_gy(int n1, int rows) { return (n1 + kBY * rows - 1) / (kBY * rows); }
 
 template <int DIM>
 __device__ __forceinline__ void norm_cell(const Level<double> &L, int i, int j, int k, double &zT2, double &zp2) {
@@ -676,19 +689,19 @@ __device__ __forceinline__ void norm_cell(const Level<double> &L, int i, int j, 
 }
 
 // Sums of (Dinv r)_T^2 and (Dinv r)_p^2 over tile (bx, by, bz) of the norm
-// grid (ceil(n0/64), ceil(n1/32), n2), added to zT2, zp2 (norm_block: reduced
-// over the block, valid in thread 0).
+// grid (norm_gx, norm_gy, n2), added to zT2, zp2 (norm_block: reduced over the
+// block).
 //
 // RED: x has just come out of a red-black sweep, so the block residual of
 // the black cells is exactly zero (z = gs_update - x recomputes the very
 // update that produced x, bit for bit) and each thread visits the one red
 // cell of its column pair per row.
-template <int DIM, bool RED = false>
+template <int DIM, bool RED, int ROWS>
 __device__ __forceinline__ void norm_tile(const Level<double> &L, int bx, int by, int bz, double &zT2, double &zp2) {
     const int k = DIM == 3 ? bz : 0;
 #pragma unroll
-    for (int r = 0; r < kNormRows; r++) {
-        const int j = (by * kNormRows + r) * kBY + threadIdx.y;
+    for (int r = 0; r < ROWS; r++) {
+        const int j = (by * ROWS + r) * kBY + threadIdx.y;
         if (j >= L.n1) continue;
         if (RED) {
             const int i = bx * kNormCols + 2 * threadIdx.x + ((j + k) & 1);
@@ -703,20 +716,23 @@ __device__ __forceinline__ void norm_tile(const Level<double> &L, int bx, int by
     }
 }
 
-template <int DIM, bool RED = false>
-__device__ __forceinline__ double2 norm_block(const Level<double> &L, int bx, int by, int bz) {
+template <int DIM, bool RED>
+__device__ __forceinline__ double2 norm_block(const Level<double> &L, int rows, int bx, int by, int bz) {
     double zT2 = 0.0, zp2 = 0.0;
-    norm_tile<DIM, RED>(L, bx, by, bz, zT2, zp2);
+    if (rows == 1) norm_tile<DIM, RED, 1>(L, bx, by, bz, zT2, zp2);
+    else if (rows == 2) norm_tile<DIM, RED, 2>(L, bx, by, bz, zT2, zp2);
+    else norm_tile<DIM, RED, 4>(L, bx, by, bz, zT2, zp2);
     block_sum2(zT2, zp2);
     return make_double2(zT2, zp2);
 }
 
-template <int DIM, bool RED, bool P>
+template <int DIM, bool RED, bool P, int ROWS>
 __global__ void __launch_bounds__(kBX * kBY) k_norm_partials(Level<double> L, double2 *__restrict__ partial,
                                                            unsigned int *__restrict__ ticket, double *__restrict__ out) {
     pdl_entry();
     double zT2 = 0.0, zp2 = 0.0;     // a block's tiles accumulate, then one reduction
-    CMG_TILES(P, norm_gx(L.n0), norm_gy(L.n1), DIM == 3 ? L.n2 : 1, (norm_tile<DIM, RED>(L, bx, by, bz, zT2, zp2)));
+    CMG_TILES(P, norm_gx(L.n0), norm_gy(L.n1, ROWS), DIM == 3 ? L.n2 : 1,
+              (norm_tile<DIM, RED, ROWS>(L, bx, by, bz, zT2, zp2)));
     block_sum2(zT2, zp2);
     const int blk = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
     if (threadIdx.x == 0 && threadIdx.y == 0) partial[blk] = make_double2(zT2, zp2);
@@ -757,15 +773,15 @@ __device__ __forceinline__ void residual64_to32_cell(const Level<double> &L, flo
 }
 
 // Block (bx, by, bz) of the norm grid.
-template <int DIM>
+template <int DIM, int ROWS>
 __device__ __forceinline__ void residual64_to32_tile(const Level<double> &L, float2 *__restrict__ b32,
                                                      float2 *__restrict__ bt32, float2 *__restrict__ e32,
                                                      double2 *__restrict__ r_out, double2 *__restrict__ r_out2,
                                                      int red_start, int bx, int by, int bz, double &zT2, double &zp2) {
     const int k = DIM == 3 ? bz : 0;
 #pragma unroll
-    for (int r = 0; r < kNormRows; r++) {
-        const int j = (by * kNormRows + r) * kBY + threadIdx.y;
+    for (int r = 0; r < ROWS; r++) {
+        const int j = (by * ROWS + r) * kBY + threadIdx.y;
         if (j >= L.n1) continue;
 #pragma unroll
         for (int e = 0; e < 2; e++) {
@@ -779,14 +795,16 @@ template <int DIM>
 __device__ __forceinline__ double2 residual64_to32_block(const Level<double> &L, float2 *__restrict__ b32,
                                                          float2 *__restrict__ bt32, float2 *__restrict__ e32,
                                                          double2 *__restrict__ r_out, double2 *__restrict__ r_out2,
-                                                         int red_start, int bx, int by, int bz) {
+                                                         int red_start, int rows, int bx, int by, int bz) {
     double zT2 = 0.0, zp2 = 0.0;
-    residual64_to32_tile<DIM>(L, b32, bt32, e32, r_out, r_out2, red_start, bx, by, bz, zT2, zp2);
+    if (rows == 1) residual64_to32_tile<DIM, 1>(L, b32, bt32, e32, r_out, r_out2, red_start, bx, by, bz, zT2, zp2);
+    else if (rows == 2) residual64_to32_tile<DIM, 2>(L, b32, bt32, e32, r_out, r_out2, red_start, bx, by, bz, zT2, zp2);
+    else residual64_to32_tile<DIM, 4>(L, b32, bt32, e32, r_out, r_out2, red_start, bx, by, bz, zT2, zp2);
     block_sum2(zT2, zp2);
     return make_double2(zT2, zp2);
 }
 
-template <int DIM, bool P>
+template <int DIM, bool P, int ROWS>
 __global__ void __launch_bounds__(kBX * kBY) k_residual64_to32(Level<double> L, float2 *__restrict__ b32,
                                                              float2 *__restrict__ bt32, float2 *__restrict__ e32,
                                                              double2 *__restrict__ r_out,
@@ -796,8 +814,8 @@ __global__ void __launch_bounds__(kBX * kBY) k_residual64_to32(Level<double> L, 
                                                              double *__restrict__ out) {
     pdl_entry();
     double zT2 = 0.0, zp2 = 0.0;
-    CMG_TILES(P, norm_gx(L.n0), norm_gy(L.n1), DIM == 3 ? L.n2 : 1,
-              (residual64_to32_tile<DIM>(L, b32, bt32, e32, r_out, r_out2, red_start, bx, by, bz, zT2, zp2)));
+    CMG_TILES(P, norm_gx(L.n0), norm_gy(L.n1, ROWS), DIM == 3 ? L.n2 : 1,
+              (residual64_to32_tile<DIM, ROWS>(L, b32, bt32, e32, r_out, r_out2, red_start, bx, by, bz, zT2, zp2)));
     block_sum2(zT2, zp2);
     const int blk = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
     if (threadIdx.x == 0 && threadIdx.y == 0) partial[blk] = make_double2(zT2, zp2);
@@ -822,21 +840,6 @@ __global__ void k_add_correction(double2 *__restrict__ x, const float2 *__restri
         v.x += (double)d.x;
         v.y += (double)d.y;
         x[c] = v;
-    }
-}
-
-// Sums the partials in a fixed order; out[0..1] = sqrt of the sums.
-__global__ void __launch_bounds__(kReduceThreads) k_reduce_norms(const double2 *__restrict__ partial, int n,
-                                                                 double *__restrict__ out) {
-    double a = 0.0, b = 0.0;
-    for (int q = threadIdx.x; q < n; q += blockDim.x) {
-        a += partial[q].x;
-        b += partial[q].y;
-    }
-    block_sum2(a, b);
-    if (threadIdx.x == 0) {
-        out[0] = sqrt(a);
-        out[1] = sqrt(b);
     }
 }
 
@@ -957,7 +960,7 @@ __global__ void __launch_bounds__(kBX * kBY) k_apply_paper(const __grid_constant
 // ---------------------------------------------------------------------------
 struct SetupOut {                 // one level's outputs
     double2 *G[3];
-    dq *S, *D, *Dinv, *W;
+    dq *S, *D, *Dinv, *W;         // S NULL: not stored (SetupFine::lam)
     double *l4;
     float2 *G32[3];               // FP32 copies (mixed precision), or NULL
     fq *D32, *Dinv32, *W32;
@@ -976,12 +979,44 @@ struct SetupGeom {
     int axisym;
     double r0, h;                 // this level's spacing
     double ih2;                   // 1 / h^2 (finest level)
-    double fac[3][2];             // boundary factor per axis / side: 2 Dirichlet, 0 wall/axis
+    double wb[3][2];              // ih2 times the boundary factor per axis / side: 2 Dirichlet, 0 wall/axis
 };
 
-// Finite test on the bit pattern (integer pipe, not the scarce FP64 pipe).
+// Tests on the bit pattern (integer pipe, not the scarce FP64 pipe).  The words
+// come from inline assembly: written as an integer mask of the double, the
+// compiler turns the test back into an FP64 comparison, 16 of them per cell of
+// k_setup_fine<3>, a quarter of its FP64 instructions.
+__device__ __forceinline__ void words_of(double v, unsigned &lo, unsigned &hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "d"(v));
+}
 __device__ __forceinline__ bool finite_bits(double v) {
-    return (__double_as_longlong(v) & 0x7ff0000000000000LL) != 0x7ff0000000000000LL;
+    unsigned lo, hi;
+    words_of(v, lo, hi);
+    return (hi & 0x7ff00000u) != 0x7ff00000u;
+}
+__device__ __forceinline__ bool zero_bits(double v) {
+    unsigned lo, hi;
+    words_of(v, lo, hi);
+    return ((hi & 0x7fffffffu) | lo) == 0u;
+}
+
+// Bit patterns of finite doubles as integers in the values' order (negative ones reversed), and back.
+__device__ __forceinline__ long long order_bits(double v) {
+    const long long b = __double_as_longlong(v);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+__device__ __forceinline__ double from_order(long long k) {
+    return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffLL));
+}
+
+// A cell's l1..l4 of the caller's [N][4] array (16-byte aligned, or only 8).
+__device__ __forceinline__ dq load_lam(const double *lam, long long c) {
+    if ((reinterpret_cast<uintptr_t>(lam) & 15u) == 0) {     // the same in every thread
+        const double2 l12 = __ldg(reinterpret_cast<const double2 *>(lam) + 2 * c);
+        const double2 l34 = __ldg(reinterpret_cast<const double2 *>(lam) + 2 * c + 1);
+        return dq{l12.x, l12.y, l34.x, l34.y};
+    }
+    return dq{__ldg(lam + 4 * c), __ldg(lam + 4 * c + 1), __ldg(lam + 4 * c + 2), __ldg(lam + 4 * c + 3)};
 }
 
 template <int DIM>
@@ -1005,17 +1040,17 @@ __device__ __forceinline__ void finish_cell(const SetupOut &o, long long c, cons
                 }
             }
         }
-    o.S[c] = S;
+    if (o.S) stq(o.S + c, S);
     o.l4[c] = l4;
     dq D{S.a - sT, S.b, S.c - l4 * sT, S.d - sp};
     const double det = D.a * D.d - D.b * D.c;
-    if ((__double_as_longlong(det) & 0x7fffffffffffffffLL) == 0 || !finite_bits(det)) atomicOr(err, 2);
+    if (zero_bits(det) || !finite_bits(det)) atomicOr(err, 2);
     const double id = 1.0 / det;
     const dq Di{D.d * id, -D.b * id, -D.c * id, D.a * id};
     const dq Wc{Di.a + Di.b * l4, Di.b, Di.c + Di.d * l4, Di.d};
-    o.D[c] = D;
-    o.Dinv[c] = Di;
-    o.W[c] = Wc;
+    stq(o.D + c, D);
+    stq(o.Dinv + c, Di);
+    stq(o.W + c, Wc);
     if (o.D32) {
         o.D32[c] = fq{(float)D.a, (float)D.b, (float)D.c, (float)D.d};
         o.Dinv32[c] = fq{(float)Di.a, (float)Di.b, (float)Di.c, (float)Di.d};
@@ -1041,8 +1076,7 @@ struct SetupIn {
 
 // Finest level from lambda [N][4] and the per-axis arrays of 1/rho and k:
 // block (bx, by, bz) of the cell grid (ceil(n0/32), ceil(n1/8), n2).
-// AXI: faces carry r_f and the rows s_i = r_i; boundary faces (rare, a
-// separate branch) carry the boundary factor.
+// AXI: faces carry r_f and the rows s_i = r_i; boundary faces carry the boundary factor.
 template <int DIM, bool AXI>
 __device__ __forceinline__ void setup_fine_cells(const SetupGeom &gm, const SetupIn &in, const SetupOut &o, int *err,
                                                  int bx, int by, int bz) {
@@ -1050,50 +1084,34 @@ __device__ __forceinline__ void setup_fine_cells(const SetupGeom &gm, const Setu
     const int j = by * kBY + threadIdx.y;
     const int k = DIM == 3 ? bz : 0;
     if (i >= gm.n[0] || j >= gm.n[1]) return;
-    const double *lam = in.lam;
     const long long c = cell_id(i, j, k, gm.n[0], gm.n[1]);
-    const double l1 = lam[4 * c], l2 = lam[4 * c + 1], l3 = lam[4 * c + 2], l4 = lam[4 * c + 3];
+    const dq lam = load_lam(in.lam, c);
+    const double l1 = lam.a, l2 = lam.b, l3 = lam.c, l4 = lam.d;
     bool bad = !finite_bits(l1) || !finite_bits(l2) || !finite_bits(l3) || !finite_bits(l4);
     const double s = AXI ? gm.r0 + (i + 0.5) * gm.h : 1.0;
-    const double ih2 = gm.ih2;
     const double *const *fa = in.fa, *const *fk = in.fk;
     const int pos[3] = {i, j, k};
     long long fid[3][2];
     face_ids(gm.n, i, j, k, fid);
     int own[3][2];
     double2 g[3][2];
-    double kf[3][2], af[3][2], wf[3][2];
-    bool edge = false;
+    double kf[3][2], af[3][2];
 #pragma unroll
     for (int a = 0; a < DIM; a++)
 #pragma unroll
         for (int sd = 0; sd < 2; sd++) {
             const int fpos = pos[a] + sd;
-            // w = rho_f / h^2 (times r_f or r_i on axisymmetric grids)
-            double w = ih2;
+            // w = rho_f / h^2 (times r_f or r_i on axisymmetric grids), on boundary faces times their factor: a
+            // selected constant, where a branch on the boundary would be taken by two warps of every row
+            double w = fpos == 0 ? gm.wb[a][0] : fpos == gm.n[a] ? gm.wb[a][1] : gm.ih2;
             if (AXI) w *= (a == 0 ? gm.r0 + (i + sd) * gm.h : s);
             const double al = fa[a][fid[a][sd]], kk = fk[a][fid[a][sd]];
             bad = bad || !finite_bits(al) || !finite_bits(kk);
             kf[a][sd] = kk;
             af[a][sd] = al;
-            wf[a][sd] = w;
             g[a][sd] = make_double2(kk * w, al * w);
             own[a][sd] = sd == 0 || fpos == gm.n[a];
-            edge = edge || fpos == 0 || fpos == gm.n[a];
         }
-    if (edge) {
-        // boundary faces: w times the factor (2 Dirichlet, 0 wall / axis)
-#pragma unroll
-        for (int a = 0; a < DIM; a++)
-#pragma unroll
-            for (int sd = 0; sd < 2; sd++) {
-                const int fpos = pos[a] + sd;
-                if (fpos == 0 || fpos == gm.n[a]) {
-                    const double w = wf[a][sd] * (fpos == 0 ? gm.fac[a][0] : gm.fac[a][1]);
-                    g[a][sd] = make_double2(kf[a][sd] * w, af[a][sd] * w);
-                }
-            }
-    }
     if (bad) atomicOr(err, 1);
     const dq S = AXI ? dq{s * l1, s * l2, 0.0, s * l3} : dq{l1, l2, 0.0, l3};
     finish_cell<DIM>(o, c, fid, own, g, S, l4, err);
@@ -1101,7 +1119,9 @@ __device__ __forceinline__ void setup_fine_cells(const SetupGeom &gm, const Setu
         // a coefficient jump at this cell: its interior faces' k or 1/rho
         // differ by more than the ratio; its 2x2 block is then applied in FP64
         // by the FP32 cycles (marked by a NaN first entry of its FP32 W)
-        double kmin = 0.0, kmax = 0.0, amin = 0.0, amax = 0.0;
+        // (minima and maxima on the bit patterns: FP64 comparisons would take
+        // the FP64 pipe, a third of this kernel's work)
+        long long kmin = 0, kmax = 0, amin = 0, amax = 0;
         bool any = false;
 #pragma unroll
         for (int a = 0; a < DIM; a++)
@@ -1109,14 +1129,15 @@ __device__ __forceinline__ void setup_fine_cells(const SetupGeom &gm, const Setu
             for (int sd = 0; sd < 2; sd++) {
                 const int fpos = pos[a] + sd;
                 if (fpos == 0 || fpos == gm.n[a]) continue;
-                const double kk = kf[a][sd], al = af[a][sd];
-                kmin = any ? fmin(kmin, kk) : kk;
-                kmax = any ? fmax(kmax, kk) : kk;
-                amin = any ? fmin(amin, al) : al;
-                amax = any ? fmax(amax, al) : al;
+                const long long kk = order_bits(kf[a][sd]), al = order_bits(af[a][sd]);
+                kmin = any ? min(kmin, kk) : kk;
+                kmax = any ? max(kmax, kk) : kk;
+                amin = any ? min(amin, al) : al;
+                amax = any ? max(amax, al) : al;
                 any = true;
             }
-        const bool jump = any && (kmax > o.jratio * kmin || amax > o.jratio * amin);
+        const bool jump = any && (from_order(kmax) > o.jratio * from_order(kmin) ||
+                                  from_order(amax) > o.jratio * from_order(amin));
         o.jflag[c] = jump ? 1 : 0;
         if (jump) {
             reinterpret_cast<float *>(o.W32 + c)[0] = __int_as_float(0x7fc00000);
@@ -1143,8 +1164,11 @@ __global__ void __launch_bounds__(kBX * kBY) k_setup_fine(SetupGeom gm, SetupIn 
 // volume-weighted mean of theirs, each face the sum of its 2^(DIM-1) fine
 // faces / 2^(DIM+1) (area-weighted mean coefficient re-discretised at 2h).
 // The level below, as the coarsening reads it.
+// lam: on Cartesian grids the finest level's S and l4 are the caller's lambda
+// itself, and level 1 coarsens that instead of a stored copy (NULL: S and l4).
 struct SetupFine {
     int n0, n1;
+    const double *lam;
     const dq *S;
     const double *l4;
     const double2 *G[3];
@@ -1170,16 +1194,25 @@ __device__ __forceinline__ void setup_coarse_cells(const SetupGeom &cg, const Se
     for (int q = 0; q < (1 << DIM); q++) {
         const int i = 2 * I + (q & 1);
         const long long f = cell_id(i, 2 * J + ((q >> 1) & 1), DIM == 3 ? 2 * K + (q >> 2) : 0, fn0, fn1);
-        const dq sf = Sf[f];
+        dq sf;
+        double w4;
+        if (!AXI && F.lam) {                             // the same branch in every thread
+            const dq q4 = load_lam(F.lam, f);
+            sf = dq{q4.a, q4.b, 0.0, q4.c};
+            w4 = q4.d;
+        } else {
+            sf = ldgq(Sf + f);
+            w4 = __ldg(l4f + f);
+        }
         // sums start from the first child: an addition to 0.0 would still take an FP64 issue slot
         if (q == 0) { a0 = sf.a; a1 = sf.b; a3 = sf.d; }
         else { a0 += sf.a; a1 += sf.b; a3 += sf.d; }
         if (AXI) {
             const double sc = cg.r0 + (i + 0.5) * hf;
-            if (q == 0) { v4 = sc * l4f[f]; vs = sc; }
-            else { v4 += sc * l4f[f]; vs += sc; }
+            if (q == 0) { v4 = sc * w4; vs = sc; }
+            else { v4 += sc * w4; vs += sc; }
         } else {
-            v4 = q == 0 ? l4f[f] : v4 + l4f[f];
+            v4 = q == 0 ? w4 : v4 + w4;
         }
     }
     const double wb = 1.0 / (1 << DIM);
