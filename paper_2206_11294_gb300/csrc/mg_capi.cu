@@ -2267,13 +2267,12 @@ mg_status mg_energy_async(const mg_grid *grid, const mg_phase phases[2], double 
     }
     A.r0 = grid->r0;
     A.h = grid->h;
-    A.inv_h = 1.0 / grid->h;
-    A.half_inv_h = 0.5 / grid->h;
     A.two_inv_h = 2.0 / grid->h;
-    A.dt = dt;
+    A.dt_h = dt / grid->h;
     for (int q = 0; q < 2; q++) {
         A.k[q] = phases[q].k;
-        A.mu[q] = phases[q].mu;
+        A.k_h[q] = phases[q].k / grid->h;
+        A.mu_8h[q] = phases[q].mu * 0.125 / grid->h;
     }
     A.x = reinterpret_cast<const double2 *>(x);
     A.C = C;

@@ -53,9 +53,7 @@ MomArgs momentum_args(const mg_momentum *m) {
     A.no_slip = (m->flags & MG_MOMENTUM_NO_SLIP) ? 1 : 0;
     A.r0 = g.r0;
     A.h = g.h;
-    A.inv_h = 1.0 / g.h;
-    A.half_inv_h = 0.5 / g.h;
-    A.two_inv_h = 2.0 / g.h;
+    A.div_scale = 0.5 / (g.h * g.h);
     A.inv_dt = 1.0 / m->dt;
     A.dt = m->dt;
     A.rho_dt = m->rho_dt;
@@ -376,6 +374,7 @@ mg_status mg_momentum_set_coeffs(mg_momentum *m, double dt, const double *rho, c
     A.dt = dt;
     A.inv_dt = 1.0 / dt;
     A.inv_h2 = 1.0 / (g.h * g.h);
+    A.half_inv_h2 = 0.5 * A.inv_h2;
     A.rho = rho;
     A.mu = mu;
     A.partial = m->partial;        // one Jacobi bound per block
@@ -549,8 +548,6 @@ MomSideArgs side_args(const mg_grid *grid, double dt) {
             A.gp[a][sd] = a < grid->dim ? grid->bc_p[a][sd] : 0.0;
         }
     }
-    A.inv_h = 1.0 / grid->h;
-    A.two_inv_h = 2.0 / grid->h;
     A.half_inv_h = 0.5 / grid->h;
     A.dt = dt;
     A.inv_dt = 1.0 / dt;
@@ -573,7 +570,7 @@ mg_status mg_momentum_rhs_async(const mg_grid *grid, double dt, double sigma, co
     for (int a = 0; a < dim; a++)
         if (R[a] == p || R[a] == C || R[a] == kappa) return fail(MG_ERR_INVALID_ARG, "R must not alias p, C or kappa");
     MomSideArgs A = side_args(grid, dt);
-    A.sigma = sigma;
+    A.sigma_half_inv_h = sigma * A.half_inv_h;
     A.p = p;
     A.C = C;
     A.kappa = kappa;
