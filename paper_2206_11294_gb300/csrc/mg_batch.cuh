@@ -49,6 +49,7 @@ struct BSetupLevel {            // one (problem, level) of the batched set-up
     SetupGeom gm;
     SetupOut out;
     SetupFine fine;             // the level below (coarse levels only)
+    int count;                  // first level of a chain: the chain's levels (the next entries)
     int from_lam;               // level 1 of a Cartesian grid: the level below as lambda (SetupFine::lam)
     int problem;
     int *err;                   // the problem's set-up error flags
@@ -230,19 +231,28 @@ __global__ void __launch_bounds__(kBatchThreads) kb_setup_fine(const BSetupLevel
     }
 }
 
-template <int DIM>
+// Chains of coarse levels (k_setup_coarse); e.x: a chain's first level.  ONE: chains of a single level.
+template <int DIM, bool ONE>
 __global__ void __launch_bounds__(kBatchThreads) kb_setup_coarse(const BSetupLevel *__restrict__ sl,
                                                                  const SetupIn *__restrict__ in,
                                                                  const int2 *__restrict__ tab, int n) {
+    ChainTile<DIM> *T = nullptr;
+    if constexpr (!ONE) {
+        __shared__ ChainTile<DIM> tile;
+        T = &tile;
+    }
     for (int v = blockIdx.x; v < n; v += gridDim.x) {
         const int2 e = tab[v];
         const BSetupLevel &L = sl[e.x];
         SetupFine fine = L.fine;
         if (L.from_lam) fine.lam = in[L.problem].lam;
-        const int gx = (L.gm.n[0] + kBX - 1) / kBX, gy = (L.gm.n[1] + kBY - 1) / kBY;
-        int bx, by, bz;
+        auto out = [&](int q) -> const SetupOut & { return sl[e.x + q].out; };
+        int gx, gy, gz, bx, by, bz;
+        chain_blocks(DIM, L.gm.n, &gx, &gy, &gz);
         block_coords(e.y, gx, gy, bx, by, bz);
-        setup_coarse_block<DIM>(L.gm, fine, L.out, L.err, bx, by, bz);
+        if (!ONE) __syncthreads();                   // the tile before this one is done with T
+        if (DIM == 2 && L.gm.axisym) setup_chain_cells<DIM, true, ONE>(L.gm, fine, out, L.count, L.err, bx, by, bz, T);
+        else setup_chain_cells<DIM, false, ONE>(L.gm, fine, out, L.count, L.err, bx, by, bz, T);
     }
 }
 
@@ -613,7 +623,8 @@ struct mg_batch {
     int max_nc_small;
     std::vector<int> big_coarse;      // problems whose coarsest inverse takes the banded three-kernel path
     std::pair<long long, int> setup_fine_tab;
-    std::vector<std::pair<long long, int>> setup_tab;   // depth 1.. (all levels at that depth)
+    std::vector<std::pair<long long, int>> setup_tab;   // chains of coarse levels, by the depth of their first
+    std::vector<bool> setup_one;                         // of a single level each
     char *host_io;                    // pinned staging for the per-call pointer tables
     int *err_d, *err_h;               // per-problem set-up error flags (device, pinned host)
 };
@@ -942,15 +953,22 @@ mg_status mg_batch_create(int count, mg_handle *const *handles, mg_batch **out) 
     b->coarse = slice(tco);
     b->cells0 = slice(tcell);
     b->setup_fine_tab = b->cells0g;
-    for (int d = 1; d < b->dmax; d++) {
+    // chains of coarse levels: a depth with many cells over the whole batch goes alone
+    std::vector<int> chain(b->dmax, 0);          // levels of the chain that starts at a depth
+    for (int d = 1; d < b->dmax; d += chain[d]) {
+        long long cells = 0;
+        for (int p = 0; p < count; p++) cells += handles[p]->nlev > d ? handles[p]->L[d].N : 0;
+        chain[d] = cells >= kChainCells ? 1 : setup_chain(dim);
         std::vector<int2> ts;
         for (int p = 0; p < count; p++) {
             const mg_handle *h = handles[p];
             if (h->nlev <= d) continue;
-            const dim3 gl = cell_grid(h->L[d], dim, h->L[d].n[0]);
-            add_blocks(ts, base[p] + d, (long long)gl.x * gl.y * gl.z);
+            int gx, gy, gz;
+            chain_blocks(dim, h->L[d].n, &gx, &gy, &gz);
+            add_blocks(ts, base[p] + d, (long long)gx * gy * gz);
         }
         b->setup_tab.push_back(slice(ts));
+        b->setup_one.push_back(chain[d] == 1);
     }
     // set-up descriptors, one per (problem, level), same indexing as lv
     std::vector<BSetupLevel> sl(lv.size());
@@ -960,6 +978,7 @@ mg_status mg_batch_create(int count, mg_handle *const *handles, mg_batch **out) 
         const mg_handle *h = handles[p];
         const bool mixed = h->opt.precision == MG_MIXED;
         double hl = h->grid.h;
+        int left = 0;                            // levels of the current chain from this one on
         for (int l = 0; l < h->nlev; l++) {
             BSetupLevel &S = sl[base[p] + l];
             std::memset(&S, 0, sizeof(S));
@@ -976,6 +995,9 @@ mg_status mg_batch_create(int count, mg_handle *const *handles, mg_batch **out) 
             if (l > 0) S.fine = setup_fine_of(h->L[l - 1], hl / 2.0);
             if (l == 0 && !S.gm.axisym) S.out.S = nullptr;
             S.from_lam = l == 1 && !S.gm.axisym ? 1 : 0;
+            if (l > 0 && chain[l] > 0) left = std::min(chain[l], h->nlev - l);
+            S.count = l > 0 && chain[l] > 0 ? left : 0;
+            if (l > 0 && --left > 0) S.out.S = nullptr;      // read by its own block only
             S.problem = p;
             S.err = h->err_d;
             hl *= 2.0;
@@ -1256,8 +1278,9 @@ mg_status mg_batch_set_coeffs(mg_batch *b, const double *const *lambda, const do
     for (size_t d = 0; d < b->setup_tab.size(); d++) {
         const int n = b->setup_tab[d].second;
         if (n == 0) continue;
-        if (dim == 2) kb_setup_coarse<2><<<batch_grid(b, n), kBlock, 0, s>>>(b->sl, b->sin, b->tabs + b->setup_tab[d].first, n);
-        else kb_setup_coarse<3><<<batch_grid(b, n), kBlock, 0, s>>>(b->sl, b->sin, b->tabs + b->setup_tab[d].first, n);
+        auto run = [&](auto kern) { kern<<<batch_grid(b, n), kBlock, 0, s>>>(b->sl, b->sin, b->tabs + b->setup_tab[d].first, n); };
+        if (dim == 2) run(b->setup_one[d] ? kb_setup_coarse<2, true> : kb_setup_coarse<2, false>);
+        else run(b->setup_one[d] ? kb_setup_coarse<3, true> : kb_setup_coarse<3, false>);
         b->launches++;
     }
     const unsigned gy = (unsigned)std::min(b->count, 65535);

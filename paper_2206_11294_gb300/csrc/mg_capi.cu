@@ -1311,18 +1311,27 @@ void enqueue_setup_levels(mg_handle *h, cudaStream_t s, const SetupGeom &gm, con
     launch_k(h, k_setup_fine<DIM>, cell_grid(f, DIM, f.n[0]), kBlock, 0, s, 0, gm, in, fine, h->err_d);
     counted(h);
     double hl = h->grid.h;
-    for (int l = 1; l < h->nlev; l++) {
+    for (int l = 1; l < h->nlev;) {
         const LevelBuf &F = h->L[l - 1];
-        const LevelBuf &C = h->L[l];
-        SetupGeom cg = gm;
-        for (int a = 0; a < 3; a++) cg.n[a] = C.n[a];
-        cg.h = 2.0 * hl;
-        SetupFine below = setup_fine_of(F, hl);
-        if (l == 1 && !gm.axisym) below.lam = in.lam;
-        launch_k(h, k_setup_coarse<DIM>, cell_grid(C, DIM, C.n[0]), kBlock, 0, s, 0, cg, below, setup_out(C, mixed),
-                 h->err_d);
+        SetupChain C;
+        std::memset(&C, 0, sizeof(C));
+        C.g = gm;
+        for (int a = 0; a < 3; a++) C.g.n[a] = h->L[l].n[a];
+        C.g.h = 2.0 * hl;
+        C.F = setup_fine_of(F, hl);
+        if (l == 1 && !gm.axisym) C.F.lam = in.lam;
+        C.count = h->L[l].N >= kChainCells ? 1 : std::min(setup_chain(DIM), h->nlev - l);
+        for (int q = 0; q < C.count; q++) {
+            C.o[q] = setup_out(h->L[l + q], mixed);
+            if (q + 1 < C.count) C.o[q].S = nullptr;      // read by its own block only
+            hl *= 2.0;
+        }
+        int gx, gy, gz;
+        chain_blocks(DIM, C.g.n, &gx, &gy, &gz);
+        launch_k(h, C.count == 1 ? k_setup_coarse<DIM, true> : k_setup_coarse<DIM, false>,
+                 dim3((unsigned)gx, (unsigned)gy, (unsigned)gz), kBlock, 0, s, 0, C, h->err_d);
         counted(h);
-        hl *= 2.0;
+        l += C.count;
     }
     const LevelBuf &c = h->L[h->nlev - 1];
     cudaMemsetAsync(h->Mtmp, 0, sizeof(double) * h->nc * h->nc, s);

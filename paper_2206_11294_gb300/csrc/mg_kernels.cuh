@@ -1160,7 +1160,19 @@ __global__ void __launch_bounds__(kBX * kBY) k_setup_fine(SetupGeom gm, SetupIn 
               (setup_fine_block<DIM>(gm, in, o, err, bx, by, bz)));
 }
 
-// Coarse level from the level below: S = mean of the children's S, l4 the
+// v / 2^K, exactly, by the exponent (the integer pipe); subnormal results, infinities and NaN by a multiplication.
+template <int K>
+__device__ __noinline__ double scale_down_slow(double v) { return v * (1.0 / (1 << K)); }
+template <int K>
+__device__ __forceinline__ double scale_down(double v) {
+    unsigned lo, hi;
+    words_of(v, lo, hi);
+    const unsigned e = hi & 0x7ff00000u;
+    if (e - ((K + 1u) << 20) < 0x7ff00000u - ((K + 1u) << 20)) return __hiloint2double((int)(hi - ((unsigned)K << 20)), (int)lo);
+    return ((hi & 0x7fffffffu) | lo) == 0u ? v : scale_down_slow<K>(v);
+}
+
+// Coarse levels from the level below: S = mean of the children's S, l4 the
 // volume-weighted mean of theirs, each face the sum of its 2^(DIM-1) fine
 // faces / 2^(DIM+1) (area-weighted mean coefficient re-discretised at 2h).
 // The level below, as the coarsening reads it.
@@ -1175,57 +1187,34 @@ struct SetupFine {
     double h;
 };
 
-template <int DIM, bool AXI>
-__device__ __forceinline__ void setup_coarse_cells(const SetupGeom &cg, const SetupFine &F, const SetupOut &o,
-                                                   int *err, int bx, int by, int bz) {
-    const int I = bx * kBX + threadIdx.x;
-    const int J = by * kBY + threadIdx.y;
-    const int K = DIM == 3 ? bz : 0;
-    if (I >= cg.n[0] || J >= cg.n[1]) return;
-    const int fn0 = F.n0, fn1 = F.n1;
-    const dq *Sf = F.S;
-    const double *l4f = F.l4;
-    const double hf = F.h;
-    const long long cc = cell_id(I, J, K, cg.n[0], cg.n[1]);
+// One coarse cell's S, l4 and faces: child(i, j, k, S, l4) gives a fine cell's, face(a, i, j, k) the fine face of
+// axis a at that position.
+template <int DIM, bool AXI, typename Child, typename Face>
+__device__ __forceinline__ void coarse_values(double r0, double hf, int I, int J, int K, Child child, Face face, dq &S,
+                                              double &l4, double2 g[3][2]) {
     // S = s [[l1, l2], [0, l3]] on every level: its lower-left entry is zero
     // by construction and is neither summed nor scaled
     double a0 = 0, a1 = 0, a3 = 0, v4 = 0, vs = 0;
 #pragma unroll
     for (int q = 0; q < (1 << DIM); q++) {
         const int i = 2 * I + (q & 1);
-        const long long f = cell_id(i, 2 * J + ((q >> 1) & 1), DIM == 3 ? 2 * K + (q >> 2) : 0, fn0, fn1);
         dq sf;
         double w4;
-        if (!AXI && F.lam) {                             // the same branch in every thread
-            const dq q4 = load_lam(F.lam, f);
-            sf = dq{q4.a, q4.b, 0.0, q4.c};
-            w4 = q4.d;
-        } else {
-            sf = ldgq(Sf + f);
-            w4 = __ldg(l4f + f);
-        }
+        child(i, 2 * J + ((q >> 1) & 1), DIM == 3 ? 2 * K + (q >> 2) : 0, sf, w4);
         // sums start from the first child: an addition to 0.0 would still take an FP64 issue slot
         if (q == 0) { a0 = sf.a; a1 = sf.b; a3 = sf.d; }
         else { a0 += sf.a; a1 += sf.b; a3 += sf.d; }
         if (AXI) {
-            const double sc = cg.r0 + (i + 0.5) * hf;
+            const double sc = r0 + (i + 0.5) * hf;
             if (q == 0) { v4 = sc * w4; vs = sc; }
             else { v4 += sc * w4; vs += sc; }
         } else {
             v4 = q == 0 ? w4 : v4 + w4;
         }
     }
-    const double wb = 1.0 / (1 << DIM);
-    const dq S{a0 * wb, a1 * wb, 0.0, a3 * wb};
-    const double l4 = AXI ? v4 / vs : v4 * wb;   // volume-weighted mean (a power-of-two mean is exact as a product)
+    S = dq{scale_down<DIM>(a0), scale_down<DIM>(a1), 0.0, scale_down<DIM>(a3)};
+    l4 = AXI ? v4 / vs : scale_down<DIM>(v4);   // volume-weighted mean
     const int P[3] = {I, J, K};
-    const int fm[3][2] = {{fn0 + 1, fn1}, {fn0, fn1 + 1}, {fn0, fn1}};   // fine face array dims (x, y) per axis
-    const double2 *const *Gf = F.G;
-    long long fid[3][2];
-    face_ids(cg.n, I, J, K, fid);
-    int own[3][2];
-    double2 g[3][2];
-    const double wf = 1.0 / (1 << (DIM + 1));
 #pragma unroll
     for (int a = 0; a < DIM; a++)
 #pragma unroll
@@ -1244,30 +1233,159 @@ __device__ __forceinline__ void setup_coarse_cells(const SetupGeom &cg, const Se
 #pragma unroll
                 for (int b = 0; b < 3; b++) fpos[b] = (b == a) ? 2 * (P[b] + sd) : 2 * P[b] + off[b];
                 if (DIM == 2) fpos[2] = 0;
-                const double2 v = Gf[a][(long long)fpos[0] + (long long)fm[a][0] * ((long long)fpos[1] +
-                                                                                  (long long)fm[a][1] * fpos[2])];
+                const double2 v = face(a, fpos[0], fpos[1], fpos[2]);
                 if (q == 0) { sT = v.x; sp = v.y; }
                 else { sT += v.x; sp += v.y; }
             }
-            g[a][sd] = make_double2(sT * wf, sp * wf);
-            own[a][sd] = sd == 0 || P[a] + sd == cg.n[a];
+            g[a][sd] = make_double2(scale_down<DIM + 1>(sT), scale_down<DIM + 1>(sp));
         }
-    finish_cell<DIM>(o, cc, fid, own, g, S, l4, err);
 }
 
-template <int DIM>
-__device__ __forceinline__ void setup_coarse_block(const SetupGeom &cg, const SetupFine &F, const SetupOut &o,
-                                                   int *err, int bx, int by, int bz) {
-    if (cg.axisym) setup_coarse_cells<DIM, true>(cg, F, o, err, bx, by, bz);
-    else setup_coarse_cells<DIM, false>(cg, F, o, err, bx, by, bz);
+// Up to setup_chain(DIM) levels per launch.  A block forms its tile of the
+// first level (32 x 8 cells, 3D 8 x 8 x 4) from the level below in global
+// memory and keeps S, l4 and the faces in shared memory; the tile's cells of
+// each further level follow from those, since coarsening reaches no farther
+// than a cell's children and their faces.  Launched level by level, each of the
+// small levels took 5.5-6 us of launch, load and FP64 chain latency.  Large
+// levels (kChainCells cells or more; over a whole batch) go alone: there the
+// FP64 pipe is the bound, and blocks that keep their SM's room through three
+// thinly filled stages cost more than the launches (24 uneven grids 291 -> 420
+// us with every level chained).  Halving is exact by the exponent, 12 FP64
+// instructions of 55 per 2D cell.  A 1024^2 hierarchy: 8 launches, 80 us;
+// 4 launches, 61 us (256^3: 552 -> 480 us).
+__host__ __device__ constexpr int setup_chain(int dim) { return dim == 3 ? 3 : 4; }
+constexpr long long kChainCells = 1LL << 16;
+
+template <int DIM> struct ChainTile {
+    static constexpr int X = DIM == 3 ? 8 : kBX, Y = 8, Z = DIM == 3 ? 4 : 1;
+    static constexpr int N = X * Y * Z;
+    static constexpr int F0 = (X + 1) * Y * Z, F1 = X * (Y + 1) * Z, F2 = DIM == 3 ? X * Y * (Z + 1) : 0;
+    double S[4][N];                  // a, b, d and l4
+    double2 G[F0 + F1 + F2];
+};
+static_assert(ChainTile<2>::N == kBX * kBY && ChainTile<3>::N == kBX * kBY, "one thread per cell of the first level");
+
+struct SetupChain {
+    SetupGeom g;                     // the first level's
+    SetupFine F;
+    SetupOut o[4];
+    int count;
+};
+
+// Blocks of a chain whose first level has n cells per axis.
+__host__ __device__ inline void chain_blocks(int dim, const int n[3], int *gx, int *gy, int *gz) {
+    const int x = dim == 3 ? 8 : kBX, z = dim == 3 ? 4 : 1;
+    *gx = (n[0] + x - 1) / x;
+    *gy = (n[1] + 7) / 8;
+    *gz = (n[2] + z - 1) / z;
 }
 
-template <int DIM>
-__global__ void __launch_bounds__(kBX * kBY) k_setup_coarse(SetupGeom cg, SetupFine F, SetupOut o,
-                                                          int *__restrict__ err) {
+// out(q): the outputs of the chain's level q.  ONE: a single level (T is not used).
+template <int DIM, bool AXI, bool ONE, typename Out>
+__device__ __forceinline__ void setup_chain_cells(const SetupGeom &cg, const SetupFine &F, Out out, int count, int *err,
+                                                  int bx, int by, int bz, ChainTile<DIM> *tile) {
+    using Tile = ChainTile<DIM>;
+    ChainTile<DIM> &T = *tile;
+    const int tid = threadIdx.x + kBX * threadIdx.y;
+    int n[3] = {cg.n[0], cg.n[1], cg.n[2]};
+    int X = Tile::X, Y = Tile::Y, Z = Tile::Z;       // the tile's cells at this level
+    double hf = F.h;
+    for (int s = 0; s < (ONE ? 1 : count); s++) {
+        const int x = tid % X, y = (tid / X) % Y, z = tid / (X * Y);
+        const int I = bx * X + x, J = by * Y + y, K = DIM == 3 ? bz * Z + z : 0;
+        const bool in = tid < X * Y * Z && I < n[0] && J < n[1] && K < n[2];
+        dq S{0.0, 0.0, 0.0, 0.0};
+        double l4 = 0.0;
+        double2 g[3][2];
+        if (in) {
+            if (ONE || s == 0) {
+                const int fn0 = F.n0, fn1 = F.n1;
+                coarse_values<DIM, AXI>(
+                    cg.r0, hf, I, J, K,
+                    [&](int i, int j, int k, dq &sf, double &w4) {
+                        const long long f = cell_id(i, j, k, fn0, fn1);
+                        if (!AXI && F.lam) {                 // the same branch in every thread
+                            const dq q4 = load_lam(F.lam, f);
+                            sf = dq{q4.a, q4.b, 0.0, q4.c};
+                            w4 = q4.d;
+                        } else {
+                            sf = ldgq(F.S + f);
+                            w4 = __ldg(F.l4 + f);
+                        }
+                    },
+                    [&](int a, int i, int j, int k) {
+                        const int m0 = fn0 + (a == 0), m1 = fn1 + (a == 1);
+                        return __ldg(F.G[a] + (i + (long long)m0 * (j + (long long)m1 * k)));
+                    },
+                    S, l4, g);
+            } else {
+                // the level below in shared memory: 2X x 2Y (x 2Z) cells of this tile
+                const int fX = 2 * X, fY = 2 * Y, fZ = DIM == 3 ? 2 * Z : 1;
+                const int i0 = bx * fX, j0 = by * fY, k0 = DIM == 3 ? bz * fZ : 0;
+                coarse_values<DIM, AXI>(
+                    cg.r0, hf, I, J, K,
+                    [&](int i, int j, int k, dq &sf, double &w4) {
+                        const int f = (i - i0) + fX * ((j - j0) + fY * (k - k0));
+                        sf = dq{T.S[0][f], T.S[1][f], 0.0, T.S[2][f]};
+                        w4 = T.S[3][f];
+                    },
+                    [&](int a, int i, int j, int k) {
+                        const int m0 = fX + (a == 0), m1 = fY + (a == 1);
+                        const int off = a == 0 ? 0 : a == 1 ? Tile::F0 : Tile::F0 + Tile::F1;
+                        return T.G[off + (i - i0) + m0 * ((j - j0) + m1 * (k - k0))];
+                    },
+                    S, l4, g);
+            }
+            long long fid[3][2];
+            face_ids(n, I, J, K, fid);
+            int own[3][2];
+            const int P[3] = {I, J, K};
+#pragma unroll
+            for (int a = 0; a < DIM; a++) {
+                own[a][0] = 1;
+                own[a][1] = P[a] + 1 == n[a];
+            }
+            finish_cell<DIM>(out(s), cell_id(I, J, K, n[0], n[1]), fid, own, g, S, l4, err);
+        }
+        if (ONE || s + 1 == count) break;
+        __syncthreads();                             // the level below is read
+        if (in) {
+            T.S[0][tid] = S.a;
+            T.S[1][tid] = S.b;
+            T.S[2][tid] = S.d;
+            T.S[3][tid] = l4;
+            const int p[3] = {x, y, z}, m[3] = {X, Y, Z}, P[3] = {I, J, K};
+#pragma unroll
+            for (int a = 0; a < DIM; a++) {
+                const int off = a == 0 ? 0 : a == 1 ? Tile::F0 : Tile::F0 + Tile::F1;
+                const int m0 = X + (a == 0), m1 = Y + (a == 1);
+                const int lo = off + x + m0 * (y + m1 * z);
+                T.G[lo] = g[a][0];
+                if (p[a] + 1 == m[a] || P[a] + 1 == n[a]) T.G[lo + (a == 0 ? 1 : a == 1 ? m0 : m0 * m1)] = g[a][1];
+            }
+        }
+        __syncthreads();
+        X /= 2;
+        Y /= 2;
+        if (DIM == 3) Z /= 2;
+        for (int a = 0; a < DIM; a++) n[a] /= 2;
+        hf *= 2.0;
+    }
+}
+
+template <int DIM, bool ONE>
+__global__ void __launch_bounds__(kBX * kBY) k_setup_coarse(const __grid_constant__ SetupChain C, int *__restrict__ err) {
     pdl_entry();
-    CMG_TILES(false, (cg.n[0] + kBX - 1) / kBX, (cg.n[1] + kBY - 1) / kBY, DIM == 3 ? cg.n[2] : 1,
-              (setup_coarse_block<DIM>(cg, F, o, err, bx, by, bz)));
+    ChainTile<DIM> *T = nullptr;
+    if constexpr (!ONE) {
+        __shared__ ChainTile<DIM> tile;
+        T = &tile;
+    }
+    auto out = [&](int q) -> const SetupOut & { return C.o[q]; };
+    if (DIM == 2 && C.g.axisym)
+        setup_chain_cells<DIM, true, ONE>(C.g, C.F, out, C.count, err, blockIdx.x, blockIdx.y, blockIdx.z, T);
+    else
+        setup_chain_cells<DIM, false, ONE>(C.g, C.F, out, C.count, err, blockIdx.x, blockIdx.y, blockIdx.z, T);
 }
 
 // FP32 copy of an FP64 array (the coarsest inverse of mixed precision).
