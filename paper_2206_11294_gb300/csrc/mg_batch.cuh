@@ -72,6 +72,8 @@ struct BState {                 // per-problem solve state, device side
 };
 
 constexpr int kBatchThreads = 256;
+// Rows per thread of the norm tiles: the other problems fill the SMs, so large tiles with few reductions.
+constexpr int kBatchNormRows = 4;
 constexpr int kBatchBlocksPerSM = 8;    // default persistent blocks per SM
 
 template <typename R> __device__ __forceinline__ const Level<R> &pick(const BLevel &L);
@@ -507,10 +509,9 @@ __global__ void __launch_bounds__(kBatchThreads) kb_norm(const BLevel *__restric
         if (!initial && !st[p].active) continue;
         const Level<double> L = B.d;
         int bx, by, bz;
-        const int rows = norm_rows(L.N);
-        block_coords(e.y, norm_gx(L.n0), norm_gy(L.n1, rows), bx, by, bz);
-        const double2 s = (red && !initial) ? norm_block<DIM, true>(L, rows, bx, by, bz)
-                                               : norm_block<DIM, false>(L, rows, bx, by, bz);
+        block_coords(e.y, norm_gx(L.n0), norm_gy(L.n1, kBatchNormRows), bx, by, bz);
+        const double2 s = (red && !initial) ? norm_block<DIM, true, kBatchNormRows>(L, bx, by, bz)
+                                               : norm_block<DIM, false, kBatchNormRows>(L, bx, by, bz);
         batch_finish(pr[p], st[p], e.y, s, initial, rtol, max_cycles, active_count);
     }
 }
@@ -530,13 +531,12 @@ __global__ void __launch_bounds__(kBatchThreads) kb_residual64(const BLevel *__r
         if (!initial && !st[p].active) continue;
         Level<double> L = B.d;
         int bx, by, bz;
-        const int rows = norm_rows(L.N);
-        block_coords(e.y, norm_gx(L.n0), norm_gy(L.n1, rows), bx, by, bz);
+        block_coords(e.y, norm_gx(L.n0), norm_gy(L.n1, kBatchNormRows), bx, by, bz);
         // defect correction: the initial call stores r0 = b - A x0 over b and sets delta = 0; later calls
         // form r0 - A delta
         if (!initial) L.x = B.delta;
-        const double2 s = residual64_to32_block<DIM>(L, B.f.b, B.f.bt, B.f.x, initial ? L.b : nullptr,
-                                                     initial ? B.delta : nullptr, red_start, rows, bx, by, bz);
+        const double2 s = residual64_to32_block<DIM, kBatchNormRows>(L, B.f.b, B.f.bt, B.f.x, initial ? L.b : nullptr,
+                                                     initial ? B.delta : nullptr, red_start, bx, by, bz);
         batch_finish(pr[p], st[p], e.y, s, initial, rtol, max_cycles, active_count);
     }
 }
@@ -904,7 +904,8 @@ mg_status mg_batch_create(int count, mg_handle *const *handles, mg_batch **out) 
         pr[p].kl = h->coarse_kl;
         pr[p].nc = h->nc;
         pr[p].coarse = base[p] + h->nlev - 1;
-        pr[p].npartial = h->npartial;
+        const LevelBuf &l0 = h->L[0];            // at most the handle's own count (norm_rows is smaller)
+        pr[p].npartial = norm_gx(l0.n[0]) * norm_gy(l0.n[1], kBatchNormRows) * l0.n[2];
         pr[p].x32_0 = h->L[0].x32;
     }
     std::vector<int2> tabs;
@@ -942,8 +943,7 @@ mg_status mg_batch_create(int count, mg_handle *const *handles, mg_batch **out) 
         const mg_handle *h = handles[p];
         const dim3 g0 = cell_grid(h->L[0], dim, h->L[0].n[0]);
         add_blocks(tn, base[p], (long long)g0.x * g0.y * g0.z);
-        const dim3 gn = norm_grid(h->L[0], dim);
-        add_blocks(tnorm, base[p], (long long)gn.x * gn.y * gn.z);
+        add_blocks(tnorm, base[p], pr[p].npartial);
         if (!h->coarse_factors)
             for (int r = 0; r * coarse_rows_per_block(h->nc) < h->nc; r++) tco.push_back(make_int2(p, r));
         add_blocks(tcell, base[p], (h->L[0].N + kBatchThreads - 1) / kBatchThreads);

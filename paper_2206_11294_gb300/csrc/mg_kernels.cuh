@@ -654,11 +654,8 @@ __device__ __forceinline__ void finish_norms(double2 *partial, int nblocks, unsi
         b += v.y;
     }
     block_sum2(a, b);
-    if (tid == 0) {
-        out[0] = sqrt(a);
-        out[1] = sqrt(b);
-        *ticket = 0u;
-    }
+    if (tid < 2) out[tid] = sqrt(tid ? b : a);      // the two roots at once
+    if (tid == 0) *ticket = 0u;
 }
 
 // Norm and FP64-residual tiles cover 64 columns and kBY x ROWS rows of one
@@ -666,12 +663,13 @@ __device__ __forceinline__ void finish_norms(double2 *partial, int nblocks, unsi
 // (norm_rows) trades the block's reduction, 24 warp-wide FP64 additions per
 // tile, against filling the chip: 4 rows make 512 tiles of a 1024^2 grid, 3.4
 // per SM, and the SMs with 4 set the time (the FP64 pipe of an average SM was
-// busy 61% of it); 2 rows make 6.7 per SM.  On small grids 1 row spreads the
-// cells over more SMs (64^2: 8 tiles instead of 2, 15.4 -> 8.3 us).  Each thread
+// busy 61% of it); 2 rows make 6.7 per SM.  On smaller grids 1 row spreads the
+// cells over more SMs (64^2: 8 tiles instead of 2, 15.4 -> 8.1 us; the residual
+// of 256 x 512 cells: 256 tiles instead of 64, 22.7 -> 12.3 us).  Each thread
 // accumulates its cells' squares with FMAs; a persistent block reduces once.
 // (The batched kernels reduce per tile.)
 constexpr int kNormCols = 64;
-__host__ __device__ __forceinline__ int norm_rows(long long N) { return N >= (1LL << 22) ? 4 : N >= (1LL << 17) ? 2 : 1; }
+__host__ __device__ __forceinline__ int norm_rows(long long N) { return N >= (1LL << 22) ? 4 : N >= (1LL << 19) ? 2 : 1; }
 __host__ __device__ __forceinline__ int norm_gx(int n0) { return (n0 + kNormCols - 1) / kNormCols; }
 __host__ __device__ __forceinline__ int norm_gy(int n1, int rows) { return (n1 + kBY * rows - 1) / (kBY * rows); }
 
@@ -716,12 +714,10 @@ __device__ __forceinline__ void norm_tile(const Level<double> &L, int bx, int by
     }
 }
 
-template <int DIM, bool RED>
-__device__ __forceinline__ double2 norm_block(const Level<double> &L, int rows, int bx, int by, int bz) {
+template <int DIM, bool RED, int ROWS>
+__device__ __forceinline__ double2 norm_block(const Level<double> &L, int bx, int by, int bz) {
     double zT2 = 0.0, zp2 = 0.0;
-    if (rows == 1) norm_tile<DIM, RED, 1>(L, bx, by, bz, zT2, zp2);
-    else if (rows == 2) norm_tile<DIM, RED, 2>(L, bx, by, bz, zT2, zp2);
-    else norm_tile<DIM, RED, 4>(L, bx, by, bz, zT2, zp2);
+    norm_tile<DIM, RED, ROWS>(L, bx, by, bz, zT2, zp2);
     block_sum2(zT2, zp2);
     return make_double2(zT2, zp2);
 }
@@ -791,15 +787,13 @@ __device__ __forceinline__ void residual64_to32_tile(const Level<double> &L, flo
     }
 }
 
-template <int DIM>
+template <int DIM, int ROWS>
 __device__ __forceinline__ double2 residual64_to32_block(const Level<double> &L, float2 *__restrict__ b32,
                                                          float2 *__restrict__ bt32, float2 *__restrict__ e32,
                                                          double2 *__restrict__ r_out, double2 *__restrict__ r_out2,
-                                                         int red_start, int rows, int bx, int by, int bz) {
+                                                         int red_start, int bx, int by, int bz) {
     double zT2 = 0.0, zp2 = 0.0;
-    if (rows == 1) residual64_to32_tile<DIM, 1>(L, b32, bt32, e32, r_out, r_out2, red_start, bx, by, bz, zT2, zp2);
-    else if (rows == 2) residual64_to32_tile<DIM, 2>(L, b32, bt32, e32, r_out, r_out2, red_start, bx, by, bz, zT2, zp2);
-    else residual64_to32_tile<DIM, 4>(L, b32, bt32, e32, r_out, r_out2, red_start, bx, by, bz, zT2, zp2);
+    residual64_to32_tile<DIM, ROWS>(L, b32, bt32, e32, r_out, r_out2, red_start, bx, by, bz, zT2, zp2);
     block_sum2(zT2, zp2);
     return make_double2(zT2, zp2);
 }
