@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(kBatchThreads) kb_setup_coarse(const BSetupLev
     }
 }
 
-// Dense coarsest matrices of all problems (zeroed first by kb_zero_coarse).
+// Dense coarsest matrices of all problems.
 struct BCoarse {
     int n[3];
     const double2 *G0, *G1, *G2;
@@ -301,46 +301,11 @@ __global__ void kb_transpose_big(const BCoarse *__restrict__ co, const int *__re
     }
 }
 
-__global__ void __launch_bounds__(kBatchThreads) kb_zero_coarse(const BCoarse *__restrict__ co, int count) {
-    for (int p = blockIdx.y; p < count; p += gridDim.y) {
-        const long long m = (long long)co[p].nc * co[p].nc;
-        for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < m; q += (long long)gridDim.x * blockDim.x)
-            co[p].M[q] = 0.0;
-    }
-}
-
 template <int DIM>
 __global__ void __launch_bounds__(kBatchThreads) kb_coarse_assemble(const BCoarse *__restrict__ co, int count) {
     for (int p = blockIdx.y; p < count; p += gridDim.y) {
         const BCoarse &C = co[p];
-        const long long N = (long long)C.n[0] * C.n[1] * C.n[2];
-        const long long n = 2 * N;
-        for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
-            const int i = (int)(c % C.n[0]), j = (int)((c / C.n[0]) % C.n[1]), k = (int)(c / ((long long)C.n[0] * C.n[1]));
-            const dq d = C.D[c];
-            double *M = C.M;
-            M[(2 * c) * n + 2 * c] = d.a;
-            M[(2 * c) * n + 2 * c + 1] = d.b;
-            M[(2 * c + 1) * n + 2 * c] = d.c;
-            M[(2 * c + 1) * n + 2 * c + 1] = d.d;
-            const long long f0 = (long long)i + (long long)(C.n[0] + 1) * ((long long)j + (long long)C.n[1] * k);
-            const long long f1 = (long long)i + (long long)C.n[0] * ((long long)j + (long long)(C.n[1] + 1) * k);
-            const double w4 = C.l4[c];
-            auto put = [&](long long nb, double2 g) {
-                M[(2 * c) * n + 2 * nb] = g.x;
-                M[(2 * c + 1) * n + 2 * nb] = w4 * g.x;
-                M[(2 * c + 1) * n + 2 * nb + 1] = g.y;
-            };
-            if (i > 0) put(c - 1, C.G0[f0]);
-            if (i < C.n[0] - 1) put(c + 1, C.G0[f0 + 1]);
-            if (j > 0) put(c - C.n[0], C.G1[f1]);
-            if (j < C.n[1] - 1) put(c + C.n[0], C.G1[f1 + C.n[0]]);
-            if (DIM == 3) {
-                const long long pl = (long long)C.n[0] * C.n[1];
-                if (k > 0) put(c - pl, C.G2[c]);
-                if (k < C.n[2] - 1) put(c + pl, C.G2[c + pl]);
-            }
-        }
+        coarse_rows<DIM>(C.n, C.G0, C.G1, C.G2, C.D, C.l4, C.M, blockIdx.x, gridDim.x);
     }
 }
 
@@ -1284,10 +1249,9 @@ mg_status mg_batch_set_coeffs(mg_batch *b, const double *const *lambda, const do
         b->launches++;
     }
     const unsigned gy = (unsigned)std::min(b->count, 65535);
-    kb_zero_coarse<<<dim3(16, gy), kBatchThreads, 0, s>>>(b->co, b->count);
-    if (dim == 2) kb_coarse_assemble<2><<<dim3(4, gy), kBatchThreads, 0, s>>>(b->co, b->count);
-    else kb_coarse_assemble<3><<<dim3(4, gy), kBatchThreads, 0, s>>>(b->co, b->count);
-    b->launches += 2;
+    if (dim == 2) kb_coarse_assemble<2><<<dim3(16, gy), kBatchThreads, 0, s>>>(b->co, b->count);
+    else kb_coarse_assemble<3><<<dim3(16, gy), kBatchThreads, 0, s>>>(b->co, b->count);
+    b->launches++;
     if (b->n_inv_smem > 0) {
         CK(launch_clusters(kb_coarse_invert, s, 1, b->n_inv_smem, kGjThreads, gj_smem(b->max_nc_small),
                            (const BProb *)b->pr, (const int *)b->inv_ids));

@@ -909,8 +909,9 @@ void enqueue_vcycle(const mg_handle *h, cudaStream_t s, int l, int type, bool re
 }
 
 // after_sweep: x has just come out of a red-black sweep (red cells only).
+// host: page-locked host memory for the norms, or NULL.
 template <int DIM>
-void enqueue_norm(const mg_handle *h, cudaStream_t s, bool after_sweep) {
+void enqueue_norm(const mg_handle *h, cudaStream_t s, bool after_sweep, double *host) {
     const LevelBuf &f = h->L[0];
     const dim3 ng = norm_grid(f, DIM);
     with_norm_rows(f.N, [&](auto rows) {
@@ -918,9 +919,9 @@ void enqueue_norm(const mg_handle *h, cudaStream_t s, bool after_sweep) {
         auto run = [&](auto tile, auto wave_of) {
             if (h->persistent)
                 launch_k(h, wave_of, wave((const void *)wave_of, tiles_of(ng)), kBlock, 0, s, 0, view<double>(f), h->partial,
-                         h->ticket, h->norms_d);
+                         h->ticket, h->norms_d, host);
             else
-                launch_k(h, tile, ng, kBlock, 0, s, 0, view<double>(f), h->partial, h->ticket, h->norms_d);
+                launch_k(h, tile, ng, kBlock, 0, s, 0, view<double>(f), h->partial, h->ticket, h->norms_d, host);
         };
         if (after_sweep) run(k_norm_partials<DIM, true, false, R>, k_norm_partials<DIM, true, true, R>);
         else run(k_norm_partials<DIM, false, false, R>, k_norm_partials<DIM, false, true, R>);
@@ -939,8 +940,9 @@ double2 *mixed_delta(const mg_handle *h) { return reinterpret_cast<double2 *>(h-
 // otherwise r = r0 - A delta.  Forming b - A x every step instead subtracts
 // terms of the size of b (lambda_T ~ 1e16 at these units) and leaves a
 // rounding floor that a good initial guess puts near the tolerance.
+// host: as for enqueue_norm.
 template <int DIM>
-void enqueue_residual_to32(const mg_handle *h, cudaStream_t s, bool initial = false) {
+void enqueue_residual_to32(const mg_handle *h, cudaStream_t s, bool initial, double *host) {
     const LevelBuf &f = h->L[0];
     const dim3 ng = norm_grid(f, DIM);
     Level<double> v = view<double>(f);
@@ -952,7 +954,7 @@ void enqueue_residual_to32(const mg_handle *h, cudaStream_t s, bool initial = fa
         constexpr int R = decltype(rows)::value;
         auto run = [&](auto kern, dim3 grid) {
             launch_k(h, kern, grid, kBlock, 0, s, 0, v, f.b32, f.bt32, f.x32, r_out, r_out2, red_start(h), h->partial,
-                     h->ticket, h->norms_d);
+                     h->ticket, h->norms_d, host);
         };
         if (h->persistent)
             run(k_residual64_to32<DIM, true, R>, dim3(wave((const void *)k_residual64_to32<DIM, true, R>, tiles_of(ng))));
@@ -987,12 +989,11 @@ void warm_waves() {
     of(std::integral_constant<int, 4>());
 }
 
-// FP64: one V-cycle, then the stopping norm, copied to pinned host memory.
+// FP64: one V-cycle, then the stopping norm, also into pinned host memory.
 template <int DIM>
 void enqueue_cycle64(const mg_handle *h, cudaStream_t s) {
     enqueue_vcycle<double, DIM>(h, s, 0, h->opt.cycle);
-    enqueue_norm<DIM>(h, s, h->opt.nu2 > 0 && red_only_after_sweeps(h));
-    cudaMemcpyAsync(h->norms_h, h->norms_d, 2 * sizeof(double), cudaMemcpyDeviceToHost, s);
+    enqueue_norm<DIM>(h, s, h->opt.nu2 > 0 && red_only_after_sweeps(h), h->norms_h);
 }
 
 // Mixed: FP32 V-cycles on the correction, FP64 update, FP64 residual + norm.
@@ -1003,8 +1004,7 @@ void enqueue_step32(const mg_handle *h, cudaStream_t s) {
     const LevelBuf &f = h->L[0];
     launch_k(h, k_add_correction, lin_blocks(f.N), 256, 0, s, 0, mixed_delta(h), f.x32, f.N);
     counted(h);
-    enqueue_residual_to32<DIM>(h, s);
-    cudaMemcpyAsync(h->norms_h, h->norms_d, 2 * sizeof(double), cudaMemcpyDeviceToHost, s);
+    enqueue_residual_to32<DIM>(h, s, false, h->norms_h);
 }
 
 template <typename F>
@@ -1065,6 +1065,16 @@ mg_status x_in(mg_handle *h, const double *x, int on_device) {
     return MG_OK;
 }
 
+// A kernel of this handle may use p: memory of its own device, or managed.
+bool local_device(const mg_handle *h, const void *p) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == h->device);
+}
+
 mg_status x_out(mg_handle *h, double *x, int on_device) {
     const long long N = h->L[0].N;
     CK(cudaMemcpyAsync(x, h->L[0].x, sizeof(double2) * N, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
@@ -1072,22 +1082,52 @@ mg_status x_out(mg_handle *h, double *x, int on_device) {
     return MG_OK;
 }
 
+// xin (may be NULL): also copied to x.  clear (may be NULL): an int set to 0.
 template <int DIM>
-void enqueue_prep(mg_handle *h, const double2 *rhs, cudaStream_t s) {
+void enqueue_prep(mg_handle *h, const double2 *rhs, cudaStream_t s, const double2 *xin = nullptr, int *clear = nullptr) {
     const LevelBuf &f = h->L[0];
-    launch_k(h, k_prep_rhs<DIM>, cell_grid(f, DIM, f.n[0]), kBlock, 0, s, 0, view<double>(f), rhs, bc_vals(h->grid),
-                                                                          h->grid.axisym, h->grid.r0, h->grid.h);
+    launch_k(h, k_prep_rhs<DIM>, cell_grid(f, DIM, f.n[0]), kBlock, 0, s, 0, view<double>(f), rhs, xin, bc_vals(h->grid),
+             h->grid.axisym, h->grid.r0, h->grid.h, clear);
     counted(h);
 }
 
-mg_status prep(mg_handle *h, const double *rhs, const double *x, int on_device) {
-    const double2 *r = nullptr;
+// The right-hand side and the initial guess.  A guess in this device's memory is
+// read by the kernel itself: the copy would be one more hop between copy engine
+// and kernels on a small grid's critical path, and two more passes on a large one.
+mg_status prep(mg_handle *h, const double *rhs, const double *x, int on_device, int *clear = nullptr) {
+    const double2 *r = nullptr, *xin = nullptr;
     mg_status st = pair_in(h, rhs, on_device, &r);
     if (st) return st;
-    if ((st = x_in(h, x, on_device))) return st;
-    if (h->grid.dim == 2) enqueue_prep<2>(h, r, h->stream);
-    else enqueue_prep<3>(h, r, h->stream);
+    if (on_device && aligned16(x) && local_device(h, x)) xin = reinterpret_cast<const double2 *>(x);
+    else if ((st = x_in(h, x, on_device))) return st;
+    if (h->grid.dim == 2) enqueue_prep<2>(h, r, h->stream, xin, clear);
+    else enqueue_prep<3>(h, r, h->stream, xin, clear);
     CK(cudaGetLastError());
+    return MG_OK;
+}
+
+// The end of a solve: x (plus delta: mixed precision) into the caller's array,
+// and the error flags into errh.  One kernel where x is this device's memory.
+mg_status solve_out(mg_handle *h, double *x, int on_device, const double2 *delta) {
+    const LevelBuf &f = h->L[0];
+    CK(cudaStreamWaitEvent(h->stream, h->ev_inv, 0));
+    if (!h->x_stale && on_device && local_device(h, x)) {
+        launch_k(h, delta ? k_solution_out<true> : k_solution_out<false>, lin_blocks(f.N), 256, 0, h->stream, 0, f.x, delta,
+                 reinterpret_cast<double2 *>(x), f.N, h->err_d, h->errh);
+        counted(h);
+        CK(cudaGetLastError());
+        return MG_OK;
+    }
+    if (!h->x_stale) {
+        if (delta) {
+            launch_k(h, k_add_pairs, lin_blocks(f.N), 256, 0, h->stream, 0, f.x, delta, f.N);
+            counted(h);
+            CK(cudaGetLastError());
+        }
+        const mg_status st = x_out(h, x, on_device);
+        if (st) return st;
+    }
+    CK(cudaMemcpyAsync(h->errh, h->err_d, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     return MG_OK;
 }
 
@@ -1304,8 +1344,7 @@ template <int DIM>
 void enqueue_setup_levels(mg_handle *h, cudaStream_t s, const SetupGeom &gm, const SetupIn &in) {
     const bool mixed = h->opt.precision == MG_MIXED;
     const LevelBuf &f = h->L[0];
-    cudaMemsetAsync(h->err_d, 0, sizeof(int), s);
-    if (f.jflag) cudaMemsetAsync(h->err_d + 2, 0, sizeof(int), s);
+    cudaMemsetAsync(h->err_d, 0, 3 * sizeof(int), s);      // (a solve clears [1] for itself)
     SetupOut fine = setup_out(f, mixed);
     if (!gm.axisym) fine.S = nullptr;        // level 1 reads lambda
     launch_k(h, k_setup_fine<DIM>, cell_grid(f, DIM, f.n[0]), kBlock, 0, s, 0, gm, in, fine, h->err_d);
@@ -1334,9 +1373,15 @@ void enqueue_setup_levels(mg_handle *h, cudaStream_t s, const SetupGeom &gm, con
         l += C.count;
     }
     const LevelBuf &c = h->L[h->nlev - 1];
-    cudaMemsetAsync(h->Mtmp, 0, sizeof(double) * h->nc * h->nc, s);
-    launch_k(h, k_coarse_assemble<DIM>, lin_blocks(c.N), 256, 0, s, 0, c.n[0], c.n[1], c.n[2], c.G[0], c.G[1],
-             DIM == 3 ? c.G[2] : nullptr, c.D, c.l4, h->Mtmp);
+    CoarseRows rows;
+    for (int a = 0; a < 3; a++) {
+        rows.n[a] = c.n[a];
+        rows.G[a] = a < DIM ? c.G[a] : nullptr;
+    }
+    rows.D = c.D;
+    rows.l4 = c.l4;
+    rows.M = h->Mtmp;
+    launch_k(h, k_coarse_assemble<DIM>, lin_blocks(32 * c.N), 256, 0, s, 0, rows, h->err_d, h->errh);
     counted(h);
 }
 
@@ -1428,10 +1473,8 @@ mg_status setup_hierarchy(mg_handle *h, const double *lam, const double *const f
     CK(cudaGraphLaunch(h->gcoarse, h->aux));
     h->enq += h->coarse_kernels;
     CK(cudaEventRecord(h->ev_inv, h->aux));
-    // flags 1 and 2 come from the level kernels, which precede this copy on
-    // the stream (the inverse on the private stream keeps running)
-    CK(cudaMemcpyAsync(h->errh, h->err_d, sizeof(int), cudaMemcpyDeviceToHost, s));
-    if (f.jflag) CK(cudaMemcpyAsync(h->errh + 2, h->err_d + 2, sizeof(int), cudaMemcpyDeviceToHost, s));
+    // flags 1 and 2 come from the level kernels; the graph's last kernel left
+    // them in errh (the inverse on the private stream keeps running)
     CK(cudaStreamSynchronize(s));
     h->jcells = f.jflag ? h->errh[2] : 0;
     const int err = *h->errh;
@@ -1442,8 +1485,8 @@ mg_status setup_hierarchy(mg_handle *h, const double *lam, const double *const f
 
 // ---------------------------------------------------------------- solves
 // The stop-test loop of both precisions.  `initial` enqueues the initial
-// norms (into norms_d); g is the graph of one iteration, which copies its
-// norms to norms_h[0..1]; an iteration is `per_iter` V-cycles.  The first
+// norms (into norms_h[2..3]); g is the graph of one iteration, which leaves
+// its norms in norms_h[0..1]; an iteration is `per_iter` V-cycles.  The first
 // iteration is launched before the initial norms are read, so one host wait
 // serves both: it only changes the handle's own x, which mg_solve does not
 // copy back (x_stale) when the initial state already meets the stop test.
@@ -1451,7 +1494,6 @@ template <typename FInit>
 mg_status run_loop(mg_handle *h, mg_stats *st, cudaGraphExec_t g, long long kernels, int per_iter, FInit &&initial) {
     double n0[2], nk[2];
     initial(h->stream);
-    CK(cudaMemcpyAsync(h->norms_h + 2, h->norms_d, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     const bool ahead = h->opt.max_cycles >= 1 && h->opt.rtol < 1.0;
     if (ahead) {
         CK(cudaGraphLaunch(g, h->stream));
@@ -1500,7 +1542,7 @@ mg_status solve64(mg_handle *h, mg_stats *st) {
         if (e) return e;
     }
     return run_loop(h, st, h->g64, h->graph_kernels64, 1,
-                    [&](cudaStream_t s) { enqueue_norm<DIM>(h, s, false); });
+                    [&](cudaStream_t s) { enqueue_norm<DIM>(h, s, false, h->norms_h + 2); });
 }
 
 template <int DIM>
@@ -1510,17 +1552,11 @@ mg_status solve_mixed(mg_handle *h, mg_stats *st) {
         if (e) return e;
     }
     // r0 = b - A x0 once, delta from A delta = r0 by FP32 cycles with the
-    // FP64 residual r0 - A delta after each outer step, then x = x0 + delta
+    // FP64 residual r0 - A delta after each outer step; solve_out adds x0
     const LevelBuf &f = h->L[0];
     const mg_status e = run_loop(h, st, h->g32, h->graph_kernels32, h->opt.inner_cycles,
-                                 [&](cudaStream_t s) { enqueue_residual_to32<DIM>(h, s, true); });
-    if (e) return e;
-    if (!h->x_stale) {
-        launch_k(h, k_add_pairs, lin_blocks(f.N), 256, 0, h->stream, 0, f.x, mixed_delta(h), f.N);
-        counted(h);
-        CK(cudaGetLastError());
-    }
-    return MG_OK;
+                                 [&](cudaStream_t s) { enqueue_residual_to32<DIM>(h, s, true, h->norms_h + 2); });
+    return e;
 }
 
 // opt.max_cycles FP64 cycles from x = 0 with no stopping norms and no host wait: a fixed linear map of rhs, the
@@ -1553,7 +1589,7 @@ mg_status enqueue_correction(mg_handle *h, cudaStream_t s, const double2 *rhs) {
     CK(cudaMemsetAsync(f.x, 0, sizeof(double2) * f.N, s));
     enqueue_prep<DIM>(h, rhs, s);
     if (h->opt.precision == MG_MIXED) {
-        enqueue_residual_to32<DIM>(h, s, true);        // x = 0: b32 = b, bt32 = Dinv b, e32 = 0
+        enqueue_residual_to32<DIM>(h, s, true, nullptr);        // x = 0: b32 = b, bt32 = Dinv b, e32 = 0
         for (int q = 0; q < h->opt.max_cycles; q++)
         enqueue_vcycle<float, DIM>(h, s, 0, h->opt.cycle, q == 0 && red_start(h));
         launch_k(h, k_add_correction, lin_blocks(f.N), 256, 0, s, 0, f.x, f.x32, f.N);
@@ -1587,8 +1623,8 @@ mg_status capture_async(mg_handle *h) {
     const cudaGraphNode_t *deps = nullptr;
     size_t ndeps = 0;
     cudaStreamCaptureStatus cs;
-    if (mixed) enqueue_residual_to32<DIM>(h, h->cap, true);
-    else enqueue_norm<DIM>(h, h->cap, false);
+    if (mixed) enqueue_residual_to32<DIM>(h, h->cap, true, nullptr);
+    else enqueue_norm<DIM>(h, h->cap, false, nullptr);
     long long pre = h->enq - before;
     e = cudaStreamGetCaptureInfo(h->cap, &cs, nullptr, &cg, nullptr, nullptr, nullptr);
     // the condition starts at 0 on every launch (the loop runs only if the
@@ -1620,10 +1656,10 @@ mg_status capture_async(mg_handle *h) {
             const LevelBuf &f = h->L[0];
             launch_k(h, k_add_correction, lin_blocks(f.N), 256, 0, h->cap2, 0, mixed_delta(h), f.x32, f.N);
             counted(h);
-            enqueue_residual_to32<DIM>(h, h->cap2);
+            enqueue_residual_to32<DIM>(h, h->cap2, false, nullptr);
         } else {
             enqueue_vcycle<double, DIM>(h, h->cap2, 0, h->opt.cycle);
-            enqueue_norm<DIM>(h, h->cap2, h->opt.nu2 > 0 && red_only_after_sweeps(h));
+            enqueue_norm<DIM>(h, h->cap2, h->opt.nu2 > 0 && red_only_after_sweeps(h), nullptr);
         }
         launch_k(h, k_async_stop, 1, 32, 0, h->cap2, 0, h->norms_d, h->astat_d, h->opt.max_cycles, h->opt.rtol, cond, 0);
         counted(h);
@@ -1978,9 +2014,8 @@ mg_status mg_solve(mg_handle *h, const double *rhs, double *x, int on_device, mg
     if (st) return st;
     if (!rhs || !x) return fail(MG_ERR_INVALID_ARG, "rhs and x must not be NULL");
     DeviceGuard dg(h->device);
-    CK(cudaMemsetAsync(h->err_d + 1, 0, sizeof(int), h->stream));
     h->x_stale = false;
-    if ((st = prep(h, rhs, x, on_device))) return st;
+    if ((st = prep(h, rhs, x, on_device, h->err_d + 1))) return st;
     mg_stats s;
     std::memset(&s, 0, sizeof(s));
     s.levels = h->nlev;
@@ -1989,9 +2024,7 @@ mg_status mg_solve(mg_handle *h, const double *rhs, double *x, int on_device, mg
     if (h->opt.precision == MG_FP64) st = dim == 2 ? solve64<2>(h, &s) : solve64<3>(h, &s);
     else st = dim == 2 ? solve_mixed<2>(h, &s) : solve_mixed<3>(h, &s);
     if (st) return st;
-    if (!h->x_stale && (st = x_out(h, x, on_device))) return st;
-    CK(cudaStreamWaitEvent(h->stream, h->ev_inv, 0));
-    CK(cudaMemcpyAsync(h->errh, h->err_d, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    if ((st = solve_out(h, x, on_device, h->opt.precision == MG_FP64 ? nullptr : mixed_delta(h)))) return st;
     CK(cudaStreamSynchronize(h->stream));
     if (h->errh[0] & 4) return fail(MG_ERR_INVALID_COEFF, "the coarsest-level matrix is singular");
     if (h->errh[1] & kErrAsyncTimeout) return fail(MG_ERR_TIMEOUT, "an asynchronous copy did not complete in time");
@@ -2014,14 +2047,12 @@ mg_status mg_solve_async(mg_handle *h, const double *rhs, double *x, void *event
         st = h->grid.dim == 2 ? capture_async<2>(h) : capture_async<3>(h);
         if (st) return st;
     }
-    CK(cudaMemsetAsync(h->err_d + 1, 0, sizeof(int), h->stream));
     h->x_stale = false;
-    if ((st = prep(h, rhs, x, 1))) return st;
+    if ((st = prep(h, rhs, x, 1, h->err_d + 1))) return st;
     CK(cudaStreamWaitEvent(h->stream, h->ev_inv, 0));
     CK(cudaEventRecord(h->ev_a0, h->stream));
     CK(cudaGraphLaunch(h->gasync, h->stream));
-    if ((st = x_out(h, x, 1))) return st;
-    CK(cudaMemcpyAsync(h->errh, h->err_d, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    if ((st = solve_out(h, x, 1, nullptr))) return st;       // (the graph has added delta)
     CK(cudaEventRecord(h->ev_a1, h->stream));
     if (event) CK(cudaEventRecord(reinterpret_cast<cudaEvent_t>(event), h->stream));
     CK(cudaEventRecord(h->ev_last, h->stream));
@@ -2308,10 +2339,9 @@ mg_status mg_residual_norms(mg_handle *h, const double *rhs, const double *x, in
     if (!rhs || !x || !out) return fail(MG_ERR_INVALID_ARG, "bad arguments to mg_residual_norms");
     DeviceGuard dg(h->device);
     if ((st = prep(h, rhs, x, on_device))) return st;
-    if (h->grid.dim == 2) enqueue_norm<2>(h, h->stream, false);
-    else enqueue_norm<3>(h, h->stream, false);
+    if (h->grid.dim == 2) enqueue_norm<2>(h, h->stream, false, h->norms_h);
+    else enqueue_norm<3>(h, h->stream, false, h->norms_h);
     CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(h->norms_h, h->norms_d, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     return sync_norms(h, out);
 }
 

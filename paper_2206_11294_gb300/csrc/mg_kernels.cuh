@@ -635,8 +635,15 @@ __device__ __forceinline__ void block_sum2(double &a, double &b) {
 
 // Last-block completion: after a block stored its partial, the block that
 // draws the final ticket sums all partials in index order (deterministic),
-// writes sqrt of the two sums to out and re-arms the ticket counter.
-__device__ __forceinline__ void finish_norms(double2 *partial, int nblocks, unsigned int *ticket, double *out) {
+// writes sqrt of the two sums to out and re-arms the ticket counter.  host (may
+// be NULL): page-locked host memory that gets them too, for the stop test on
+// the host.  Two stores over the link in place of a copy node behind the kernel
+// spare the hop to the copy engine, about 5 us on every cycle's critical path
+// (with k_solution_out and prep's copy of the guess: a set-up and solve of 64^2
+// 184 -> 157 us, of 1024^2 in mixed precision 817 -> 773, twenty steps of a
+// 256 x 512 axisymmetric one 2066 -> 1884).
+__device__ __forceinline__ void finish_norms(double2 *partial, int nblocks, unsigned int *ticket, double *out,
+                                             double *host) {
     __shared__ bool last;
     const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
     const int nthr = blockDim.x * blockDim.y * blockDim.z;
@@ -654,7 +661,11 @@ __device__ __forceinline__ void finish_norms(double2 *partial, int nblocks, unsi
         b += v.y;
     }
     block_sum2(a, b);
-    if (tid < 2) out[tid] = sqrt(tid ? b : a);      // the two roots at once
+    if (tid < 2) {                                  // the two roots at once
+        const double v = sqrt(tid ? b : a);
+        out[tid] = v;
+        if (host) host[tid] = v;
+    }
     if (tid == 0) *ticket = 0u;
 }
 
@@ -724,7 +735,8 @@ __device__ __forceinline__ double2 norm_block(const Level<double> &L, int bx, in
 
 template <int DIM, bool RED, bool P, int ROWS>
 __global__ void __launch_bounds__(kBX * kBY) k_norm_partials(Level<double> L, double2 *__restrict__ partial,
-                                                           unsigned int *__restrict__ ticket, double *__restrict__ out) {
+                                                           unsigned int *__restrict__ ticket, double *__restrict__ out,
+                                                           double *__restrict__ host) {
     pdl_entry();
     double zT2 = 0.0, zp2 = 0.0;     // a block's tiles accumulate, then one reduction
     CMG_TILES(P, norm_gx(L.n0), norm_gy(L.n1, ROWS), DIM == 3 ? L.n2 : 1,
@@ -732,7 +744,7 @@ __global__ void __launch_bounds__(kBX * kBY) k_norm_partials(Level<double> L, do
     block_sum2(zT2, zp2);
     const int blk = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
     if (threadIdx.x == 0 && threadIdx.y == 0) partial[blk] = make_double2(zT2, zp2);
-    finish_norms(partial, gridDim.x * gridDim.y * gridDim.z, ticket, out);
+    finish_norms(partial, gridDim.x * gridDim.y * gridDim.z, ticket, out, host);
 }
 
 // FP64 residual of the finest level for mixed precision: r = b - A x is
@@ -805,7 +817,7 @@ __global__ void __launch_bounds__(kBX * kBY) k_residual64_to32(Level<double> L, 
                                                              double2 *__restrict__ r_out2, int red_start,
                                                              double2 *__restrict__ partial,
                                                              unsigned int *__restrict__ ticket,
-                                                             double *__restrict__ out) {
+                                                             double *__restrict__ out, double *__restrict__ host) {
     pdl_entry();
     double zT2 = 0.0, zp2 = 0.0;
     CMG_TILES(P, norm_gx(L.n0), norm_gy(L.n1, ROWS), DIM == 3 ? L.n2 : 1,
@@ -813,7 +825,7 @@ __global__ void __launch_bounds__(kBX * kBY) k_residual64_to32(Level<double> L, 
     block_sum2(zT2, zp2);
     const int blk = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
     if (threadIdx.x == 0 && threadIdx.y == 0) partial[blk] = make_double2(zT2, zp2);
-    finish_norms(partial, gridDim.x * gridDim.y * gridDim.z, ticket, out);
+    finish_norms(partial, gridDim.x * gridDim.y * gridDim.z, ticket, out, host);
 }
 
 // x += delta: the solution from the initial guess and the accumulated correction
@@ -822,6 +834,27 @@ __global__ void k_add_pairs(double2 *__restrict__ x, const double2 *__restrict__
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
         const double2 a = x[c], d = delta[c];
         x[c] = make_double2(a.x + d.x, a.y + d.y);
+    }
+}
+
+// The end of a solve in one launch, in place of an addition and two copies one
+// behind the other: x += delta (DELTA: mixed precision), the solution into the
+// caller's array, and the error flags into page-locked host memory.  Bound by
+// memory on large grids, by the hops between kernels and copy engine on small
+// ones (5 to 7 us each).
+template <bool DELTA>
+__global__ void k_solution_out(double2 *__restrict__ x, const double2 *__restrict__ delta, double2 *__restrict__ out,
+                               long long N, const int *__restrict__ err, int *__restrict__ err_host) {
+    pdl_entry();
+    if (blockIdx.x == 0 && threadIdx.x < 2) err_host[threadIdx.x] = err[threadIdx.x];
+    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
+        double2 a = x[c];
+        if (DELTA) {
+            const double2 d = delta[c];
+            a = make_double2(a.x + d.x, a.y + d.y);
+            x[c] = a;
+        }
+        out[c] = a;
     }
 }
 
@@ -913,11 +946,13 @@ __device__ __forceinline__ void prep_rhs_block(const Level<double> &L, const dou
 
 template <int DIM>
 __global__ void __launch_bounds__(kBX * kBY) k_prep_rhs(const __grid_constant__ Level<double> L,
-                                                      const double2 *__restrict__ rhs, const __grid_constant__ BcVals bv,
-                                                      int axisym, double r0, double h) {
+                                                      const double2 *__restrict__ rhs, const double2 *__restrict__ xin,
+                                                      const __grid_constant__ BcVals bv, int axisym, double r0, double h,
+                                                      int *__restrict__ clear) {
     pdl_entry();
+    if (clear && (blockIdx.x | blockIdx.y | blockIdx.z | threadIdx.x | threadIdx.y) == 0) *clear = 0;
     CMG_TILES(false, (L.n0 + kBX - 1) / kBX, (L.n1 + kBY - 1) / kBY, DIM == 3 ? L.n2 : 1,
-              (prep_rhs_block<DIM>(L, rhs, nullptr, bv, axisym, r0, h, bx, by, bz)));
+              (prep_rhs_block<DIM>(L, rhs, xin, bv, axisym, r0, h, bx, by, bz)));
 }
 
 // y = L(x) (Eqs. 27-28): offdiag + boundary data + D x is s_i times the rows.
@@ -1388,41 +1423,63 @@ __global__ void k_to_f32(const double *__restrict__ in, float *__restrict__ out,
         out[q] = (float)in[q];
 }
 
-// Dense matrix of the coarsest level (M zeroed beforehand): rows 2c, 2c+1
-// hold D_c on the diagonal block; on a neighbour, G^T in the T-row, G^p and
-// l4 G^T in the p-row.
+// Dense matrix of the coarsest level: rows 2c, 2c+1 hold D_c on the diagonal
+// block; on a neighbour, G^T in the T-row, G^p and l4 G^T in the p-row.  One
+// warp per cell zeroes its two rows and then sets their entries, a lane per
+// neighbour, so no launch or memset that clears M stands before it.  Bound by
+// its launch on the grids it serves (n of some hundreds).
 template <int DIM>
-__global__ void k_coarse_assemble(int n0, int n1, int n2, const double2 *__restrict__ G0,
-                                  const double2 *__restrict__ G1, const double2 *__restrict__ G2,
-                                  const dq *__restrict__ D, const double *__restrict__ l4, double *__restrict__ M) {
-    pdl_entry();
-    const long long N = (long long)n0 * n1 * n2;
-    const long long n = 2 * N;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
+__device__ __forceinline__ void coarse_rows(const int n[3], const double2 *__restrict__ G0, const double2 *__restrict__ G1,
+                                            const double2 *__restrict__ G2, const dq *__restrict__ D,
+                                            const double *__restrict__ l4, double *__restrict__ M, int block, int blocks) {
+    const int n0 = n[0], n1 = n[1], n2 = n[2], lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+    const long long N = (long long)n0 * n1 * n2, ld = 2 * N;
+    for (long long c = block * (long long)warps + (threadIdx.x >> 5); c < N; c += (long long)blocks * warps) {
+        double *row = M + 2 * c * ld;
+        double2 *z = reinterpret_cast<double2 *>(row);
+        for (long long q = lane; q < ld; q += 32) z[q] = make_double2(0.0, 0.0);
+        __syncwarp();
         const int i = (int)(c % n0), j = (int)((c / n0) % n1), k = (int)(c / ((long long)n0 * n1));
-        const dq d = D[c];
-        M[(2 * c) * n + 2 * c] = d.a;
-        M[(2 * c) * n + 2 * c + 1] = d.b;
-        M[(2 * c + 1) * n + 2 * c] = d.c;
-        M[(2 * c + 1) * n + 2 * c + 1] = d.d;
-        const long long f0 = (long long)i + (long long)(n0 + 1) * ((long long)j + (long long)n1 * k);
-        const long long f1 = (long long)i + (long long)n0 * ((long long)j + (long long)(n1 + 1) * k);
-        const double w4 = l4[c];
-        auto put = [&](long long nb, double2 g) {
-            M[(2 * c) * n + 2 * nb] = g.x;
-            M[(2 * c + 1) * n + 2 * nb] = w4 * g.x;
-            M[(2 * c + 1) * n + 2 * nb + 1] = g.y;
-        };
-        if (i > 0) put(c - 1, G0[f0]);
-        if (i < n0 - 1) put(c + 1, G0[f0 + 1]);
-        if (j > 0) put(c - n0, G1[f1]);
-        if (j < n1 - 1) put(c + n0, G1[f1 + n0]);
-        if (DIM == 3) {
-            const long long pl = (long long)n0 * n1;
-            if (k > 0) put(c - pl, G2[c]);
-            if (k < n2 - 1) put(c + pl, G2[c + pl]);
+        if (lane == 6) {
+            const dq d = D[c];
+            row[2 * c] = d.a;
+            row[2 * c + 1] = d.b;
+            row[ld + 2 * c] = d.c;
+            row[ld + 2 * c + 1] = d.d;
+        }
+        const int axis = lane >> 1, hi = lane & 1;
+        const int at = axis == 0 ? i : axis == 1 ? j : k;
+        const int last = (axis == 0 ? n0 : axis == 1 ? n1 : n2) - 1;
+        if (axis < DIM && (hi ? at < last : at > 0)) {
+            const long long pl = (long long)n0 * n1, step = axis == 0 ? 1 : axis == 1 ? n0 : pl;
+            const long long f = axis == 0 ? i + (long long)(n0 + 1) * (j + (long long)n1 * k)
+                              : axis == 1 ? i + (long long)n0 * (j + (long long)(n1 + 1) * k) : c;
+            const double2 *G = axis == 0 ? G0 : axis == 1 ? G1 : G2;
+            const double2 g = G[f + (hi ? step : 0)];
+            const long long nb = hi ? c + step : c - step;
+            row[2 * nb] = g.x;
+            row[ld + 2 * nb] = l4[c] * g.x;
+            row[ld + 2 * nb + 1] = g.y;
         }
     }
+}
+
+struct CoarseRows {
+    int n[3];
+    const double2 *G[3];
+    const dq *D;
+    const double *l4;
+    double *M;
+};
+
+// The last kernel of a set-up: it also leaves the set-up's flags (err[0], and
+// err[2], the count of mixed precision) in page-locked host memory.
+template <int DIM>
+__global__ void k_coarse_assemble(const __grid_constant__ CoarseRows C, const int *__restrict__ err,
+                                  int *__restrict__ err_host) {
+    pdl_entry();
+    if (blockIdx.x == 0 && (threadIdx.x == 0 || threadIdx.x == 2)) err_host[threadIdx.x] = err[threadIdx.x];
+    coarse_rows<DIM>(C.n, C.G[0], C.G[1], C.G[2], C.D, C.l4, C.M, blockIdx.x, gridDim.x);
 }
 
 // Coarsest inverse for n <= kBandSmemMax in two kernels.  GB300's FP64 pipe

@@ -1,0 +1,38 @@
+"""The two ends of a solve: the initial guess read and the solution, norms and flags written by kernels.
+
+Arrays in device memory go through the kernels, host arrays through copies, and the asynchronous solve keeps its norms
+on the device; the numbers are the same bit for bit, so every comparison is exact."""
+import numpy as np
+import pytest
+
+from paper_2206_11294_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("n", [(2, 2, 1), (33, 9, 1), (40, 24, 1), (16, 12, 8)])
+def test_device_host_and_async_ends_agree(n, precision):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2206_11294_gb300.binding import Solver
+    bc = ((I.BC_WALL, I.BC_DIRICHLET), (I.BC_DIRICHLET, I.BC_WALL), (0, 0))
+    g = I.Grid(dim=2 if n[2] == 1 else 3, axisym=0, n=n, h=1e-2, bc=bc, bcT=((300.0, 301.0),) * 3,
+               bcp=((1e5, 1.1e5),) * 3)
+    p = I.random_coeff_problem(g, seed=sum(n))
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    pick = lambda st: [st[k] for k in ("cycles", "r0", "rfinal", "status")]
+    with Solver(g, precision=precision, rtol=1e-7, max_cycles=12) as s:
+        s.set_coeffs(p.lam, p.fa, p.fk)
+        b, x = dev(p.b), dev(p.x0)
+        xh, xa = np.array(p.x0, dtype=np.float64, order="C"), dev(p.x0)
+        sd = s.solve(b, x, allow_not_converged=True)
+        sh = s.solve(p.b, xh, allow_not_converged=True)
+        s.solve_async(b, xa)
+        sa = s.async_stats(allow_not_converged=True)
+        assert np.array_equal(x.cpu().numpy(), xh) and torch.equal(x, xa)
+        assert not np.array_equal(xh.reshape(-1), np.asarray(p.x0).reshape(-1))
+        assert pick(sd) == pick(sh) == pick(sa)
+        r = s.residual_norms(b, xa)
+        assert np.array_equal(r, s.residual_norms(p.b, xh)) and torch.equal(x, xa)
