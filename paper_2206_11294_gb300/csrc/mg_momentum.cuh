@@ -9,7 +9,7 @@
 // coefficients lambda_2 = lambda_4 = 0).  The cross terms div(mu grad u^T)
 // off the diagonal are the difference the outer loop removes.  When the
 // set-up's row bound 2 (off-diagonal sum) / diagonal is small (the mass term
-// dominates), the corrections are point-Jacobi steps instead (k_mom_jacobi);
+// dominates), the corrections are point-Jacobi steps instead (k_mom_step);
 // optionally the loop is restarted GMRES right-preconditioned by the
 // multigrid correction (the k_kry_* kernels).
 //
@@ -36,6 +36,8 @@ struct MomCoeffArgs {
     double *mu_o;            // owned copy of mu
     double *inv_diag[3];     // per component: 1 / the diagonal of the component-diagonal operator
     double *partial;         // per block: the largest Jacobi bound 2 off / diag of its cells and components
+    unsigned int *ticket;    // last-block counter (re-armed by the kernel)
+    double *nu_host;         // page-locked host memory: the largest bound of all
     double2 *lamA, *lamB;    // [N][2 pairs] of the correction hierarchies (B: 3D, component z)
     double *fA[2][3];        // face coefficients of components 0 and 1 (the hierarchies' T and p slots)
     double *fB[3];           // component 2 (3D)
@@ -86,6 +88,30 @@ __device__ __noinline__ void mom_off_edge(const MomCoeffArgs &A, int i, int j, i
 // arithmetic makes it) the largest, and a negative value the smallest.  On the integer pipe.
 __device__ __forceinline__ long long max_bits(long long a, long long b) { return a > b ? a : b; }
 
+__device__ __forceinline__ unsigned grid_blocks() { return gridDim.x * gridDim.y * gridDim.z; }
+
+// Called by one thread of a block after its partial is stored: true in the last block of the grid.
+__device__ __forceinline__ bool last_block(unsigned int *ticket) {
+    __threadfence();
+    return atomicAdd(ticket, 1u) == grid_blocks() - 1u;
+}
+
+// Sum of v over the block in a fixed order, in thread 0: warp 0 sums a column per lane, then one tree.
+template <int T>
+__device__ __forceinline__ double column_sum(double *red, int tid, double v) {
+    red[tid] = v;
+    __syncthreads();
+    double b = 0.0;
+    if (tid < 32) {
+        b = red[tid];
+#pragma unroll
+        for (int w = 1; w < T / 32; w++) b += red[32 * w + tid];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) b += __shfl_down_sync(0xffffffffu, b, o);
+    }
+    return b;
+}
+
 // Per cell: the owned copies, the inverse diagonals of the component-diagonal operator and the row bound
 // 2 (off-diagonal sum) / diagonal; per block, the largest bound.  Bound by the FP64 pipe: inside Cartesian grids
 // off_q is 1/(2 h^2) (S + S_q) with S_a = 2 mu + mu_lo + mu_hi the face sums of axis a and S their sum, the weight
@@ -94,6 +120,7 @@ __device__ __forceinline__ long long max_bits(long long a, long long b) { return
 template <int DIM, bool AXI>
 __global__ void __launch_bounds__(256) k_mom_diag(const __grid_constant__ MomCoeffArgs A) {
     __shared__ long long red[8];
+    __shared__ bool last;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
     const int k = DIM == 3 ? (int)blockIdx.z : 0;
@@ -141,6 +168,23 @@ __global__ void __launch_bounds__(256) k_mom_diag(const __grid_constant__ MomCoe
         long long t = 0;
         for (int w = 0; w < (int)(blockDim.x * blockDim.y) / 32; w++) t = max_bits(t, red[w]);
         A.partial[blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * (long long)blockIdx.z)] = __longlong_as_double(t);
+        last = last_block(A.ticket);
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    nu = 0;
+    for (unsigned b = tid; b < grid_blocks(); b += blockDim.x * blockDim.y)
+        nu = max_bits(nu, __double_as_longlong(__ldcg(A.partial + b)));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) nu = max_bits(nu, __shfl_down_sync(0xffffffffu, nu, o));
+    if ((tid & 31) == 0) red[tid >> 5] = nu;
+    __syncthreads();
+    if (tid == 0) {
+        long long t = 0;
+        for (int w = 0; w < (int)(blockDim.x * blockDim.y) / 32; w++) t = max_bits(t, red[w]);
+        *A.nu_host = __longlong_as_double(t);
+        *A.ticket = 0u;
     }
 }
 
@@ -206,6 +250,9 @@ struct MomArgs {
     const double *R[3];       // residual mode: the right-hand side
     double2 *rA, *rB;         // residual mode: -r as the inner right-hand sides (B: 3D, (-r_z, 0))
     double *partial;          // residual mode: per block sum of (dt r / rho)^2 over its cells and components
+    unsigned int *ticket;     // residual mode: last-block counter (re-armed by the kernel)
+    double *norm2;            // residual mode: the sum over all blocks
+    double *norm2_host;       // residual mode: the same in page-locked host memory
     double *r_out[3];         // residual mode, optional: r itself
     double *y[3];             // apply mode: A(u)
 };
@@ -267,6 +314,7 @@ __global__ void __launch_bounds__(TX * TY) k_mom_residual(const __grid_constant_
     constexpr int NX = (TX + 1) * TY, NY = TX * (TY + 1), NZ = DIM == 3 ? 2 * TX * TY : 0, NF = NX + NY + NZ;
     __shared__ double F[DIM][NF];
     __shared__ double red[APPLY ? 1 : TX * TY];
+    __shared__ bool last;
     const int i0 = blockIdx.x * TX, j0 = blockIdx.y * TY, k = DIM == 3 ? (int)blockIdx.z : 0;
     const int tid = threadIdx.x + TX * threadIdx.y;
     for (int t = tid; t < NF; t += TX * TY) {
@@ -357,62 +405,55 @@ __global__ void __launch_bounds__(TX * TY) k_mom_residual(const __grid_constant_
         }
     }
     if constexpr (!APPLY) {
-        // fixed-order block sum of the stopping norm: warp 0 sums a column of eight per lane, then one tree
-        red[tid] = s;
+        // fixed-order sums of the stopping norm: the block's, then (the last block to finish) the blocks'
+        const double b = column_sum<TX * TY>(red, tid, s);
+        if (tid == 0) {
+            A.partial[blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * (long long)blockIdx.z)] = b;
+            last = last_block(A.ticket);
+        }
         __syncthreads();
-        if (tid < 32) {
-            double b = red[tid];
-#pragma unroll
-            for (int w = 1; w < TX * TY / 32; w++) b += red[32 * w + tid];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) b += __shfl_down_sync(0xffffffffu, b, o);
-            if (tid == 0) A.partial[blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * (long long)blockIdx.z)] = b;
+        if (!last) return;
+        __threadfence();
+        s = 0.0;
+        for (unsigned q = tid; q < grid_blocks(); q += TX * TY) s += __ldcg(A.partial + q);
+        const double t = column_sum<TX * TY>(red, tid, s);
+        if (tid == 0) {
+            *A.norm2 = t;
+            *A.norm2_host = t;
+            *A.ticket = 0u;
         }
     }
 }
 
-// Largest value of an array of doubles >= 0 or NaN (one block; see max_bits).
-__global__ void __launch_bounds__(1024) k_mom_max(const double *v, long long n, double *out) {
-    __shared__ long long red[32];
-    long long s = 0;
-    for (long long b = threadIdx.x; b < n; b += blockDim.x) s = max_bits(s, __double_as_longlong(v[b]));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s = max_bits(s, __shfl_down_sync(0xffffffffu, s, o));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        long long t = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) t = max_bits(t, red[w]);
-        out[0] = __longlong_as_double(t);
+// What follows a residual in the point-Jacobi loop, launched with it: the stop test of the host (norm2[0]: the initial
+// sum of squares, norm2[1]: the latest) decides between delta_q += r_q / diag_q, r read back from the correction
+// right-hand sides (-r), and u_q += delta_q at the end (`last`: whatever the norm).  FIRST: delta is set, not added
+// to, and u needs no update.  So the host reads the norm while this kernel runs and the device does not wait for it
+// (1024^2, two steps, with the norms summed by the last block of each residual: a predictor step 576 -> 520 us).
+template <int DIM, bool FIRST>
+__global__ void __launch_bounds__(256) k_mom_step(long long N, const double *__restrict__ norm2, double rtol,
+                                                  bool last, const double2 *rA, const double2 *rB, const double *i0,
+                                                  const double *i1, const double *i2, double *d0, double *d1,
+                                                  double *d2, double *u0, double *u1, double *u2) {
+    __shared__ bool met;
+    if (threadIdx.x == 0) {         // one thread's square roots: by all they would cost three times the update
+        const double r0 = sqrt(norm2[0]), r = FIRST ? r0 : sqrt(norm2[1]);
+        met = r == 0.0 || (rtol > 0.0 && r <= rtol * r0) || (last && isfinite(r));
     }
-}
-
-// Point-Jacobi correction: delta_q += r_q / diag_q, r read back from the correction right-hand sides (-r).
-template <int DIM>
-__global__ void __launch_bounds__(256) k_mom_jacobi(long long N, const double2 *rA, const double2 *rB,
-                                                    const double *i0, const double *i1, const double *i2, double *d0,
-                                                    double *d1, double *d2) {
+    __syncthreads();
+    const bool done = met;
+    if (FIRST && done) return;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
-        const double2 r = rA[c];
-        d0[c] -= r.x * i0[c];
-        d1[c] -= r.y * i1[c];
-        if (DIM == 3) d2[c] -= rB[c].x * i2[c];
-    }
-}
-
-// Sum of the per-block partials in a fixed order (one block).
-__global__ void __launch_bounds__(1024) k_mom_norm(const double *partial, long long nblocks, double *out) {
-    __shared__ double red[32];
-    double s = 0.0;
-    for (long long b = threadIdx.x; b < nblocks; b += blockDim.x) s += partial[b];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) t += red[w];
-        out[0] = t;
+        if (done) {
+            u0[c] += d0[c];
+            u1[c] += d1[c];
+            if (DIM == 3) u2[c] += d2[c];
+        } else {
+            const double2 q = rA[c];
+            d0[c] = (FIRST ? 0.0 : d0[c]) - q.x * i0[c];
+            d1[c] = (FIRST ? 0.0 : d1[c]) - q.y * i1[c];
+            if (DIM == 3) d2[c] = (FIRST ? 0.0 : d2[c]) - rB[c].x * i2[c];
+        }
     }
 }
 

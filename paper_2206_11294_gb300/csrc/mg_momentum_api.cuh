@@ -18,10 +18,13 @@ struct mg_momentum {
     double nu;                         // Jacobi bound of the last set-up: max over rows of 2 off / diag
     bool jacobi;                       // corrections by point-Jacobi (no hierarchy set up)
     double *V, *Z;                     // Krylov basis (kKryM + 1 vectors of dim N) and one work vector
-    double *kpart, *kdot_d, *kdot_h;   // dot partials, dots (device), dots (pinned host)
+    double *kpart, *kdot_h;            // dot partials, dots (pinned host, written by the kernel)
     double2 *lamA, *lamB, *rA, *rB;
     double *fA[2][3], *fB[3], *fzero[3];
-    double *partial, *norm_d, *norm_h;
+    double *partial;
+    unsigned int *ticket;              // last-block counter of the kernels that sum partials
+    double *norm_d, *norm_h;           // squared norms of the initial [0] and latest [1] residual; host also [2]: nu
+    cudaEvent_t ev;                    // norm of the last residual written
 };
 
 namespace {
@@ -78,10 +81,10 @@ mg_status launch_momentum(const mg_momentum *m, const MomArgs &A, bool apply) {
     return MG_OK;
 }
 
-// r = R - A(u) into the correction right-hand sides (and into r_out, if given); returns ||dt r / rho||_2 (one
-// host wait).
-mg_status momentum_residual(mg_momentum *m, const double *const R[3], const double *const u[3], double *const r_out[3],
-                            double *norm) {
+// r = R - A(u) into the correction right-hand sides (and into r_out, if given); enqueues only.  ||dt r / rho||^2 goes
+// to slot `slot` of norm_d and norm_h.
+mg_status enqueue_momentum_residual(mg_momentum *m, const double *const R[3], const double *const u[3],
+                                    double *const r_out[3], int slot) {
     MomArgs A = momentum_args(m);
     for (int a = 0; a < m->grid.dim; a++) {
         A.u[a] = u[a];
@@ -91,13 +94,19 @@ mg_status momentum_residual(mg_momentum *m, const double *const R[3], const doub
     A.rA = m->rA;
     A.rB = m->rB;
     A.partial = m->partial;
-    mg_status st = launch_momentum(m, A, false);
+    A.ticket = m->ticket;
+    A.norm2 = m->norm_d + slot;
+    A.norm2_host = m->norm_h + slot;
+    return launch_momentum(m, A, false);
+}
+
+// The same with one host wait; returns the norm.
+mg_status momentum_residual(mg_momentum *m, const double *const R[3], const double *const u[3], double *const r_out[3],
+                            int slot, double *norm) {
+    mg_status st = enqueue_momentum_residual(m, R, u, r_out, slot);
     if (st) return st;
-    k_mom_norm<<<1, 1024, 0, m->stream>>>(m->partial, m->nblocks, m->norm_d);
-    CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(m->norm_h, m->norm_d, sizeof(double), cudaMemcpyDeviceToHost, m->stream));
     CK(cudaStreamSynchronize(m->stream));
-    *norm = std::sqrt(m->norm_h[0]);
+    *norm = std::sqrt(m->norm_h[slot]);
     return MG_OK;
 }
 
@@ -106,9 +115,8 @@ mg_status momentum_residual(mg_momentum *m, const double *const R[3], const doub
 mg_status kry_dots(mg_momentum *m, const double *V, int nd, const double *w, double *out) {
     const long long N = m->N, stride = (long long)m->grid.dim * N;
     k_kry_dots<<<kKryBlocks, 256, 0, m->stream>>>(N, m->grid.dim, m->wgt, V, stride, nd, w, m->kpart);
-    k_kry_reduce<<<1, 32 * nd, 0, m->stream>>>(m->kpart, kKryBlocks, nd, m->kdot_d);
+    k_kry_reduce<<<1, 32 * nd, 0, m->stream>>>(m->kpart, kKryBlocks, nd, m->kdot_h);
     CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(m->kdot_h, m->kdot_d, nd * sizeof(double), cudaMemcpyDeviceToHost, m->stream));
     CK(cudaStreamSynchronize(m->stream));
     for (int d = 0; d < nd; d++) out[d] = m->kdot_h[d];
     return MG_OK;
@@ -152,7 +160,7 @@ mg_status momentum_gmres(mg_momentum *m, double target, int max_iters, int *iter
     for (;;) {
         double *v0[3];
         comps(vec(0), v0);
-        if ((st = momentum_residual(m, r0c, dc, v0, r))) return st;
+        if ((st = momentum_residual(m, r0c, dc, v0, 1, r))) return st;
         if (!std::isfinite(*r)) return fail(MG_ERR_INVALID_COEFF, "non-finite momentum residual");
         if (*r <= target || *iters >= max_iters) return MG_OK;
         KryCoef none;
@@ -240,6 +248,7 @@ mg_status mg_momentum_destroy(mg_momentum *m) {
     mg_destroy(m->hA);
     mg_destroy(m->hB);
     if (m->arena) cudaFree(m->arena);
+    if (m->ev) cudaEventDestroy(m->ev);
     if (m->norm_h) cudaFreeHost(m->norm_h);
     if (m->kdot_h) cudaFreeHost(m->kdot_h);
     delete m;
@@ -305,12 +314,13 @@ mg_status mg_momentum_create(const mg_grid *grid, int flags, const mg_options *i
     size_t o_f[4][3] = {};
     for (int q = 0; q < (dim == 3 ? 4 : 2); q++)
         for (int a = 0; a < dim; a++) o_f[q][a] = take((size_t)nf[a] * 8);
-    const size_t o_part = take((size_t)m->nblocks * 8), o_norm = take(8);
+    const size_t o_part = take((size_t)m->nblocks * 8), o_norm = take(16), o_tick = take(4);
     const bool kry = (flags & MG_MOMENTUM_KRYLOV) != 0;
     const size_t o_V = kry ? take((size_t)(kKryM + 1) * dim * N * 8) : 0, o_Z = kry ? take((size_t)dim * N * 8) : 0,
-                 o_kp = kry ? take((size_t)(kKryM + 1) * kKryBlocks * 8) : 0, o_kd = kry ? take((kKryM + 1) * 8) : 0;
+                 o_kp = kry ? take((size_t)(kKryM + 1) * kKryBlocks * 8) : 0;
     DeviceGuard dg(m->device);
-    if (cudaMalloc(&m->arena, off) != cudaSuccess || cudaMallocHost(&m->norm_h, sizeof(double)) != cudaSuccess ||
+    if (cudaMalloc(&m->arena, off) != cudaSuccess || cudaMallocHost(&m->norm_h, 3 * sizeof(double)) != cudaSuccess ||
+        cudaEventCreateWithFlags(&m->ev, cudaEventDisableTiming) != cudaSuccess ||
         (kry && cudaMallocHost(&m->kdot_h, (kKryM + 1) * sizeof(double)) != cudaSuccess)) {
         cudaGetLastError();
         mg_momentum_destroy(m);
@@ -342,11 +352,12 @@ mg_status mg_momentum_create(const mg_grid *grid, int flags, const mg_options *i
     }
     m->partial = reinterpret_cast<double *>(at(o_part));
     m->norm_d = reinterpret_cast<double *>(at(o_norm));
+    m->ticket = reinterpret_cast<unsigned int *>(at(o_tick));
+    CK(cudaMemsetAsync(m->ticket, 0, sizeof(unsigned int), m->stream));
     if (kry) {
         m->V = reinterpret_cast<double *>(at(o_V));
         m->Z = reinterpret_cast<double *>(at(o_Z));
         m->kpart = reinterpret_cast<double *>(at(o_kp));
-        m->kdot_d = reinterpret_cast<double *>(at(o_kd));
     }
     CK(cudaStreamSynchronize(m->stream));
     *out = m;
@@ -378,6 +389,8 @@ mg_status mg_momentum_set_coeffs(mg_momentum *m, double dt, const double *rho, c
     A.rho = rho;
     A.mu = mu;
     A.partial = m->partial;        // one Jacobi bound per block
+    A.ticket = m->ticket;
+    A.nu_host = m->norm_h + 2;
     for (int a = 0; a < dim; a++) A.inv_diag[a] = m->inv_diag[a];
     A.rho_dt = m->rho_dt;
     A.wgt = m->wgt;
@@ -394,11 +407,8 @@ mg_status mg_momentum_set_coeffs(mg_momentum *m, double dt, const double *rho, c
     else if (g.axisym) k_mom_diag<2, true><<<gr, kBlock, 0, m->stream>>>(A);
     else k_mom_diag<2, false><<<gr, kBlock, 0, m->stream>>>(A);
     CK(cudaGetLastError());
-    k_mom_max<<<1, 1024, 0, m->stream>>>(m->partial, m->nblocks, m->norm_d);
-    CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(m->norm_h, m->norm_d, sizeof(double), cudaMemcpyDeviceToHost, m->stream));
     CK(cudaStreamSynchronize(m->stream));
-    const double nu = m->norm_h[0];
+    const double nu = m->norm_h[2];
     if (!std::isfinite(nu)) return fail(MG_ERR_INVALID_COEFF, "non-finite momentum coefficients");
     m->nu = nu;
     // Point-Jacobi corrections contract the residual by at least nu per step; below kJacobiNu they beat a V-cycle
@@ -465,39 +475,60 @@ mg_status mg_momentum_solve(mg_momentum *m, const double *const R[3], double *co
     const double *r0c[3] = {m->r0[0], m->r0[1], m->r0[2]};
     const double *dc[3] = {m->delta[0], m->delta[1], m->delta[2]};
     double r0 = 0.0, r = 0.0;
-    CK(cudaMemsetAsync(m->hA->err_d + 1, 0, sizeof(int), m->stream));
-    if (dim == 3) CK(cudaMemsetAsync(m->hB->err_d + 1, 0, sizeof(int), m->stream));
-    mg_status st = momentum_residual(m, R, uc, m->r0, &r0);
-    if (st) return st;
-    for (int a = 0; a < dim; a++) CK(cudaMemsetAsync(m->delta[a], 0, (size_t)m->N * 8, m->stream));
-    if (!std::isfinite(r0)) return fail(MG_ERR_INVALID_COEFF, "non-finite momentum residual");
-    r = r0;
     int it = 0, cycles = 0;
-    mg_status result = MG_OK;
-    if (m->V && !m->jacobi && !(r == 0.0 || (rtol > 0.0 && r <= rtol * r0))) {
-        int precs = 0;
-        const double target = rtol > 0.0 ? rtol * r0 : 0.0;
-        if ((st = momentum_gmres(m, target, max_iters, &it, &precs, &r))) return st;
-        cycles = precs * m->hA->opt.max_cycles * (dim == 3 ? 2 : 1);
-        if (!(r == 0.0 || (rtol > 0.0 && r <= rtol * r0))) result = rtol > 0.0 ? MG_ERR_NOT_CONVERGED : MG_OK;
-    }
-    for (; !m->V || m->jacobi;) {
-        if (r == 0.0 || (rtol > 0.0 && r <= rtol * r0)) break;
-        if (it >= max_iters) {
-            result = rtol > 0.0 ? MG_ERR_NOT_CONVERGED : MG_OK;
-            break;
-        }
-        const int blocks = (int)std::min<long long>((m->N + 255) / 256, 152LL * 16);
-        double *const *d = m->delta;
+    mg_status st, result = MG_OK;
+    const int blocks = (int)std::min<long long>((m->N + 255) / 256, 152LL * 16);
+    double *const *d = m->delta;
+    auto met = [&]() { return r == 0.0 || (rtol > 0.0 && r <= rtol * r0); };
+    if (m->jacobi) {
+        // each residual is followed at once by the kernel that its norm leads to, so the device does not wait for
+        // the host's stop test
         double *const *id = m->inv_diag;
-        if (m->jacobi) {
+        auto follow = [&](auto kern2, auto kern3, bool last) -> mg_status {
+            CK(cudaEventRecord(m->ev, m->stream));
             if (dim == 3)
-                k_mom_jacobi<3><<<blocks, 256, 0, m->stream>>>(m->N, m->rA, m->rB, id[0], id[1], id[2], d[0], d[1],
-                                                               d[2]);
+                kern3<<<blocks, 256, 0, m->stream>>>(m->N, m->norm_d, rtol, last, m->rA, m->rB, id[0], id[1], id[2], d[0],
+                                                     d[1], d[2], u[0], u[1], u[2]);
             else
-                k_mom_jacobi<2><<<blocks, 256, 0, m->stream>>>(m->N, m->rA, nullptr, id[0], id[1], nullptr, d[0],
-                                                               d[1], nullptr);
-        } else {
+                kern2<<<blocks, 256, 0, m->stream>>>(m->N, m->norm_d, rtol, last, m->rA, nullptr, id[0], id[1], nullptr,
+                                                     d[0], d[1], nullptr, u[0], u[1], nullptr);
+            CK(cudaGetLastError());
+            CK(cudaEventSynchronize(m->ev));
+            return MG_OK;
+        };
+        if ((st = enqueue_momentum_residual(m, R, uc, m->r0, 0))) return st;
+        if ((st = follow(k_mom_step<2, true>, k_mom_step<3, true>, false))) return st;
+        r = r0 = std::sqrt(m->norm_h[0]);
+        bool finite = std::isfinite(r);
+        while (finite && !met() && it < max_iters) {
+            if ((st = enqueue_momentum_residual(m, r0c, dc, nullptr, 1))) return st;
+            it++;
+            if ((st = follow(k_mom_step<2, false>, k_mom_step<3, false>, it >= max_iters))) return st;
+            r = std::sqrt(m->norm_h[1]);
+            finite = std::isfinite(r);
+        }
+        CK(cudaStreamSynchronize(m->stream));
+        if (!finite) return fail(MG_ERR_INVALID_COEFF, "non-finite momentum residual");
+        if (!met()) result = rtol > 0.0 ? MG_ERR_NOT_CONVERGED : MG_OK;
+    } else {
+        CK(cudaMemsetAsync(m->hA->err_d + 1, 0, sizeof(int), m->stream));
+        if (dim == 3) CK(cudaMemsetAsync(m->hB->err_d + 1, 0, sizeof(int), m->stream));
+        if ((st = momentum_residual(m, R, uc, m->r0, 0, &r0))) return st;
+        for (int a = 0; a < dim; a++) CK(cudaMemsetAsync(m->delta[a], 0, (size_t)m->N * 8, m->stream));
+        if (!std::isfinite(r0)) return fail(MG_ERR_INVALID_COEFF, "non-finite momentum residual");
+        r = r0;
+        if (m->V && !met()) {
+            int precs = 0;
+            const double target = rtol > 0.0 ? rtol * r0 : 0.0;
+            if ((st = momentum_gmres(m, target, max_iters, &it, &precs, &r))) return st;
+            cycles = precs * m->hA->opt.max_cycles * (dim == 3 ? 2 : 1);
+            if (!met()) result = rtol > 0.0 ? MG_ERR_NOT_CONVERGED : MG_OK;
+        }
+        while (!m->V && !met()) {
+            if (it >= max_iters) {
+                result = rtol > 0.0 ? MG_ERR_NOT_CONVERGED : MG_OK;
+                break;
+            }
             if (dim == 3) {
                 if ((st = correction_cycles<3>(m->hA, m->rA)) || (st = correction_cycles<3>(m->hB, m->rB))) return st;
                 cycles += 2 * m->hA->opt.max_cycles;
@@ -508,20 +539,18 @@ mg_status mg_momentum_solve(mg_momentum *m, const double *const R[3], double *co
             const double2 *xa = m->hA->L[0].x, *xb = dim == 3 ? m->hB->L[0].x : nullptr;
             if (dim == 3) k_mom_update<3><<<blocks, 256, 0, m->stream>>>(m->N, xa, xb, d[0], d[1], d[2]);
             else k_mom_update<2><<<blocks, 256, 0, m->stream>>>(m->N, xa, xb, d[0], d[1], nullptr);
+            CK(cudaGetLastError());
+            if ((st = momentum_residual(m, r0c, dc, nullptr, 1, &r))) return st;
+            it++;
+            if (!std::isfinite(r)) return fail(MG_ERR_INVALID_COEFF, "non-finite momentum residual");
         }
-        CK(cudaGetLastError());
-        if ((st = momentum_residual(m, r0c, dc, nullptr, &r))) return st;
-        it++;
-        if (!std::isfinite(r)) return fail(MG_ERR_INVALID_COEFF, "non-finite momentum residual");
-    }
-    if (it > 0) {
-        const int blocks = (int)std::min<long long>((m->N + 255) / 256, 152LL * 16);
-        double *const *d = m->delta;
-        if (dim == 3) k_mom_add<3><<<blocks, 256, 0, m->stream>>>(m->N, d[0], d[1], d[2], u[0], u[1], u[2]);
-        else k_mom_add<2><<<blocks, 256, 0, m->stream>>>(m->N, d[0], d[1], nullptr, u[0], u[1], nullptr);
-        CK(cudaGetLastError());
-        CK(cudaStreamSynchronize(m->stream));
-        if (!m->jacobi && ((st = handle_errors(m->hA)) || (dim == 3 && (st = handle_errors(m->hB))))) return st;
+        if (it > 0) {
+            if (dim == 3) k_mom_add<3><<<blocks, 256, 0, m->stream>>>(m->N, d[0], d[1], d[2], u[0], u[1], u[2]);
+            else k_mom_add<2><<<blocks, 256, 0, m->stream>>>(m->N, d[0], d[1], nullptr, u[0], u[1], nullptr);
+            CK(cudaGetLastError());
+            CK(cudaStreamSynchronize(m->stream));
+            if ((st = handle_errors(m->hA)) || (dim == 3 && (st = handle_errors(m->hB)))) return st;
+        }
     }
     if (stats) {
         stats->iterations = it;
