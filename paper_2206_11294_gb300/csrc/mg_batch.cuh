@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(kBatchThreads) kb_prep(const BLevel *__restric
         const int gx = (L.n0 + kBX - 1) / kBX, gy = (L.n1 + kBY - 1) / kBY;
         int bx, by, bz;
         block_coords(e.y, gx, gy, bx, by, bz);
-        prep_rhs_block<DIM>(L, P.rhs, P.xin, P.bv, P.axisym, P.r0, P.h, bx, by, bz);
+        prep_rhs_block<DIM>(L, P.rhs, P.xin, P.bv, P.axisym, P.r0, P.h, false, bx, by, bz);
     }
 }
 

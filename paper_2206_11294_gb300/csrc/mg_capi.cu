@@ -1082,12 +1082,13 @@ mg_status x_out(mg_handle *h, double *x, int on_device) {
     return MG_OK;
 }
 
-// xin (may be NULL): also copied to x.  clear (may be NULL): an int set to 0.
+// xin (may be NULL): also copied to x.  clear (may be NULL): an int set to 0.  zero: x is set to 0.
 template <int DIM>
-void enqueue_prep(mg_handle *h, const double2 *rhs, cudaStream_t s, const double2 *xin = nullptr, int *clear = nullptr) {
+void enqueue_prep(mg_handle *h, const double2 *rhs, cudaStream_t s, const double2 *xin = nullptr, int *clear = nullptr,
+                  bool zero = false) {
     const LevelBuf &f = h->L[0];
     launch_k(h, k_prep_rhs<DIM>, cell_grid(f, DIM, f.n[0]), kBlock, 0, s, 0, view<double>(f), rhs, xin, bc_vals(h->grid),
-             h->grid.axisym, h->grid.r0, h->grid.h, clear);
+             h->grid.axisym, h->grid.r0, h->grid.h, clear, zero ? 1 : 0);
     counted(h);
 }
 
@@ -1569,9 +1570,7 @@ mg_status correction_cycles(mg_handle *h, const double2 *rhs) {
         });
         if (e) return e;
     }
-    const LevelBuf &f = h->L[0];
-    CK(cudaMemsetAsync(f.x, 0, sizeof(double2) * f.N, h->stream));
-    enqueue_prep<DIM>(h, rhs, h->stream);
+    enqueue_prep<DIM>(h, rhs, h->stream, nullptr, nullptr, true);
     CK(cudaGetLastError());
     CK(cudaGraphLaunch(h->gcorr, h->stream));
     h->enq += h->graph_kernels_corr;
@@ -1586,8 +1585,7 @@ mg_status correction_cycles(mg_handle *h, const double2 *rhs) {
 template <int DIM>
 mg_status enqueue_correction(mg_handle *h, cudaStream_t s, const double2 *rhs) {
     const LevelBuf &f = h->L[0];
-    CK(cudaMemsetAsync(f.x, 0, sizeof(double2) * f.N, s));
-    enqueue_prep<DIM>(h, rhs, s);
+    enqueue_prep<DIM>(h, rhs, s, nullptr, nullptr, true);
     if (h->opt.precision == MG_MIXED) {
         enqueue_residual_to32<DIM>(h, s, true, nullptr);        // x = 0: b32 = b, bt32 = Dinv b, e32 = 0
         for (int q = 0; q < h->opt.max_cycles; q++)

@@ -23,7 +23,7 @@
 // Cells are x-fastest; base faces of axis 0 are (n0 + 1) per row, of axis 1
 // n0 per row over n1 + 1 rows; the patch's likewise with m0, m1.
 #pragma once
-#include "mg_types.cuh"
+#include "mg_kernels.cuh"
 
 namespace cmg {
 
@@ -62,22 +62,26 @@ __device__ __forceinline__ long long cf_fface(const CfGeom &g, int a, int i, int
 
 // (T, p) of base cell (I, J), or across the domain boundary its ghost: the
 // mirror at a wall, 2 g - u at a Dirichlet side, each side's rule in turn
-// (x first) at a corner.
-__device__ __forceinline__ double2 cf_base_value(const CfGeom &g, const double2 *__restrict__ xb, int I, int J) {
-    int out[2] = {-1, -1};
-    int ci = I, cj = J;
-    if (I < 0) { ci = 0; out[0] = 0; }
-    if (I >= g.n0) { ci = g.n0 - 1; out[0] = 1; }
-    if (J < 0) { cj = 0; out[1] = 0; }
-    if (J >= g.n1) { cj = g.n1 - 1; out[1] = 1; }
-    double2 u = xb[ci + (long long)g.n0 * cj];
-#pragma unroll
+// (x first) at a corner.  In two parts, so that a caller of several values has
+// all their loads in flight: the cell's own or its inner neighbour's value, and
+// the rule.
+__device__ __forceinline__ double2 cf_base_load(const CfGeom &g, const double2 *__restrict__ xb, int I, int J) {
+    return xb[min(max(I, 0), g.n0 - 1) + (long long)g.n0 * min(max(J, 0), g.n1 - 1)];
+}
+
+__device__ __forceinline__ double2 cf_base_rule(const CfGeom &g, double2 u, int I, int J) {
+    if (I >= 0 && I < g.n0 && J >= 0 && J < g.n1) return u;
+#pragma unroll 1
     for (int ax = 0; ax < 2; ax++) {
-        const int s = out[ax];
-        if (s < 0 || !g.dir[ax][s]) continue;
-        u = make_double2(2.0 * g.gT[ax][s] - u.x, 2.0 * g.gp[ax][s] - u.y);
+        const int q = ax == 0 ? I : J, s = q < 0 ? 0 : 1;
+        if ((q < 0 || q >= (ax == 0 ? g.n0 : g.n1)) && g.dir[ax][s])
+            u = make_double2(2.0 * g.gT[ax][s] - u.x, 2.0 * g.gp[ax][s] - u.y);
     }
     return u;
+}
+
+__device__ __forceinline__ double2 cf_base_value(const CfGeom &g, const double2 *__restrict__ xb, int I, int J) {
+    return cf_base_rule(g, cf_base_load(g, xb, I, J), I, J);
 }
 
 // u~ of patch cell (fi, fj) across its interface side (a, s).
@@ -92,98 +96,117 @@ __device__ __forceinline__ double2 cf_ghost(const CfGeom &g, const double2 *__re
     int Cp[2] = {C[0], C[1]}, Cm[2] = {C[0], C[1]};
     Cp[t] += 1;
     Cm[t] -= 1;
-    const double2 uc = cf_base_value(g, xb, C[0], C[1]);
-    const double2 up = cf_base_value(g, xb, Cp[0], Cp[1]);
-    const double2 um = cf_base_value(g, xb, Cm[0], Cm[1]);
+    double2 uc = cf_base_load(g, xb, C[0], C[1]), up = cf_base_load(g, xb, Cp[0], Cp[1]),
+            um = cf_base_load(g, xb, Cm[0], Cm[1]);
+    uc = cf_base_rule(g, uc, C[0], C[1]);
+    up = cf_base_rule(g, up, Cp[0], Cp[1]);
+    um = cf_base_rule(g, um, Cm[0], Cm[1]);
     return make_double2(uc.x + sgn * (up.x - um.x) * 0.125, uc.y + sgn * (up.y - um.y) * 0.125);
 }
 
-// div(k grad T), div((1/rho) grad p) of valid base cell (I, J).
-__device__ __forceinline__ void cf_base_div(const CfGeom &g, const CfCoef &k, const double2 *__restrict__ xb,
-                                            const double2 *__restrict__ xf, int I, int J, double &lapT, double &lapp) {
-    const double2 u = xb[I + (long long)g.n0 * J];
-    lapT = 0.0;
-    lapp = 0.0;
-#pragma unroll
-    for (int a = 0; a < 2; a++)
-#pragma unroll
-        for (int s = 0; s < 2; s++) {
-            int nb[2] = {I, J};
-            nb[a] += s ? 1 : -1;
-            const int na = a == 0 ? g.n0 : g.n1;
-            const bool inside = nb[a] >= 0 && nb[a] < na;
-            if (inside && cf_covered(g, nb[0], nb[1])) {
-                const int t = 1 - a, side = s ? 0 : 1;
-                const int fin = side == 0 ? 0 : (a == 0 ? g.m0 : g.m1) - 1;
-                const int ct = t == 0 ? I : J;
-#pragma unroll
-                for (int q = 0; q < 2; q++) {
-                    int ff[2];
-                    ff[a] = fin;
-                    ff[t] = 2 * (ct - g.b0[t]) + q;
-                    int fface[2] = {ff[0], ff[1]};
-                    fface[a] += side;
-                    const long long fid = cf_fface(g, a, fface[0], fface[1]);
-                    const double2 uf = xf[ff[0] + (long long)g.m0 * ff[1]];
-                    const double2 gu = cf_ghost(g, xb, a, side, ff[0], ff[1]);
-                    lapT += k.fkf[a][fid] * (uf.x - gu.x) * g.rbif;
-                    lapp += k.faf[a][fid] * (uf.y - gu.y) * g.rbif;
-                }
-            } else if (inside) {
-                const long long fid = cf_bface(g, a, I + (a == 0 ? s : 0), J + (a == 1 ? s : 0));
-                const double2 un = xb[nb[0] + (long long)g.n0 * nb[1]];
-                lapT += k.fkb[a][fid] * (un.x - u.x) * g.rH2;
-                lapp += k.fab[a][fid] * (un.y - u.y) * g.rH2;
-            } else if (g.dir[a][s]) {
-                const long long fid = cf_bface(g, a, I + (a == 0 ? s : 0), J + (a == 1 ? s : 0));
-                lapT += k.fkb[a][fid] * (g.gT[a][s] - u.x) * g.rdb;
-                lapp += k.fab[a][fid] * (g.gp[a][s] - u.y) * g.rdb;
-            }
-        }
+// The sides of a cell whose neighbour lies on its own level (bit 2 a + s) are taken by every cell in one straight line,
+// a missing side with coefficient 0 and the cell's own value; what the missing sides add follows in a rolled loop, one
+// pass for nearly every cell that has any.  Branches per side, with the ghosts' code four times over, set the time of
+// these kernels: the few warps along the patch's sides ran it serially and from a cold instruction cache.  With the
+// spacing's factor taken once, the base rows of 512^2 went 18.3 -> 15.4 us; the rest is the FP64 pipe, 26
+// instructions a cell.
+__device__ __forceinline__ double2 cf_own_div(const double *const fk[2], const double *const fa[2],
+                                              const double2 *__restrict__ x, int sides, int n0, long long c, long long f,
+                                              double2 u, double r2) {
+    const bool w = sides & 1, e = sides & 2, so = sides & 4, no = sides & 8;
+    const double2 xw = x[w ? c - 1 : c], xe = x[e ? c + 1 : c], xs = x[so ? c - n0 : c], xn = x[no ? c + n0 : c];
+    const double k0 = fk[0][f], k1 = fk[0][f + 1], k2 = fk[1][c], k3 = fk[1][c + n0];
+    const double a0 = fa[0][f], a1 = fa[0][f + 1], a2 = fa[1][c], a3 = fa[1][c + n0];
+    double T = (w ? k0 : 0.0) * (xw.x - u.x), p = (w ? a0 : 0.0) * (xw.y - u.y);
+    T = fma(e ? k1 : 0.0, xe.x - u.x, T);
+    p = fma(e ? a1 : 0.0, xe.y - u.y, p);
+    T = fma(so ? k2 : 0.0, xs.x - u.x, T);
+    p = fma(so ? a2 : 0.0, xs.y - u.y, p);
+    T = fma(no ? k3 : 0.0, xn.x - u.x, T);
+    p = fma(no ? a3 : 0.0, xn.y - u.y, p);
+    return make_double2(T * r2, p * r2);
 }
 
-// div(k grad T), div((1/rho) grad p) of patch cell (i, j), and the diagonal
-// terms sigma_k, sigma_a (minus the coefficients of its own T and p).
-__device__ __forceinline__ void cf_fine_div(const CfGeom &g, const CfCoef &k, const double2 *__restrict__ xb,
-                                            const double2 *__restrict__ xf, int i, int j, double &lapT, double &lapp,
-                                            double &sk, double &sa) {
-    const double2 u = xf[i + (long long)g.m0 * j];
-    lapT = lapp = sk = sa = 0.0;
+// The sides of base cell (I, J) with a covered neighbour (which lies in the domain).
+__device__ __forceinline__ int cf_covered_sides(const CfGeom &g, int I, int J) {
+    if (!(I >= g.b0[0] - 1 && I <= g.b1[0] && J >= g.b0[1] - 1 && J <= g.b1[1])) return 0;
+    return (int)cf_covered(g, I - 1, J) | (int)cf_covered(g, I + 1, J) << 1 | (int)cf_covered(g, I, J - 1) << 2 |
+           (int)cf_covered(g, I, J + 1) << 3;
+}
+
+// div(k grad T), div((1/rho) grad p) of valid base cell (I, J).
+__device__ __forceinline__ double2 cf_base_div(const CfGeom &g, const CfCoef &k, const double2 *__restrict__ xb,
+                                               const double2 *__restrict__ xf, int I, int J, double2 u) {
+    const long long c = I + (long long)g.n0 * J;
+    const int in = (I > 0) | (I < g.n0 - 1) << 1 | (J > 0) << 2 | (J < g.n1 - 1) << 3;
+    const int covered = cf_covered_sides(g, I, J);
+    double2 lap = cf_own_div(k.fkb, k.fab, xb, in & ~covered, g.n0, c, cf_bface(g, 0, I, J), u, g.rH2);
+#pragma unroll 1
+    for (int left = 15 & ~(in & ~covered); left; left &= left - 1) {
+        const int bit = __ffs(left) - 1, a = bit >> 1, s = bit & 1;
+        if (covered >> bit & 1) {
+            const int side = s ^ 1;                                       // the patch's side
+            const int fin = side == 0 ? 0 : (a == 0 ? g.m0 : g.m1) - 1;
+            const int f0 = 2 * (a == 0 ? J - g.b0[1] : I - g.b0[0]);      // first of the two fine cells
+            const double *fk = k.fkf[a], *fa = k.faf[a];
+            double2 uf[2];
+            double ck[2], ca[2];
 #pragma unroll
-    for (int a = 0; a < 2; a++)
-#pragma unroll
-        for (int s = 0; s < 2; s++) {
-            int nb[2] = {i, j};
-            nb[a] += s ? 1 : -1;
-            const int ma = a == 0 ? g.m0 : g.m1;
-            const long long fid = cf_fface(g, a, i + (a == 0 ? s : 0), j + (a == 1 ? s : 0));
-            const double ck = k.fkf[a][fid], ca = k.faf[a][fid];
-            if (nb[a] >= 0 && nb[a] < ma) {
-                const double2 un = xf[nb[0] + (long long)g.m0 * nb[1]];
-                lapT += ck * (un.x - u.x) * g.rh2;
-                lapp += ca * (un.y - u.y) * g.rh2;
-                sk += ck * g.rh2;
-                sa += ca * g.rh2;
-            } else if (g.iface[a][s]) {
-                const double2 gu = cf_ghost(g, xb, a, s, i, j);
-                lapT += ck * (gu.x - u.x) * g.rif;
-                lapp += ca * (gu.y - u.y) * g.rif;
-                sk += ck * g.rif;
-                sa += ca * g.rif;
-            } else if (g.dir[a][s]) {
-                lapT += ck * (g.gT[a][s] - u.x) * g.rdf;
-                lapp += ca * (g.gp[a][s] - u.y) * g.rdf;
-                sk += ck * g.rdf;
-                sa += ca * g.rdf;
+            for (int q = 0; q < 2; q++) {
+                const int i = a == 0 ? fin : f0 + q, j = a == 0 ? f0 + q : fin;
+                const long long fid = cf_fface(g, a, i + (a == 0 ? side : 0), j + (a == 1 ? side : 0));
+                uf[q] = xf[i + (long long)g.m0 * j];
+                ck[q] = fk[fid];
+                ca[q] = fa[fid];
             }
+            // both ghosts: their coarse cell is this one, its tangential neighbours the next ones along the side
+            double2 up = cf_base_load(g, xb, I + (a == 1), J + (a == 0));
+            double2 um = cf_base_load(g, xb, I - (a == 1), J - (a == 0));
+            up = cf_base_rule(g, up, I + (a == 1), J + (a == 0));
+            um = cf_base_rule(g, um, I - (a == 1), J - (a == 0));
+            const double dT = (up.x - um.x) * 0.125, dp = (up.y - um.y) * 0.125;
+            lap.x += (ck[0] * (uf[0].x - (u.x - dT)) + ck[1] * (uf[1].x - (u.x + dT))) * g.rbif;
+            lap.y += (ca[0] * (uf[0].y - (u.y - dp)) + ca[1] * (uf[1].y - (u.y + dp))) * g.rbif;
+        } else if (g.dir[a][s]) {
+            const long long fid = cf_bface(g, a, I + (a == 0 ? s : 0), J + (a == 1 ? s : 0));
+            lap.x += k.fkb[a][fid] * (g.gT[a][s] - u.x) * g.rdb;
+            lap.y += k.fab[a][fid] * (g.gp[a][s] - u.y) * g.rdb;
         }
+    }
+    return lap;
+}
+
+__device__ __forceinline__ int cf_fine_sides(const CfGeom &g, int i, int j) {
+    return (i > 0) | (i < g.m0 - 1) << 1 | (j > 0) << 2 | (j < g.m1 - 1) << 3;
+}
+
+// div(k grad T), div((1/rho) grad p) of patch cell (i, j).
+__device__ __forceinline__ double2 cf_fine_div(const CfGeom &g, const CfCoef &k, const double2 *__restrict__ xb,
+                                               const double2 *__restrict__ xf, int i, int j, double2 u) {
+    const int in = cf_fine_sides(g, i, j);
+    double2 lap = cf_own_div(k.fkf, k.faf, xf, in, g.m0, i + (long long)g.m0 * j, cf_fface(g, 0, i, j), u, g.rh2);
+#pragma unroll 1
+    for (int left = 15 & ~in; left; left &= left - 1) {
+        const int bit = __ffs(left) - 1, a = bit >> 1, s = bit & 1;
+        if (!g.iface[a][s] && !g.dir[a][s]) continue;
+        const long long fid = cf_fface(g, a, i + (a == 0 ? s : 0), j + (a == 1 ? s : 0));
+        const double ck = k.fkf[a][fid], ca = k.faf[a][fid];
+        double2 v = make_double2(g.gT[a][s], g.gp[a][s]);
+        if (g.iface[a][s]) v = cf_ghost(g, xb, a, s, i, j);
+        const double w = g.iface[a][s] ? g.rif : g.rdf;
+        lap.x += ck * (v.x - u.x) * w;
+        lap.y += ca * (v.y - u.y) * w;
+    }
+    return lap;
 }
 
 // Composite rows: y = L(x) on the valid base cells (covered cells 0) or, with
 // b, r = b - L(x).
-__global__ void __launch_bounds__(256) k_cf_rows_base(CfGeom g, CfCoef k, const double2 *__restrict__ xb,
+__global__ void __launch_bounds__(256) k_cf_rows_base(const __grid_constant__ CfGeom g,
+                                                      const __grid_constant__ CfCoef k, const double2 *__restrict__ xb,
                                                       const double2 *__restrict__ xf, const double2 *__restrict__ b,
                                                       double2 *__restrict__ out) {
+    pdl_entry();
     const int I = blockIdx.x * blockDim.x + threadIdx.x, J = blockIdx.y * blockDim.y + threadIdx.y;
     if (I >= g.n0 || J >= g.n1) return;
     const long long c = I + (long long)g.n0 * J;
@@ -191,49 +214,84 @@ __global__ void __launch_bounds__(256) k_cf_rows_base(CfGeom g, CfCoef k, const 
         out[c] = make_double2(0.0, 0.0);
         return;
     }
-    double lapT, lapp;
-    cf_base_div(g, k, xb, xf, I, J, lapT, lapp);
+    const double2 u = xb[c], lap = cf_base_div(g, k, xb, xf, I, J, u);
+    const double lapT = lap.x, lapp = lap.y;
     const double *l = k.lamb + 4 * c;
-    const double2 u = xb[c];
     const double yT = lapT + l[0] * u.x + l[1] * u.y;
     const double yp = lapp + l[2] * u.y + l[3] * lapT;
     out[c] = b ? make_double2(b[c].x - yT, b[c].y - yp) : make_double2(yT, yp);
 }
 
-__global__ void __launch_bounds__(256) k_cf_rows_fine(CfGeom g, CfCoef k, const double2 *__restrict__ xb,
+__global__ void __launch_bounds__(256) k_cf_rows_fine(const __grid_constant__ CfGeom g,
+                                                      const __grid_constant__ CfCoef k, const double2 *__restrict__ xb,
                                                       const double2 *__restrict__ xf, const double2 *__restrict__ b,
                                                       double2 *__restrict__ out) {
+    pdl_entry();
     const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
     if (i >= g.m0 || j >= g.m1) return;
     const long long c = i + (long long)g.m0 * j;
-    double lapT, lapp, sk, sa;
-    cf_fine_div(g, k, xb, xf, i, j, lapT, lapp, sk, sa);
+    const double2 u = xf[c], lap = cf_fine_div(g, k, xb, xf, i, j, u);
+    const double lapT = lap.x, lapp = lap.y;
     const double *l = k.lamf + 4 * c;
-    const double2 u = xf[c];
     const double yT = lapT + l[0] * u.x + l[1] * u.y;
     const double yp = lapp + l[2] * u.y + l[3] * lapT;
     out[c] = b ? make_double2(b[c].x - yT, b[c].y - yp) : make_double2(yT, yp);
 }
 
+// Off-diagonal sums and diagonal terms (the coefficients of the cell's own T and p, negated) of a patch row of the
+// correction problem: zero base values and Dirichlet values, so only the patch's own neighbours enter the sums.
+struct CfRow {
+    double T, p, sk, sa;
+};
+
+__device__ __forceinline__ CfRow cf_row(const CfGeom &g, const CfCoef &k, const double2 *xf, int first, int i, int j,
+                                        long long c) {
+    const long long f = cf_fface(g, 0, i, j);
+    const int in = cf_fine_sides(g, i, j);
+    const bool w = in & 1, e = in & 2, so = in & 4, no = in & 8;
+    double k0 = k.fkf[0][f], k1 = k.fkf[0][f + 1], k2 = k.fkf[1][c], k3 = k.fkf[1][c + g.m0];
+    double a0 = k.faf[0][f], a1 = k.faf[0][f + 1], a2 = k.faf[1][c], a3 = k.faf[1][c + g.m0];
+    if (!w) k0 = a0 = 0.0;
+    if (!e) k1 = a1 = 0.0;
+    if (!so) k2 = a2 = 0.0;
+    if (!no) k3 = a3 = 0.0;
+    CfRow r = {0.0, 0.0, ((k0 + k1) + (k2 + k3)) * g.rh2, ((a0 + a1) + (a2 + a3)) * g.rh2};
+    if (!first) {
+        const double2 xw = xf[w ? c - 1 : c + 1], xe = xf[e ? c + 1 : c - 1], xs = xf[so ? c - g.m0 : c + g.m0],
+                      xn = xf[no ? c + g.m0 : c - g.m0];                  // (a patch has two cells per axis at least)
+        r.T = fma(k3, xn.x, fma(k2, xs.x, fma(k1, xe.x, k0 * xw.x))) * g.rh2;
+        r.p = fma(a3, xn.y, fma(a2, xs.y, fma(a1, xe.y, a0 * xw.y))) * g.rh2;
+    }
+#pragma unroll 1
+    for (int left = 15 & ~in; left; left &= left - 1) {
+        const int bit = __ffs(left) - 1, a = bit >> 1, s = bit & 1;
+        const double wt = g.iface[a][s] ? g.rif : g.dir[a][s] ? g.rdf : 0.0;
+        const long long fid = cf_fface(g, a, i + (a == 0 ? s : 0), j + (a == 1 ? s : 0));
+        r.sk = fma(k.fkf[a][fid], wt, r.sk);
+        r.sa = fma(k.faf[a][fid], wt, r.sa);
+    }
+    return r;
+}
+
 // One colour of a red-black block Gauss-Seidel sweep on the patch rows of the
-// correction problem (homogeneous: g has zero Dirichlet values and the base
-// values xb0 are zero; a nonzero base correction enters through rhs).
-__global__ void __launch_bounds__(256) k_cf_rbgs_fine(CfGeom g, CfCoef k, const double2 *__restrict__ xb0,
-                                                      const double2 *__restrict__ rhs, double2 *__restrict__ xf,
-                                                      int colour) {
+// correction problem (homogeneous: g has zero Dirichlet values; a nonzero base
+// correction enters through rhs).  first: the correction is zero, xf holds
+// nothing yet.  Bound by the FP64 pipe: the off-diagonal sums are formed alone
+// rather than as the row less its diagonal, about half the instructions (a colour of a 250^2 patch: 6.4 -> 4.6 us).
+__global__ void __launch_bounds__(256) k_cf_rbgs_fine(const __grid_constant__ CfGeom g, const __grid_constant__ CfCoef k,
+                                                      const double2 *__restrict__ rhs, double2 *xf, int colour,
+                                                      int first) {
+    pdl_entry();
     const int ii = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
     const int i = 2 * ii + ((j + colour) & 1);
     if (i >= g.m0 || j >= g.m1) return;
     const long long c = i + (long long)g.m0 * j;
-    double lapT, lapp, sk, sa;
-    cf_fine_div(g, k, xb0, xf, i, j, lapT, lapp, sk, sa);
-    const double *l = k.lamf + 4 * c;
-    const double2 u = xf[c];
-    const double e0 = lapT + l[0] * u.x + l[1] * u.y;
-    const double e1 = lapp + l[2] * u.y + l[3] * lapT;
-    const double D0 = l[0] - sk, D1 = l[1], D2 = -l[3] * sk, D3 = l[2] - sa;
-    const double s0 = rhs[c].x - (e0 - (D0 * u.x + D1 * u.y));
-    const double s1 = rhs[c].y - (e1 - (D2 * u.x + D3 * u.y));
+    const CfRow r = cf_row(g, k, xf, first, i, j, c);
+    const dq l = ldgq(reinterpret_cast<const dq *>(k.lamf) + c);
+    const double2 b = rhs[c];
+    // the p-row holds l4 times the T-row's fluxes
+    const double s0 = b.x - r.T, s1 = b.y - fma(l.d, r.T, r.p);
+    const double D0 = l.a - r.sk, D1 = l.b, D2 = -l.d * r.sk, D3 = l.c - r.sa;
     const double rdet = 1.0 / (D0 * D3 - D1 * D2);
     xf[c] = make_double2((D3 * s0 - D1 * s1) * rdet, (D0 * s1 - D2 * s0) * rdet);
 }
@@ -242,9 +300,10 @@ __global__ void __launch_bounds__(256) k_cf_rbgs_fine(CfGeom g, CfCoef k, const 
 // residual rb minus what the patch correction df adds to their rows through
 // the interface (zero base values); covered cells the mean of their four
 // children's patch residual sf.
-__global__ void __launch_bounds__(256) k_cf_base_rhs(CfGeom g, CfCoef k, const double2 *__restrict__ rb,
+__global__ void __launch_bounds__(256) k_cf_base_rhs(const __grid_constant__ CfGeom g, const __grid_constant__ CfCoef k, const double2 *__restrict__ rb,
                                                      const double2 *__restrict__ df, const double2 *__restrict__ sf,
                                                      double2 *__restrict__ sb) {
+    pdl_entry();
     const int I = blockIdx.x * blockDim.x + threadIdx.x, J = blockIdx.y * blockDim.y + threadIdx.y;
     if (I >= g.n0 || J >= g.n1) return;
     const long long c = I + (long long)g.n0 * J;
@@ -260,30 +319,20 @@ __global__ void __launch_bounds__(256) k_cf_base_rhs(CfGeom g, CfCoef k, const d
         return;
     }
     double tT = 0.0, tp = 0.0;
+#pragma unroll 1
+    for (int left = cf_covered_sides(g, I, J); left; left &= left - 1) {
+        const int bit = __ffs(left) - 1, a = bit >> 1, side = (bit & 1) ^ 1;
+        const int fin = side == 0 ? 0 : (a == 0 ? g.m0 : g.m1) - 1;
+        const int f0 = 2 * (a == 0 ? J - g.b0[1] : I - g.b0[0]);
 #pragma unroll
-    for (int a = 0; a < 2; a++)
-#pragma unroll
-        for (int s = 0; s < 2; s++) {
-            int nb[2] = {I, J};
-            nb[a] += s ? 1 : -1;
-            const int na = a == 0 ? g.n0 : g.n1;
-            if (!(nb[a] >= 0 && nb[a] < na && cf_covered(g, nb[0], nb[1]))) continue;
-            const int t = 1 - a, side = s ? 0 : 1;
-            const int fin = side == 0 ? 0 : (a == 0 ? g.m0 : g.m1) - 1;
-            const int ct = t == 0 ? I : J;
-#pragma unroll
-            for (int q = 0; q < 2; q++) {
-                int ff[2];
-                ff[a] = fin;
-                ff[t] = 2 * (ct - g.b0[t]) + q;
-                int fface[2] = {ff[0], ff[1]};
-                fface[a] += side;
-                const long long fid = cf_fface(g, a, fface[0], fface[1]);
-                const double2 d = df[ff[0] + (long long)g.m0 * ff[1]];
-                tT += k.fkf[a][fid] * d.x * g.rbif;
-                tp += k.faf[a][fid] * d.y * g.rbif;
-            }
+        for (int q = 0; q < 2; q++) {
+            const int i = a == 0 ? fin : f0 + q, j = a == 0 ? f0 + q : fin;
+            const long long fid = cf_fface(g, a, i + (a == 0 ? side : 0), j + (a == 1 ? side : 0));
+            const double2 d = df[i + (long long)g.m0 * j];
+            tT += k.fkf[a][fid] * d.x * g.rbif;
+            tp += k.faf[a][fid] * d.y * g.rbif;
         }
+    }
     const double oT = tT, op = tp + k.lamb[4 * c + 3] * tT;
     sb[c] = make_double2(rb[c].x - oT, rb[c].y - op);
 }
@@ -292,54 +341,45 @@ __global__ void __launch_bounds__(256) k_cf_base_rhs(CfGeom g, CfCoef k, const d
 // prolongation (the fine cells' positions in the whole domain; homogeneous
 // ghosts outside it), and out = rf minus what db adds to the patch rows
 // through the interface ghosts (the p-row's l4 div(k grad T) included).
-__global__ void __launch_bounds__(256) k_cf_prolong_ghost(CfGeom g, CfCoef k, const double2 *__restrict__ db,
+__global__ void __launch_bounds__(256) k_cf_prolong_ghost(const __grid_constant__ CfGeom g, const __grid_constant__ CfCoef k, const double2 *__restrict__ db,
                                                           const double2 *__restrict__ rf, double2 *__restrict__ df,
                                                           double2 *__restrict__ out) {
+    pdl_entry();
     const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
     if (i >= g.m0 || j >= g.m1) return;
     const long long c = i + (long long)g.m0 * j;
     const int gi = 2 * g.b0[0] + i, gj = 2 * g.b0[1] + j;
     const int P[2] = {gi / 2, gj / 2};
     const int sg[2] = {(gi & 1) ? 1 : -1, (gj & 1) ? 1 : -1};
+    double2 v[4];
+#pragma unroll
+    for (int q = 0; q < 4; q++) v[q] = cf_base_load(g, db, P[0] + (q & 1 ? sg[0] : 0), P[1] + (q >> 1 ? sg[1] : 0));
     double aT = 0.0, ap = 0.0;
 #pragma unroll
     for (int q = 0; q < 4; q++) {
-        double w = 1.0;
-        int Q[2] = {P[0], P[1]};
-#pragma unroll
-        for (int a = 0; a < 2; a++) {
-            if ((q >> a) & 1) {
-                w *= 0.25;
-                Q[a] += sg[a];
-            } else {
-                w *= 0.75;
-            }
-        }
-        const double2 v = cf_base_value(g, db, Q[0], Q[1]);
-        aT += w * v.x;
-        ap += w * v.y;
+        const double w = (q & 1 ? 0.25 : 0.75) * (q >> 1 ? 0.25 : 0.75);
+        v[q] = cf_base_rule(g, v[q], P[0] + (q & 1 ? sg[0] : 0), P[1] + (q >> 1 ? sg[1] : 0));
+        aT += w * v[q].x;
+        ap += w * v[q].y;
     }
     df[c] = make_double2(df[c].x + aT, df[c].y + ap);
     double gT = 0.0, gp = 0.0;
-    const int pos[2] = {i, j};
-#pragma unroll
-    for (int a = 0; a < 2; a++)
-#pragma unroll
-        for (int s = 0; s < 2; s++) {
-            if (!g.iface[a][s]) continue;
-            const int ma = a == 0 ? g.m0 : g.m1;
-            if ((s == 0 && pos[a] != 0) || (s == 1 && pos[a] != ma - 1)) continue;
-            const long long fid = cf_fface(g, a, i + (a == 0 ? s : 0), j + (a == 1 ? s : 0));
-            const double2 gu = cf_ghost(g, db, a, s, i, j);
-            gT += k.fkf[a][fid] * gu.x * g.rif;
-            gp += k.faf[a][fid] * gu.y * g.rif;
-        }
+#pragma unroll 1
+    for (int left = 15 & ~cf_fine_sides(g, i, j); left; left &= left - 1) {
+        const int bit = __ffs(left) - 1, a = bit >> 1, s = bit & 1;
+        if (!g.iface[a][s]) continue;
+        const long long fid = cf_fface(g, a, i + (a == 0 ? s : 0), j + (a == 1 ? s : 0));
+        const double2 gu = cf_ghost(g, db, a, s, i, j);
+        gT += k.fkf[a][fid] * gu.x * g.rif;
+        gp += k.faf[a][fid] * gu.y * g.rif;
+    }
     out[c] = make_double2(rf[c].x - gT, rf[c].y - (gp + k.lamf[4 * c + 3] * gT));
 }
 
 // x += correction on the valid base cells and the patch.
 __global__ void __launch_bounds__(256) k_cf_update(CfGeom g, double2 *__restrict__ xb, double2 *__restrict__ xf,
                                                    const double2 *__restrict__ db, const double2 *__restrict__ df) {
+    pdl_entry();
     const int I = blockIdx.x * blockDim.x + threadIdx.x, J = blockIdx.y * blockDim.y + threadIdx.y;
     if (I < g.n0 && J < g.n1 && !cf_covered(g, I, J)) {
         const long long c = I + (long long)g.n0 * J;
@@ -354,6 +394,7 @@ __global__ void __launch_bounds__(256) k_cf_update(CfGeom g, double2 *__restrict
 // Covered base cells of xb: the mean of their four children in xf.
 __global__ void __launch_bounds__(256) k_cf_covered_mean(CfGeom g, double2 *__restrict__ xb,
                                                          const double2 *__restrict__ xf) {
+    pdl_entry();
     const int I = blockIdx.x * blockDim.x + threadIdx.x + g.b0[0], J = blockIdx.y * blockDim.y + threadIdx.y + g.b0[1];
     if (I >= g.b1[0] || J >= g.b1[1]) return;
     double s0 = 0.0, s1 = 0.0;
@@ -373,6 +414,7 @@ __global__ void __launch_bounds__(256) k_cf_covered_mean(CfGeom g, double2 *__re
 __global__ void __launch_bounds__(256) k_cf_cover(CfGeom g, CfCoef k, double *__restrict__ lam,
                                                   double *__restrict__ fa0, double *__restrict__ fa1,
                                                   double *__restrict__ fk0, double *__restrict__ fk1) {
+    pdl_entry();
     const int I = blockIdx.x * blockDim.x + threadIdx.x + g.b0[0], J = blockIdx.y * blockDim.y + threadIdx.y + g.b0[1];
     if (I >= g.b1[0] || J >= g.b1[1]) return;
     const long long c = I + (long long)g.n0 * J;
@@ -414,6 +456,7 @@ __global__ void __launch_bounds__(256) k_cf_norms(CfGeom g, const double2 *__res
                                                   const double2 *__restrict__ rf, long long nb, long long nf,
                                                   double *__restrict__ partial, unsigned int *__restrict__ ticket,
                                                   double *__restrict__ out) {
+    pdl_entry();
     __shared__ double sm[4][256];
     __shared__ bool last;
     double a[4] = {0.0, 0.0, 0.0, 0.0};
@@ -452,6 +495,52 @@ __global__ void __launch_bounds__(256) k_cf_norms(CfGeom g, const double2 *__res
 #pragma unroll
         for (int v = 0; v < 4; v++) out[v] = sqrt(s[v]);
         *ticket = 0u;
+    }
+}
+
+// Copies of several arrays in one launch (blockIdx.y: the array; dst2 may be
+// NULL), 16 bytes at a time where the pointers allow.  Sizes are multiples of
+// 8, pointers 8-byte aligned.  The coefficients of a refined grid are 12
+// arrays; as a copy each they took 4 us apiece, bound by the launches (512^2 with
+// a 250^2 patch: 65 us of copies -> 9).
+constexpr int kCopyJobs = 12;
+struct CopyJob {
+    const void *src;
+    void *dst, *dst2;
+    long long bytes;
+};
+struct CopyList {
+    CopyJob job[kCopyJobs];
+    int count;
+};
+
+__global__ void __launch_bounds__(256) k_copy_list(const __grid_constant__ CopyList C) {
+    pdl_entry();
+    const CopyJob &J = C.job[blockIdx.y];
+    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+    if (((reinterpret_cast<unsigned long long>(J.src) | reinterpret_cast<unsigned long long>(J.dst) |
+          reinterpret_cast<unsigned long long>(J.dst2)) & 15) == 0) {
+        const double2 *s = static_cast<const double2 *>(J.src);
+        double2 *d = static_cast<double2 *>(J.dst), *e = static_cast<double2 *>(J.dst2);
+        for (long long q = t; q < J.bytes / 16; q += step) {
+            const double2 v = s[q];
+            d[q] = v;
+            if (e) e[q] = v;
+        }
+        if (t == 0 && (J.bytes & 8)) {
+            const long long q = J.bytes / 8 - 1;
+            const double v = static_cast<const double *>(J.src)[q];
+            static_cast<double *>(J.dst)[q] = v;
+            if (e) static_cast<double *>(J.dst2)[q] = v;
+        }
+        return;
+    }
+    const double *s = static_cast<const double *>(J.src);
+    double *d = static_cast<double *>(J.dst), *e = static_cast<double *>(J.dst2);
+    for (long long q = t; q < J.bytes / 8; q += step) {
+        const double v = s[q];
+        d[q] = v;
+        if (e) e[q] = v;
     }
 }
 

@@ -17,7 +17,7 @@ struct mg_composite {
     // the base hierarchy's coefficients (covered cells from the patch)
     double *clam, *cfa[2], *cfk[2];
     double2 *rb, *rf, *sb, *sf, *df, *zb, *xb, *xf, *bb, *bf;
-    double *partial, *norms_d, *norms_h;
+    double *partial, *norms_h;     // norms_h: page-locked host memory, written by the norm kernel
     unsigned int *ticket;
     int nblk;
     bool coeffs_set;
@@ -43,42 +43,49 @@ dim3 cf_grid2(int nx, int ny) { return dim3((unsigned)((nx + 31) / 32), (unsigne
 
 // (T, p) norms of the current residuals rb, rf into norms_h (after the stream is synchronised)
 void cf_enqueue_norms(mg_composite *m) {
-    k_cf_norms<<<m->nblk, 256, 0, m->stream>>>(m->g, m->rb, m->rf, m->Nb, m->Nf, m->partial, m->ticket, m->norms_d);
-    cudaMemcpyAsync(m->norms_h, m->norms_d, 4 * sizeof(double), cudaMemcpyDeviceToHost, m->stream);
+    launch_k(m->hb, k_cf_norms, m->nblk, 256, 0, m->stream, 0, m->g, m->rb, m->rf, m->Nb, m->Nf, m->partial,
+             m->ticket, m->norms_h);
 }
 
 // The composite residuals r = b - L(x) of the current x.
 void cf_enqueue_residual(mg_composite *m, cudaStream_t s) {
     const CfCoef k = cf_coef(m);
-    k_cf_rows_base<<<cf_grid2(m->g.n0, m->g.n1), dim3(32, 8), 0, s>>>(m->g, k, m->xb, m->xf, m->bb, m->rb);
-    k_cf_rows_fine<<<cf_grid2(m->g.m0, m->g.m1), dim3(32, 8), 0, s>>>(m->g, k, m->xb, m->xf, m->bf, m->rf);
+    launch_k(m->hb, k_cf_rows_base, cf_grid2(m->g.n0, m->g.n1), dim3(32, 8), 0, s, 0, m->g, k, m->xb, m->xf, m->bb,
+             m->rb);
+    launch_k(m->hb, k_cf_rows_fine, cf_grid2(m->g.m0, m->g.m1), dim3(32, 8), 0, s, 0, m->g, k, m->xb, m->xf, m->bf,
+             m->rf);
 }
 
-void cf_enqueue_sweeps(mg_composite *m, cudaStream_t s, const double2 *rhs, int sweeps) {
+// from_zero: the correction df is zero (and need not hold it).
+void cf_enqueue_sweeps(mg_composite *m, cudaStream_t s, const double2 *rhs, int sweeps, bool from_zero) {
     const CfCoef k = cf_coef(m);
     const dim3 gr = cf_grid2((m->g.m0 + 1) / 2, m->g.m1);
     for (int q = 0; q < sweeps; q++)
         for (int colour = 0; colour < 2; colour++)
-            k_cf_rbgs_fine<<<gr, dim3(32, 8), 0, s>>>(m->g0, k, m->zb, rhs, m->df, colour);
+            launch_k(m->hb, k_cf_rbgs_fine, gr, dim3(32, 8), 0, s, 0, m->g0, k, rhs, m->df, colour,
+                     (from_zero && q == 0 && colour == 0) ? 1 : 0);
 }
 
 // One FAC cycle on the residuals rb, rf, x += the correction, and the
 // residuals of the new x.
 mg_status cf_enqueue_fac_cycle(mg_composite *m, cudaStream_t s) {
     const CfCoef k = cf_coef(m);
-    CK(cudaMemsetAsync(m->df, 0, sizeof(double2) * m->Nf, s));
-    cf_enqueue_sweeps(m, s, m->rf, m->opt.nu1);
+    if (m->opt.nu1 == 0) CK(cudaMemsetAsync(m->df, 0, sizeof(double2) * m->Nf, s));
+    cf_enqueue_sweeps(m, s, m->rf, m->opt.nu1, true);
     // the patch residual of the correction (zero base values), then the base right-hand side
-    k_cf_rows_fine<<<cf_grid2(m->g.m0, m->g.m1), dim3(32, 8), 0, s>>>(m->g0, k, m->zb, m->df, m->rf, m->sf);
-    k_cf_base_rhs<<<cf_grid2(m->g.n0, m->g.n1), dim3(32, 8), 0, s>>>(m->g0, k, m->rb, m->df, m->sf, m->sb);
+    launch_k(m->hb, k_cf_rows_fine, cf_grid2(m->g.m0, m->g.m1), dim3(32, 8), 0, s, 0, m->g0, k, m->zb, m->df,
+             m->rf, m->sf);
+    launch_k(m->hb, k_cf_base_rhs, cf_grid2(m->g.n0, m->g.n1), dim3(32, 8), 0, s, 0, m->g0, k, m->rb, m->df, m->sf,
+             m->sb);
     // one V-cycle of the base hierarchy from zero; the result is in its finest level's x
     mg_status st = enqueue_correction<2>(m->hb, s, m->sb);
     if (st) return st;
     const double2 *db = m->hb->L[0].x;
-    k_cf_prolong_ghost<<<cf_grid2(m->g.m0, m->g.m1), dim3(32, 8), 0, s>>>(m->g0, k, db, m->rf, m->df, m->sf);
-    cf_enqueue_sweeps(m, s, m->sf, m->opt.nu2);
+    launch_k(m->hb, k_cf_prolong_ghost, cf_grid2(m->g.m0, m->g.m1), dim3(32, 8), 0, s, 0, m->g0, k, db, m->rf,
+             m->df, m->sf);
+    cf_enqueue_sweeps(m, s, m->sf, m->opt.nu2, false);
     const dim3 ug = cf_grid2(std::max(m->g.n0, m->g.m0), std::max(m->g.n1, m->g.m1));
-    k_cf_update<<<ug, dim3(32, 8), 0, s>>>(m->g, m->xb, m->xf, db, m->df);
+    launch_k(m->hb, k_cf_update, ug, dim3(32, 8), 0, s, 0, m->g, m->xb, m->xf, db, m->df);
     cf_enqueue_residual(m, s);
     CK(cudaGetLastError());
     return MG_OK;
@@ -111,6 +118,32 @@ mg_status cf_capture(mg_composite *m) {
 mg_status cf_check_pair(const double *p) {
     if (!p) return fail(MG_ERR_INVALID_ARG, "NULL array");
     if (!aligned16(p)) return fail(MG_ERR_INVALID_ARG, "pair arrays must be 16-byte aligned");
+    return MG_OK;
+}
+
+// The copies of a list in one kernel where every pointer is this device's own memory and aligned to 8 bytes, else one
+// by one.
+mg_status cf_copies(mg_composite *m, const std::vector<CopyJob> &jobs) {
+    bool ok = true;
+    CopyList C;
+    std::memset(&C, 0, sizeof(C));
+    long long most = 0;
+    for (const CopyJob &j : jobs) {
+        ok = ok && ((reinterpret_cast<uintptr_t>(j.src) | reinterpret_cast<uintptr_t>(j.dst)) & 7) == 0 &&
+             local_device(m->hb, j.src) && local_device(m->hb, j.dst);
+        most = std::max(most, j.bytes);
+        if (C.count < kCopyJobs) C.job[C.count++] = j;
+    }
+    if (ok && (int)jobs.size() <= kCopyJobs) {
+        const unsigned gx = (unsigned)std::min<long long>((most / 16 + 255) / 256 + 1, 152 * 2);
+        launch_k(m->hb, k_copy_list, dim3(gx, (unsigned)C.count), 256, 0, m->stream, 0, C);
+        CK(cudaGetLastError());
+        return MG_OK;
+    }
+    for (const CopyJob &j : jobs) {
+        CK(cudaMemcpyAsync(j.dst, j.src, j.bytes, cudaMemcpyDeviceToDevice, m->stream));
+        if (j.dst2) CK(cudaMemcpyAsync(j.dst2, j.src, j.bytes, cudaMemcpyDeviceToDevice, m->stream));
+    }
     return MG_OK;
 }
 
@@ -209,7 +242,7 @@ mg_status mg_composite_create(const mg_grid *grid, const int box[2][2], const mg
     }
     const size_t o_cfk[2] = {take(8 * m->nfb[0]), take(8 * m->nfb[1])};
     const size_t o_pairs_b = take(16 * m->Nb * 5), o_pairs_f = take(16 * m->Nf * 5);
-    const size_t o_part = take(8 * 4 * (size_t)m->nblk), o_norm = take(8 * 4), o_tick = take(4);
+    const size_t o_part = take(8 * 4 * (size_t)m->nblk), o_tick = take(4);
     if (cudaMalloc(&m->arena, off + 256) != cudaSuccess) {
         cudaGetLastError();
         mg_destroy(m->hb);
@@ -240,7 +273,6 @@ mg_status mg_composite_create(const mg_grid *grid, const int box[2][2], const mg
     m->xf = pf + 3 * m->Nf;
     m->bf = pf + 4 * m->Nf;
     m->partial = reinterpret_cast<double *>(A + o_part);
-    m->norms_d = reinterpret_cast<double *>(A + o_norm);
     m->ticket = reinterpret_cast<unsigned int *>(A + o_tick);
     if (cudaMallocHost(&m->norms_h, 4 * sizeof(double)) != cudaSuccess ||
         cudaMemsetAsync(m->zb, 0, sizeof(double2) * m->Nb, m->stream) != cudaSuccess ||
@@ -262,24 +294,21 @@ mg_status mg_composite_set_coeffs(mg_composite *m, const double *lam_b, const do
         if (!fa_b[a] || !fk_b[a] || !fa_f[a] || !fk_f[a]) return fail(MG_ERR_INVALID_ARG, "NULL face array");
     DeviceGuard dg(m->device);
     cudaStream_t s = m->stream;
-    CK(cudaMemcpyAsync(m->lamb, lam_b, 32 * m->Nb, cudaMemcpyDeviceToDevice, s));
-    CK(cudaMemcpyAsync(m->lamf, lam_f, 32 * m->Nf, cudaMemcpyDeviceToDevice, s));
-    CK(cudaMemcpyAsync(m->clam, lam_b, 32 * m->Nb, cudaMemcpyDeviceToDevice, s));
+    std::vector<CopyJob> jobs = {{lam_b, m->lamb, m->clam, 32 * m->Nb}, {lam_f, m->lamf, nullptr, 32 * m->Nf}};
     for (int a = 0; a < 2; a++) {
-        CK(cudaMemcpyAsync(m->fab[a], fa_b[a], 8 * m->nfb[a], cudaMemcpyDeviceToDevice, s));
-        CK(cudaMemcpyAsync(m->fkb[a], fk_b[a], 8 * m->nfb[a], cudaMemcpyDeviceToDevice, s));
-        CK(cudaMemcpyAsync(m->cfa[a], fa_b[a], 8 * m->nfb[a], cudaMemcpyDeviceToDevice, s));
-        CK(cudaMemcpyAsync(m->cfk[a], fk_b[a], 8 * m->nfb[a], cudaMemcpyDeviceToDevice, s));
-        CK(cudaMemcpyAsync(m->faf[a], fa_f[a], 8 * m->nff[a], cudaMemcpyDeviceToDevice, s));
-        CK(cudaMemcpyAsync(m->fkf[a], fk_f[a], 8 * m->nff[a], cudaMemcpyDeviceToDevice, s));
+        jobs.push_back({fa_b[a], m->fab[a], m->cfa[a], 8 * m->nfb[a]});
+        jobs.push_back({fk_b[a], m->fkb[a], m->cfk[a], 8 * m->nfb[a]});
+        jobs.push_back({fa_f[a], m->faf[a], nullptr, 8 * m->nff[a]});
+        jobs.push_back({fk_f[a], m->fkf[a], nullptr, 8 * m->nff[a]});
     }
+    mg_status st = cf_copies(m, jobs);
+    if (st) return st;
     const int bx = m->g.b1[0] - m->g.b0[0], by = m->g.b1[1] - m->g.b0[1];
-    k_cf_cover<<<cf_grid2(bx, by), dim3(32, 8), 0, s>>>(m->g, cf_coef(m), m->clam, m->cfa[0], m->cfa[1], m->cfk[0],
-                                                        m->cfk[1]);
+    launch_k(m->hb, k_cf_cover, cf_grid2(bx, by), dim3(32, 8), 0, s, 0, m->g, cf_coef(m), m->clam, m->cfa[0],
+             m->cfa[1], m->cfk[0], m->cfk[1]);
     CK(cudaGetLastError());
     const double *pa[3] = {m->cfa[0], m->cfa[1], nullptr}, *pk[3] = {m->cfk[0], m->cfk[1], nullptr};
-    mg_status st = mg_set_coeffs(m->hb, m->clam, pa, pk, 1);
-    if (st) return st;
+    if ((st = mg_set_coeffs(m->hb, m->clam, pa, pk, 1))) return st;
     m->coeffs_set = true;
     return MG_OK;
 }
@@ -293,10 +322,10 @@ mg_status mg_composite_apply(mg_composite *m, const double *xb, const double *xf
     DeviceGuard dg(m->device);
     const CfCoef k = cf_coef(m);
     const double2 *xb2 = reinterpret_cast<const double2 *>(xb), *xf2 = reinterpret_cast<const double2 *>(xf);
-    k_cf_rows_base<<<cf_grid2(m->g.n0, m->g.n1), dim3(32, 8), 0, m->stream>>>(m->g, k, xb2, xf2, nullptr,
-                                                                             reinterpret_cast<double2 *>(yb));
-    k_cf_rows_fine<<<cf_grid2(m->g.m0, m->g.m1), dim3(32, 8), 0, m->stream>>>(m->g, k, xb2, xf2, nullptr,
-                                                                             reinterpret_cast<double2 *>(yf));
+    launch_k(m->hb, k_cf_rows_base, cf_grid2(m->g.n0, m->g.n1), dim3(32, 8), 0, m->stream, 0, m->g, k, xb2, xf2,
+             nullptr, reinterpret_cast<double2 *>(yb));
+    launch_k(m->hb, k_cf_rows_fine, cf_grid2(m->g.m0, m->g.m1), dim3(32, 8), 0, m->stream, 0, m->g, k, xb2, xf2,
+             nullptr, reinterpret_cast<double2 *>(yf));
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(m->stream));
     return MG_OK;
@@ -312,10 +341,9 @@ mg_status mg_composite_solve(mg_composite *m, const double *bb, const double *bf
         return st;
     DeviceGuard dg(m->device);
     cudaStream_t s = m->stream;
-    CK(cudaMemcpyAsync(m->bb, bb, 16 * m->Nb, cudaMemcpyDeviceToDevice, s));
-    CK(cudaMemcpyAsync(m->bf, bf, 16 * m->Nf, cudaMemcpyDeviceToDevice, s));
-    CK(cudaMemcpyAsync(m->xb, xb, 16 * m->Nb, cudaMemcpyDeviceToDevice, s));
-    CK(cudaMemcpyAsync(m->xf, xf, 16 * m->Nf, cudaMemcpyDeviceToDevice, s));
+    if ((st = cf_copies(m, {{bb, m->bb, nullptr, 16 * m->Nb}, {bf, m->bf, nullptr, 16 * m->Nf},
+                            {xb, m->xb, nullptr, 16 * m->Nb}, {xf, m->xf, nullptr, 16 * m->Nf}})))
+        return st;
     if (cycles > 0 && !m->gcyc && (st = cf_capture(m))) return st;
     cf_enqueue_residual(m, s);
     for (int k = 0;; k++) {
@@ -328,10 +356,9 @@ mg_status mg_composite_solve(mg_composite *m, const double *bb, const double *bf
         CK(cudaGraphLaunch(m->gcyc, s));
     }
     const int bx = m->g.b1[0] - m->g.b0[0], by = m->g.b1[1] - m->g.b0[1];
-    k_cf_covered_mean<<<cf_grid2(bx, by), dim3(32, 8), 0, s>>>(m->g, m->xb, m->xf);
+    launch_k(m->hb, k_cf_covered_mean, cf_grid2(bx, by), dim3(32, 8), 0, s, 0, m->g, m->xb, m->xf);
     CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(xb, m->xb, 16 * m->Nb, cudaMemcpyDeviceToDevice, s));
-    CK(cudaMemcpyAsync(xf, m->xf, 16 * m->Nf, cudaMemcpyDeviceToDevice, s));
+    if ((st = cf_copies(m, {{m->xb, xb, nullptr, 16 * m->Nb}, {m->xf, xf, nullptr, 16 * m->Nf}}))) return st;
     CK(cudaStreamWaitEvent(s, m->hb->ev_inv, 0));
     CK(cudaMemcpyAsync(m->hb->errh, m->hb->err_d, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));

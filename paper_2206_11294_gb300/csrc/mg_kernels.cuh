@@ -907,12 +907,12 @@ __device__ __forceinline__ bool on_boundary(const Level<double> &L, int i, int j
     return i == 0 || i == L.n0 - 1 || j == 0 || j == L.n1 - 1 || (DIM == 3 && (k == 0 || k == L.n2 - 1));
 }
 
-// Block (bx, by, bz) of the cell grid; xin (may be NULL) is also copied into L.x.
+// Block (bx, by, bz) of the cell grid; xin (may be NULL) is also copied into L.x, or L.x set to zero.
 // AXI: the rows carry the factor s_i = r_i (else 1, with no arithmetic).
 template <int DIM, bool AXI>
 __device__ __forceinline__ void prep_rhs_cells(const Level<double> &L, const double2 *__restrict__ rhs,
                                                const double2 *__restrict__ xin, const BcVals &bv, double r0,
-                                               double h, int bx, int by, int bz) {
+                                               double h, bool zero, int bx, int by, int bz) {
     const int i = bx * kBX + threadIdx.x;
     const int j = by * kBY + threadIdx.y;
     const int k = DIM == 3 ? bz : 0;
@@ -934,25 +934,26 @@ __device__ __forceinline__ void prep_rhs_cells(const Level<double> &L, const dou
     const dq Di = ldgq(L.Dinv + c);
     L.bt[c] = make_double2(Di.a * bT + Di.b * bp, Di.c * bT + Di.d * bp);
     if (xin) L.x[c] = xin[c];
+    else if (zero) L.x[c] = make_double2(0.0, 0.0);
 }
 
 template <int DIM>
 __device__ __forceinline__ void prep_rhs_block(const Level<double> &L, const double2 *__restrict__ rhs,
                                                const double2 *__restrict__ xin, const BcVals &bv, int axisym,
-                                               double r0, double h, int bx, int by, int bz) {
-    if (axisym) prep_rhs_cells<DIM, true>(L, rhs, xin, bv, r0, h, bx, by, bz);
-    else prep_rhs_cells<DIM, false>(L, rhs, xin, bv, r0, h, bx, by, bz);
+                                               double r0, double h, bool zero, int bx, int by, int bz) {
+    if (axisym) prep_rhs_cells<DIM, true>(L, rhs, xin, bv, r0, h, zero, bx, by, bz);
+    else prep_rhs_cells<DIM, false>(L, rhs, xin, bv, r0, h, zero, bx, by, bz);
 }
 
 template <int DIM>
 __global__ void __launch_bounds__(kBX * kBY) k_prep_rhs(const __grid_constant__ Level<double> L,
                                                       const double2 *__restrict__ rhs, const double2 *__restrict__ xin,
                                                       const __grid_constant__ BcVals bv, int axisym, double r0, double h,
-                                                      int *__restrict__ clear) {
+                                                      int *__restrict__ clear, int zero) {
     pdl_entry();
     if (clear && (blockIdx.x | blockIdx.y | blockIdx.z | threadIdx.x | threadIdx.y) == 0) *clear = 0;
     CMG_TILES(false, (L.n0 + kBX - 1) / kBX, (L.n1 + kBY - 1) / kBY, DIM == 3 ? L.n2 : 1,
-              (prep_rhs_block<DIM>(L, rhs, xin, bv, axisym, r0, h, bx, by, bz)));
+              (prep_rhs_block<DIM>(L, rhs, xin, bv, axisym, r0, h, zero, bx, by, bz)));
 }
 
 // y = L(x) (Eqs. 27-28): offdiag + boundary data + D x is s_i times the rows.
