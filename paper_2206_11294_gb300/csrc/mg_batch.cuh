@@ -87,6 +87,7 @@ template <typename R, int DIM>
 __global__ void __launch_bounds__(kBatchThreads) kb_rbgs_colour(const BLevel *__restrict__ lv,
                                                                 const BState *__restrict__ st,
                                                                 const int2 *__restrict__ tab, int n, int colour) {
+    pdl_entry();
     for (int v = blockIdx.x; v < n; v += gridDim.x) {
         const int2 e = tab[v];
         const BLevel &B = lv[e.x];
@@ -103,6 +104,7 @@ template <typename R, int TX, int TY>
 __global__ void __launch_bounds__(kBatchThreads, sizeof(R) == 4 ? 8 : 4)
     kb_rbgs_fused2d(const BLevel *__restrict__ lv, const BState *__restrict__ st, const int2 *__restrict__ tab, int n,
                     int to_alt) {
+    pdl_entry();
     for (int v = blockIdx.x; v < n; v += gridDim.x) {
         const int2 e = tab[v];
         const BLevel &B = lv[e.x];
@@ -120,6 +122,7 @@ template <typename R, int DIM>
 __global__ void __launch_bounds__(kBatchThreads) kb_restrict(const BLevel *__restrict__ lv,
                                                              const BState *__restrict__ st,
                                                              const int2 *__restrict__ tab, int n, int red) {
+    pdl_entry();
     for (int v = blockIdx.x; v < n; v += gridDim.x) {
         const int2 e = tab[v];
         const BLevel &B = lv[e.x];
@@ -139,6 +142,7 @@ template <typename R, int DIM, bool BLACK>
 __global__ void __launch_bounds__(kBatchThreads) kb_prolong(const BLevel *__restrict__ lv,
                                                             const BState *__restrict__ st,
                                                             const int2 *__restrict__ tab, int n) {
+    pdl_entry();
     for (int v = blockIdx.x; v < n; v += gridDim.x) {
         const int2 e = tab[v];
         const BLevel &B = lv[e.x];
@@ -159,6 +163,7 @@ __global__ void __launch_bounds__(kBatchThreads) kb_coarse(const BLevel *__restr
                                                            const BProb *__restrict__ pr,
                                                            const BState *__restrict__ st,
                                                            const int2 *__restrict__ tab, int n) {
+    pdl_entry();
     for (int v = blockIdx.x; v < n; v += gridDim.x) {
         const int2 e = tab[v];
         if (!st[e.x].active) continue;
@@ -223,6 +228,7 @@ template <int DIM>
 __global__ void __launch_bounds__(kBatchThreads) kb_setup_fine(const BSetupLevel *__restrict__ sl,
                                                                const SetupIn *__restrict__ in,
                                                                const int2 *__restrict__ tab, int n) {
+    pdl_entry();
     for (int v = blockIdx.x; v < n; v += gridDim.x) {
         const int2 e = tab[v];
         const BSetupLevel &L = sl[e.x];
@@ -238,6 +244,7 @@ template <int DIM, bool ONE>
 __global__ void __launch_bounds__(kBatchThreads) kb_setup_coarse(const BSetupLevel *__restrict__ sl,
                                                                  const SetupIn *__restrict__ in,
                                                                  const int2 *__restrict__ tab, int n) {
+    pdl_entry();
     ChainTile<DIM> *T = nullptr;
     if constexpr (!ONE) {
         __shared__ ChainTile<DIM> tile;
@@ -303,6 +310,7 @@ __global__ void kb_transpose_big(const BCoarse *__restrict__ co, const int *__re
 
 template <int DIM>
 __global__ void __launch_bounds__(kBatchThreads) kb_coarse_assemble(const BCoarse *__restrict__ co, int count) {
+    pdl_entry();
     for (int p = blockIdx.y; p < count; p += gridDim.y) {
         const BCoarse &C = co[p];
         coarse_rows<DIM>(C.n, C.G0, C.G1, C.G2, C.D, C.l4, C.M, blockIdx.x, gridDim.x);
@@ -366,6 +374,7 @@ __global__ void __launch_bounds__(32 * kInvRows) kb_band_inv_cols_warp(const BCo
 template <int DIM>
 __global__ void __launch_bounds__(kBatchThreads) kb_prep(const BLevel *__restrict__ lv, const BIo *__restrict__ io,
                                                          const int2 *__restrict__ tab, int n) {
+    pdl_entry();
     for (int v = blockIdx.x; v < n; v += gridDim.x) {
         const int2 e = tab[v];
         const BLevel &B = lv[e.x];
@@ -394,15 +403,24 @@ __global__ void kb_gather_err(const BCoarse *__restrict__ co, int count, int *__
     }
 }
 
-// Results of all problems to the callers' device arrays.
-__global__ void __launch_bounds__(kBatchThreads) kb_copy_out(const BLevel *__restrict__ lv, const BIo *__restrict__ io,
-                                                             const int2 *__restrict__ tab, int n) {
+// Results of all problems: x, plus delta in mixed precision, into the callers' device arrays, or (xout NULL) in place.
+template <bool DELTA>
+__global__ void __launch_bounds__(kBatchThreads) kb_solution_out(const BLevel *__restrict__ lv,
+                                                                 const BIo *__restrict__ io,
+                                                                 const int2 *__restrict__ tab, int n) {
+    pdl_entry();
     for (int v = blockIdx.x; v < n; v += gridDim.x) {
         const int2 e = tab[v];
         const BLevel &B = lv[e.x];
         double2 *dst = io[B.problem].xout;
         const long long c = (long long)e.y * kBatchThreads + threadIdx.x;
-        if (dst && c < B.d.N) dst[c] = B.d.x[c];
+        if (c >= B.d.N || !(DELTA || dst)) continue;
+        double2 a = B.d.x[c];
+        if (DELTA) {
+            const double2 d = B.delta[c];
+            a = make_double2(a.x + d.x, a.y + d.y);
+        }
+        (dst ? dst : B.d.x)[c] = a;
     }
 }
 
@@ -417,9 +435,10 @@ __device__ __forceinline__ bool batch_converged(const double n0[2], const double
 
 // After a block stored its partial: the problem's last block sums them (in
 // order), updates that problem's state with mg_solve's stopping rule and
-// counts it in active_count if it continues.
+// leaves a copy in page-locked host memory, where the host counts the problems
+// that continue (a counter with its memset and copy nodes cost 9 us a cycle).
 __device__ __forceinline__ void batch_finish(const BProb &P, BState &S, int local, double2 s, int initial,
-                                             double rtol, int max_cycles, int *active_count) {
+                                             double rtol, int max_cycles, BState *host) {
     __shared__ bool last;
     const int tid = threadIdx.x + blockDim.x * threadIdx.y;
     const int nthr = blockDim.x * blockDim.y;
@@ -456,7 +475,7 @@ __device__ __forceinline__ void batch_finish(const BProb &P, BState &S, int loca
             const bool ok = batch_converged(S.n0, nk, rtol);
             S.active = (!ok && S.cycles < max_cycles) ? 1 : 0;
         }
-        atomicAdd(active_count, S.active);
+        *host = S;
     }
 }
 
@@ -465,7 +484,8 @@ template <int DIM>
 __global__ void __launch_bounds__(kBatchThreads) kb_norm(const BLevel *__restrict__ lv, const BProb *__restrict__ pr,
                                                          BState *__restrict__ st, const int2 *__restrict__ tab, int n,
                                                          int initial, int red, double rtol, int max_cycles,
-                                                         int *__restrict__ active_count) {
+                                                         BState *__restrict__ host) {
+    pdl_entry();
     for (int v = blockIdx.x; v < n; v += gridDim.x) {
         __syncthreads();
         const int2 e = tab[v];
@@ -477,7 +497,7 @@ __global__ void __launch_bounds__(kBatchThreads) kb_norm(const BLevel *__restric
         block_coords(e.y, norm_gx(L.n0), norm_gy(L.n1, kBatchNormRows), bx, by, bz);
         const double2 s = (red && !initial) ? norm_block<DIM, true, kBatchNormRows>(L, bx, by, bz)
                                                : norm_block<DIM, false, kBatchNormRows>(L, bx, by, bz);
-        batch_finish(pr[p], st[p], e.y, s, initial, rtol, max_cycles, active_count);
+        batch_finish(pr[p], st[p], e.y, s, initial, rtol, max_cycles, host + p);
     }
 }
 
@@ -487,7 +507,8 @@ __global__ void __launch_bounds__(kBatchThreads) kb_residual64(const BLevel *__r
                                                                const BProb *__restrict__ pr, BState *__restrict__ st,
                                                                const int2 *__restrict__ tab, int n, int initial,
                                                                int red_start, double rtol, int max_cycles,
-                                                               int *__restrict__ active_count) {
+                                                               BState *__restrict__ host) {
+    pdl_entry();
     for (int v = blockIdx.x; v < n; v += gridDim.x) {
         __syncthreads();
         const int2 e = tab[v];
@@ -502,20 +523,7 @@ __global__ void __launch_bounds__(kBatchThreads) kb_residual64(const BLevel *__r
         if (!initial) L.x = B.delta;
         const double2 s = residual64_to32_block<DIM, kBatchNormRows>(L, B.f.b, B.f.bt, B.f.x, initial ? L.b : nullptr,
                                                      initial ? B.delta : nullptr, red_start, bx, by, bz);
-        batch_finish(pr[p], st[p], e.y, s, initial, rtol, max_cycles, active_count);
-    }
-}
-
-// Mixed precision, at the end: x = x0 + delta.
-__global__ void __launch_bounds__(kBatchThreads) kb_finish_correction(const BLevel *__restrict__ lv,
-                                                                      const int2 *__restrict__ tab, int n) {
-    for (int v = blockIdx.x; v < n; v += gridDim.x) {
-        const int2 e = tab[v];
-        const BLevel &B = lv[e.x];
-        const long long c = (long long)e.y * kBatchThreads + threadIdx.x;
-        if (c >= B.d.N) continue;
-        const double2 a = B.d.x[c], d = B.delta[c];
-        B.d.x[c] = make_double2(a.x + d.x, a.y + d.y);
+        batch_finish(pr[p], st[p], e.y, s, initial, rtol, max_cycles, host + p);
     }
 }
 
@@ -523,6 +531,7 @@ __global__ void __launch_bounds__(kBatchThreads) kb_finish_correction(const BLev
 __global__ void __launch_bounds__(kBatchThreads) kb_add_correction(const BLevel *__restrict__ lv,
                                                                    const BState *__restrict__ st,
                                                                    const int2 *__restrict__ tab, int n) {
+    pdl_entry();
     for (int v = blockIdx.x; v < n; v += gridDim.x) {
         const int2 e = tab[v];
         const BLevel &B = lv[e.x];
@@ -552,8 +561,7 @@ struct mg_batch {
     BLevel *lv;
     BProb *pr;
     BState *st;
-    int *active_count;
-    int *active_h;                    // pinned
+    BState *state_h;                  // pinned: each problem's last state, written by the kernels
     int2 *tabs;
     // table slices: {offset, count}
     std::vector<std::pair<long long, int>> colour, restr, prolong;
@@ -606,8 +614,8 @@ template <typename R, int TX, int TY>
 void b_fused_pair(mg_batch *b, cudaStream_t s, int d, int t) {
     const int2 *ft = b->tabs + b->fusedt[t][d].first;
     const int nf = b->fusedt[t][d].second;
-    kb_rbgs_fused2d<R, TX, TY><<<batch_grid(b, nf), kBlock, 0, s>>>(b->lv, b->st, ft, nf, 1);
-    kb_rbgs_fused2d<R, TX, TY><<<batch_grid(b, nf), kBlock, 0, s>>>(b->lv, b->st, ft, nf, 0);
+    launch_k(b->h[0], kb_rbgs_fused2d<R, TX, TY>, batch_grid(b, nf), kBlock, 0, s, 0, b->lv, b->st, ft, nf, 1);
+    launch_k(b->h[0], kb_rbgs_fused2d<R, TX, TY>, batch_grid(b, nf), kBlock, 0, s, 0, b->lv, b->st, ft, nf, 0);
 }
 
 // red_done: the guess is zero with the first red half-sweep applied (enqueue_sweeps).
@@ -627,7 +635,8 @@ void b_smooth(mg_batch *b, cudaStream_t s, int d, int sweeps, bool red_done = fa
     }
     for (; q < sweeps; q++)
         for (int colour = red_done && q == 0 ? 1 : 0; colour < 2; colour++) {
-            kb_rbgs_colour<R, DIM><<<batch_grid(b, nc), kBlock, 0, s>>>(b->lv, b->st, ct, nc, colour);
+            launch_k(b->h[0], kb_rbgs_colour<R, DIM>, batch_grid(b, nc), kBlock, 0, s, 0, b->lv, b->st, ct, nc,
+                     colour);
             b->launches++;
         }
 }
@@ -639,13 +648,14 @@ void b_vcycle(mg_batch *b, cudaStream_t s, bool red_done = false) {
         if (b->colour[d].second == 0) continue;
         b_smooth<R, DIM>(b, s, d, b->opt.nu1, d > 0 || red_done);
         const int nr = b->restr[d].second;
-        kb_restrict<R, DIM><<<batch_grid(b, nr), kBlock, 0, s>>>(b->lv, b->st, b->tabs + b->restr[d].first, nr,
-                                                              b->opt.nu1 > 0);
+        launch_k(b->h[0], kb_restrict<R, DIM>, batch_grid(b, nr), kBlock, 0, s, 0, b->lv, b->st,
+                 b->tabs + b->restr[d].first, nr, b->opt.nu1 > 0);
         b->launches++;
     }
     const int ncs = b->coarse.second;
     if (ncs > 0) {
-        kb_coarse<R><<<batch_grid(b, ncs), kBatchThreads, 0, s>>>(b->lv, b->pr, b->st, b->tabs + b->coarse.first, ncs);
+        launch_k(b->h[0], kb_coarse<R>, batch_grid(b, ncs), kBatchThreads, 0, s, 0, b->lv, b->pr, b->st,
+                 b->tabs + b->coarse.first, ncs);
         b->launches++;
     }
     if (b->win_factors) {
@@ -657,10 +667,12 @@ void b_vcycle(mg_batch *b, cudaStream_t s, bool red_done = false) {
         if (b->colour[d].second == 0) continue;
         if (b->opt.nu2 > 0) {
             const int np = b->colour[d].second;
-            kb_prolong<R, DIM, true><<<batch_grid(b, np), kBlock, 0, s>>>(b->lv, b->st, b->tabs + b->colour[d].first, np);
+            launch_k(b->h[0], kb_prolong<R, DIM, true>, batch_grid(b, np), kBlock, 0, s, 0, b->lv, b->st,
+                     b->tabs + b->colour[d].first, np);
         } else {
             const int np = b->prolong[d].second;
-            kb_prolong<R, DIM, false><<<batch_grid(b, np), kBlock, 0, s>>>(b->lv, b->st, b->tabs + b->prolong[d].first, np);
+            launch_k(b->h[0], kb_prolong<R, DIM, false>, batch_grid(b, np), kBlock, 0, s, 0, b->lv, b->st,
+                     b->tabs + b->prolong[d].first, np);
         }
         b->launches++;
         b_smooth<R, DIM>(b, s, d, b->opt.nu2);
@@ -669,18 +681,14 @@ void b_vcycle(mg_batch *b, cudaStream_t s, bool red_done = false) {
 
 template <int DIM>
 void b_norm(mg_batch *b, cudaStream_t s, int initial) {
-    cudaMemsetAsync(b->active_count, 0, sizeof(int), s);
     const int n = b->norm.second;
     if (b->opt.precision == MG_FP64)
-        kb_norm<DIM><<<batch_grid(b, n), kBlock, 0, s>>>(b->lv, b->pr, b->st, b->tabs + b->norm.first, n, initial,
-                                                      b->opt.nu2 > 0, b->opt.rtol, b->opt.max_cycles,
-                                                      b->active_count);
+        launch_k(b->h[0], kb_norm<DIM>, batch_grid(b, n), kBlock, 0, s, 0, b->lv, b->pr, b->st,
+                 b->tabs + b->norm.first, n, initial, b->opt.nu2 > 0, b->opt.rtol, b->opt.max_cycles, b->state_h);
     else
-        kb_residual64<DIM><<<batch_grid(b, n), kBlock, 0, s>>>(b->lv, b->pr, b->st, b->tabs + b->norm.first, n, initial,
-                                                            b->opt.nu1 > 0, b->opt.rtol, b->opt.max_cycles,
-                                                            b->active_count);
+        launch_k(b->h[0], kb_residual64<DIM>, batch_grid(b, n), kBlock, 0, s, 0, b->lv, b->pr, b->st,
+                 b->tabs + b->norm.first, n, initial, b->opt.nu1 > 0, b->opt.rtol, b->opt.max_cycles, b->state_h);
     b->launches++;
-    cudaMemcpyAsync(b->active_h, b->active_count, sizeof(int), cudaMemcpyDeviceToHost, s);
 }
 
 // Captures body on the first handle's private stream and times the graph on
@@ -781,7 +789,8 @@ void b_step(mg_batch *b, cudaStream_t s) {
     } else {
         for (int q = 0; q < b->opt.inner_cycles; q++) b_vcycle<float, DIM>(b, s, q == 0);
         const int n = b->cells0.second;
-        kb_add_correction<<<batch_grid(b, n), kBatchThreads, 0, s>>>(b->lv, b->st, b->tabs + b->cells0.first, n);
+        launch_k(b->h[0], kb_add_correction, batch_grid(b, n), kBatchThreads, 0, s, 0, b->lv, b->st,
+                 b->tabs + b->cells0.first, n);
         b->launches++;
     }
     b_norm<DIM>(b, s, 0);
@@ -1022,7 +1031,7 @@ mg_status mg_batch_create(int count, mg_handle *const *handles, mg_batch **out) 
         return o;
     };
     const size_t o_lv = take(sizeof(BLevel) * lv.size()), o_pr = take(sizeof(BProb) * count),
-                 o_st = take(sizeof(BState) * count), o_ac = take(sizeof(int)),
+                 o_st = take(sizeof(BState) * count),
                  o_tab = take(sizeof(int2) * std::max<size_t>(1, tabs.size())),
                  o_sl = take(sizeof(BSetupLevel) * sl.size()), o_sin = take(sizeof(SetupIn) * count),
                  o_co = take(sizeof(BCoarse) * count), o_io = take(sizeof(BIo) * count),
@@ -1038,7 +1047,6 @@ mg_status mg_batch_create(int count, mg_handle *const *handles, mg_batch **out) 
     b->lv = reinterpret_cast<BLevel *>(b->mem + o_lv);
     b->pr = reinterpret_cast<BProb *>(b->mem + o_pr);
     b->st = reinterpret_cast<BState *>(b->mem + o_st);
-    b->active_count = reinterpret_cast<int *>(b->mem + o_ac);
     b->tabs = reinterpret_cast<int2 *>(b->mem + o_tab);
     b->sl = reinterpret_cast<BSetupLevel *>(b->mem + o_sl);
     b->sin = reinterpret_cast<SetupIn *>(b->mem + o_sin);
@@ -1063,7 +1071,7 @@ mg_status mg_batch_create(int count, mg_handle *const *handles, mg_batch **out) 
         cudaMemset(b->st, 0, sizeof(BState) * count) != cudaSuccess ||
         cudaMallocHost(&b->host_io, std::max(sizeof(SetupIn), sizeof(BIo)) * count) != cudaSuccess ||
         cudaMallocHost(&b->err_h, sizeof(int) * 2 * count) != cudaSuccess ||
-        cudaMallocHost(&b->active_h, sizeof(int)) != cudaSuccess) {
+        cudaMallocHost(&b->state_h, sizeof(BState) * count) != cudaSuccess) {
         cudaGetLastError();
         mg_batch_destroy(b);
         return fail(MG_ERR_CUDA, "batch table upload failed");
@@ -1107,8 +1115,10 @@ mg_status mg_batch_solve(mg_batch *b, const double *const *rhs, double *const *x
         }
         CK(cudaMemcpyAsync(b->io, io, sizeof(BIo) * b->count, cudaMemcpyHostToDevice, s));
         const int n = b->cells0g.second;
-        if (b->dim == 2) kb_prep<2><<<batch_grid(b, n), kBlock, 0, s>>>(b->lv, b->io, b->tabs + b->cells0g.first, n);
-        else kb_prep<3><<<batch_grid(b, n), kBlock, 0, s>>>(b->lv, b->io, b->tabs + b->cells0g.first, n);
+        if (b->dim == 2) launch_k(b->h[0], kb_prep<2>, batch_grid(b, n), kBlock, 0, s, 0, b->lv, b->io,
+                                  b->tabs + b->cells0g.first, n);
+        else launch_k(b->h[0], kb_prep<3>, batch_grid(b, n), kBlock, 0, s, 0, b->lv, b->io,
+                      b->tabs + b->cells0g.first, n);
         b->launches++;
         CK(cudaGetLastError());
     }
@@ -1116,9 +1126,10 @@ mg_status mg_batch_solve(mg_batch *b, const double *const *rhs, double *const *x
     else b_norm<3>(b, s, 1);
     const bool mixed = b->opt.precision == MG_MIXED;
     CK(cudaGetLastError());
-    CK(cudaStreamSynchronize(s));
-    int active = *b->active_h;
-    if (active > 0 && !b->graph) {
+    // The first cycle is launched before the initial norms are read (its kernels pass over a problem that met the stop
+    // test at the start), so one host wait serves both.
+    const bool ahead = b->opt.max_cycles >= 1 && b->opt.rtol < 1.0;
+    auto capture_step = [&]() -> mg_status {
         cudaGraph_t graph = nullptr;
         // capture on the first handle's private stream
         cudaStream_t cs = b->h[0]->cap;
@@ -1138,38 +1149,49 @@ mg_status mg_batch_solve(mg_batch *b, const double *const *rhs, double *const *x
         e = cudaGraphInstantiate(&b->graph, graph, 0);
         cudaGraphDestroy(graph);
         if (e != cudaSuccess) return fail(MG_ERR_CUDA, std::string("batch graph: ") + cudaGetErrorString(e));
-    }
-    int steps = 0;
-    while (active > 0 && steps <= b->opt.max_cycles) {
+        return MG_OK;
+    };
+    auto active = [&]() {
+        int n = 0;
+        for (int p = 0; p < b->count; p++) n += b->state_h[p].active;
+        return n;
+    };
+    auto step = [&]() -> mg_status {
+        mg_status e = MG_OK;
+        if (!b->graph && (e = capture_step())) return e;
         CK(cudaGraphLaunch(b->graph, s));
         b->launches += b->graph_kernels;
+        return MG_OK;
+    };
+    mg_status se;
+    int steps = 0;
+    if (ahead) {
+        if ((se = step())) return se;
+        steps = 1;
+    }
+    CK(cudaStreamSynchronize(s));
+    while (active() > 0 && steps <= b->opt.max_cycles) {
+        if ((se = step())) return se;
         CK(cudaStreamSynchronize(s));
-        active = *b->active_h;
         steps++;
     }
-    if (mixed) {
+    if (mixed || on_device) {
         const int n = b->cells0.second;
-        kb_finish_correction<<<batch_grid(b, n), kBatchThreads, 0, s>>>(b->lv, b->tabs + b->cells0.first, n);
-        b->launches++;
-    }
-    std::vector<BState> host(b->count);
-    CK(cudaMemcpyAsync(host.data(), b->st, sizeof(BState) * b->count, cudaMemcpyDeviceToHost, s));
-    if (on_device) {
-        const int n = b->cells0.second;
-        kb_copy_out<<<batch_grid(b, n), kBatchThreads, 0, s>>>(b->lv, b->io, b->tabs + b->cells0.first, n);
+        launch_k(b->h[0], mixed ? kb_solution_out<true> : kb_solution_out<false>, batch_grid(b, n), kBatchThreads,
+                 0, s, 0, b->lv, b->io, b->tabs + b->cells0.first, n);
         b->launches++;
         CK(cudaGetLastError());
-    } else {
+    }
+    if (!on_device)
         for (int p = 0; p < b->count; p++) {
             mg_status st = x_out(b->h[p], x[p], 0);
             if (st) return st;
         }
-    }
     CK(cudaStreamSynchronize(s));
     const double secs = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     bool all_ok = true;
     for (int p = 0; p < b->count; p++) {
-        const BState &S = host[p];
+        const BState &S = b->state_h[p];
         const mg_handle *h = b->h[p];
         const bool zero = S.n0[0] == 0.0 && S.n0[1] == 0.0;
         bool ok = zero || !(h->opt.rtol > 0.0) || converged(S.n0, S.nk, h->opt.rtol);
@@ -1237,20 +1259,24 @@ mg_status mg_batch_set_coeffs(mg_batch *b, const double *const *lambda, const do
     CK(cudaMemcpyAsync(b->sin, in, sizeof(SetupIn) * b->count, cudaMemcpyHostToDevice, s));
     kb_zero_err<<<(b->count + 255) / 256, 256, 0, s>>>(b->co, b->count);
     const int nf = b->setup_fine_tab.second;
-    if (dim == 2) kb_setup_fine<2><<<batch_grid(b, nf), kBlock, 0, s>>>(b->sl, b->sin, b->tabs + b->setup_fine_tab.first, nf);
-    else kb_setup_fine<3><<<batch_grid(b, nf), kBlock, 0, s>>>(b->sl, b->sin, b->tabs + b->setup_fine_tab.first, nf);
+    if (dim == 2) launch_k(b->h[0], kb_setup_fine<2>, batch_grid(b, nf), kBlock, 0, s, 0, b->sl, b->sin,
+                           b->tabs + b->setup_fine_tab.first, nf);
+    else launch_k(b->h[0], kb_setup_fine<3>, batch_grid(b, nf), kBlock, 0, s, 0, b->sl, b->sin,
+                  b->tabs + b->setup_fine_tab.first, nf);
     b->launches += 2;
     for (size_t d = 0; d < b->setup_tab.size(); d++) {
         const int n = b->setup_tab[d].second;
         if (n == 0) continue;
-        auto run = [&](auto kern) { kern<<<batch_grid(b, n), kBlock, 0, s>>>(b->sl, b->sin, b->tabs + b->setup_tab[d].first, n); };
+        auto run = [&](auto kern) {
+            launch_k(b->h[0], kern, batch_grid(b, n), kBlock, 0, s, 0, b->sl, b->sin, b->tabs + b->setup_tab[d].first, n);
+        };
         if (dim == 2) run(b->setup_one[d] ? kb_setup_coarse<2, true> : kb_setup_coarse<2, false>);
         else run(b->setup_one[d] ? kb_setup_coarse<3, true> : kb_setup_coarse<3, false>);
         b->launches++;
     }
     const unsigned gy = (unsigned)std::min(b->count, 65535);
-    if (dim == 2) kb_coarse_assemble<2><<<dim3(16, gy), kBatchThreads, 0, s>>>(b->co, b->count);
-    else kb_coarse_assemble<3><<<dim3(16, gy), kBatchThreads, 0, s>>>(b->co, b->count);
+    if (dim == 2) launch_k(b->h[0], kb_coarse_assemble<2>, dim3(16, gy), kBatchThreads, 0, s, 0, b->co, b->count);
+    else launch_k(b->h[0], kb_coarse_assemble<3>, dim3(16, gy), kBatchThreads, 0, s, 0, b->co, b->count);
     b->launches++;
     if (b->n_inv_smem > 0) {
         CK(launch_clusters(kb_coarse_invert, s, 1, b->n_inv_smem, kGjThreads, gj_smem(b->max_nc_small),
@@ -1416,7 +1442,7 @@ mg_status mg_batch_destroy(mg_batch *b) {
     DeviceGuard dg(b->device);
     if (b->stream) cudaStreamSynchronize(b->stream);
     if (b->graph) cudaGraphExecDestroy(b->graph);
-    if (b->active_h) cudaFreeHost(b->active_h);
+    if (b->state_h) cudaFreeHost(b->state_h);
     if (b->host_io) cudaFreeHost(b->host_io);
     if (b->err_h) cudaFreeHost(b->err_h);
     if (b->mem) cudaFree(b->mem);

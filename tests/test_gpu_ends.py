@@ -36,3 +36,33 @@ def test_device_host_and_async_ends_agree(n, precision):
         assert pick(sd) == pick(sh) == pick(sa)
         r = s.residual_norms(b, xa)
         assert np.array_equal(r, s.residual_norms(p.b, xh)) and torch.equal(x, xa)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("max_cycles,rtol", [(0, 1e-7), (1, 1e-7), (12, 1e-7), (12, 1.0), (3, 0.0)])
+def test_batch_ends_agree(max_cycles, rtol, precision):
+    """The first cycle runs ahead of the initial norms: problems that met the test at the start are left as they were."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2206_11294_gb300.binding import Batch, Solver
+    bc = ((I.BC_WALL, I.BC_DIRICHLET), (I.BC_DIRICHLET, I.BC_WALL), (0, 0))
+    problems = [I.random_coeff_problem(I.Grid(dim=2, axisym=0, n=n, h=1e-2, bc=bc, bcT=((300.0, 301.0),) * 3,
+                                              bcp=((1e5, 1.1e5),) * 3), seed=sum(n))
+                for n in ((33, 9, 1), (40, 24, 1), (8, 4, 1))]
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    solvers = [Solver(p.grid, precision=precision, rtol=rtol, max_cycles=max_cycles) for p in problems]
+    batch = Batch(solvers)
+    batch.set_coeffs([p.lam for p in problems], [p.fa for p in problems], [p.fk for p in problems])
+    xd, xh = [dev(p.x0) for p in problems], [np.array(p.x0, order="C") for p in problems]
+    sd = batch.solve([dev(p.b) for p in problems], xd, allow_not_converged=True)
+    sh = batch.solve([p.b for p in problems], xh, allow_not_converged=True)
+    for p, a, h, d, e in zip(problems, xd, xh, sd, sh):
+        assert np.array_equal(a.cpu().numpy(), h)
+        assert [d[k] for k in ("cycles", "r0", "rfinal")] == [e[k] for k in ("cycles", "r0", "rfinal")]
+        want = 0 if max_cycles == 0 or rtol >= 1.0 else max_cycles if rtol <= 0.0 else None
+        assert want is None or d["outer"] == want, d
+        assert (d["outer"] > 0) == (not np.array_equal(h.reshape(-1), np.asarray(p.x0).reshape(-1)))
+    batch.close()
+    for s in solvers:
+        s.close()
