@@ -102,12 +102,14 @@ typedef struct {
                             about two cells changes the coefficients by up to ~5x per cell there).  Ignored in
                             FP64. */
     int coarse_solve;    /* The exact coarsest solve (Sec. 3 names a direct solve there).  Both factor the
-                            coarsest matrix once per mg_set_coeffs (banded LU with partial pivoting, FP64).
+                            coarsest matrix once per mg_set_coeffs, in FP64.
                             MG_COARSE_AUTO (default): coarsest systems above 128 unknowns (odd grid factors of 9
-                            or more, e.g. 31 x 31 cells for n = 992) keep the factors and each cycle runs the two
-                            triangular solves, one warp, 2n dependent steps; smaller ones form the inverse and
-                            each cycle multiplies by it.  MG_COARSE_INVERSE: always form the inverse (its n^2
-                            (kl + ku) set-up work pays back only over many cycles).  A hierarchy that solves
+                            or more, e.g. 31 x 31 cells for n = 992) keep the factors of a block cyclic reduction
+                            along the longest axis (where a check of the factors fails, of a banded LU with
+                            partial pivoting) and each cycle solves from them; smaller ones form the inverse and
+                            each cycle multiplies by it.  MG_COARSE_INVERSE: always form the inverse (above 128
+                            unknowns from the banded LU; its n^2 (kl + ku) set-up work pays back only over many
+                            cycles).  A hierarchy that solves
                             from the factors runs without the V-cycle tail kernel (mg_tuning.tail_level must be
                             >= levels).  Batches need one value for all their handles. */
 } mg_options;

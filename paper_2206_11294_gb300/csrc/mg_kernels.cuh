@@ -2278,14 +2278,15 @@ __global__ void __launch_bounds__(256) k_band_inv_block(const double *__restrict
 }
 
 // ---------------------------------------------------------------------------
-// The coarsest solve from the factors (mg_options.coarse_solve AUTO on the
-// windowed path): x = U^-1 L^-1 P b with the factors k_band_lu_window leaves
+// The coarsest solve from the factors of the banded LU (mg_options.coarse_solve
+// AUTO where the reduction's check failed; see mg_coarse.cuh, whose solve kernel
+// calls it): x = U^-1 L^-1 P b with the factors k_band_lu_window leaves
 // (Lb, piv; Uc with each column scaled by its reciprocal pivot, see
-// k_scale_uc), one block of kLuSolveThreads per system, in FP64 whatever R
+// k_scale_uc), one block per system, in FP64 whatever R
 // is.  The steps are those of one column of k_band_inv_block with b in place
 // of e_j: the row swaps and multipliers in the order the factorisation
 // applied them, then U from the last row up.  A step's multiply-adds are
-// spread over the block's four warps, one per SM sub-partition: GB300's FP64
+// spread over the block's warps and so over the SM's sub-partitions: GB300's FP64
 // pipe issues a warp's FMA over many cycles, so one warp would take four
 // times as long per step.  One barrier per step, two for a forward step that
 // swaps rows: every thread reads the pivot row's value itself (and, for a
@@ -2299,9 +2300,8 @@ __global__ void __launch_bounds__(256) k_band_inv_block(const double *__restrict
 // the solve) x is set to 0.
 // ---------------------------------------------------------------------------
 constexpr int kLuSolveRows = 16;
-constexpr int kLuSolveThreads = 128;
 
-// Shared memory of k_coarse_lu (bytes): y, then two chunks each of Lb rows,
+// Shared memory of that solve (bytes): y, then two chunks each of Lb rows,
 // Uc rows and piv.
 inline long long coarse_lu_smem(int n, int kl, int ku) {
     const long long C = kl + ku + 1;
