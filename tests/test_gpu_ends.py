@@ -66,3 +66,33 @@ def test_batch_ends_agree(max_cycles, rtol, precision):
     batch.close()
     for s in solvers:
         s.close()
+
+
+def test_arrays_of_the_wrong_kind_are_refused_as_before():
+    """One look at plain CUDA tensors; anything else goes the general way and raises there."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2206_11294_gb300.binding import Batch, Solver
+    g = I.Grid(dim=2, axisym=0, n=(8, 4, 1), h=1e-2, bc=((I.BC_WALL, I.BC_WALL),) * 2 + ((0, 0),))
+    p = I.random_coeff_problem(g, seed=3)
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    s = Solver(g, rtol=0.0, max_cycles=1)
+    batch = Batch([s])
+    lam, fa, fk, b, x = dev(p.lam), [dev(f) for f in p.fa], [dev(f) for f in p.fk], dev(p.b), dev(p.x0)
+    wide = torch.zeros(2 * b.numel(), dtype=torch.float64, device="cuda")
+    for bad, error in ((b.reshape(-1)[:-2], ValueError), (b.float(), TypeError), (wide[::2], TypeError),
+                       (b.cpu(), TypeError)):
+        s.set_coeffs(lam, fa, fk)
+        for call in (lambda: s.solve(bad, x), lambda: batch.solve([bad], [x])):
+            with pytest.raises(error):
+                call()
+    for bad, error in ((fa[:1], (ValueError, IndexError)), ([fa[0], fa[0][:-1]], ValueError), ([fa[0], fa[1].cpu()], TypeError)):
+        for call in (lambda: s.set_coeffs(lam, bad, fk), lambda: batch.set_coeffs([lam], [bad], [fk])):
+            with pytest.raises(error):
+                call()
+    s.set_coeffs(lam, fa + [fa[0]], fk)          # more face arrays than axes: the first ones count
+    st = s.solve(b, x)
+    assert st["cycles"] == 1
+    batch.close()
+    s.close()
