@@ -84,8 +84,16 @@ __device__ __noinline__ void mom_off_edge(const MomCoeffArgs &A, int i, int j, i
     mom_off<DIM, false>(A, i, j, k, c, mu, 0.0, off);
 }
 
-// The larger of two doubles that are >= 0 or NaN, as bit patterns: their order is the values', a NaN (positive, as
-// arithmetic makes it) the largest, and a negative value the smallest.  On the integer pipe.
+// A double as an integer whose order, from zero up, is the values': a NaN of either sign (the input's, or the one the
+// hardware makes) above infinity, a negative value below zero.  On the integer pipe, from words_of: an integer mask of
+// the double itself becomes an FP64 absolute value, which leaves a NaN's sign.
+__device__ __forceinline__ long long bound_bits(double v) {
+    unsigned lo, hi;
+    words_of(v, lo, hi);
+    const unsigned m = hi & 0x7fffffffu;
+    if (m > 0x7ff00000u || (m == 0x7ff00000u && lo != 0u)) hi = m;
+    return (long long)((unsigned long long)hi << 32 | lo);
+}
 __device__ __forceinline__ long long max_bits(long long a, long long b) { return a > b ? a : b; }
 
 __device__ __forceinline__ unsigned grid_blocks() { return gridDim.x * gridDim.y * gridDim.z; }
@@ -156,7 +164,7 @@ __global__ void __launch_bounds__(256) k_mom_diag(const __grid_constant__ MomCoe
             const double diag = rdt + off[q] + ((AXI && q == 0) ? 2.0 * mu / (ri * ri) : 0.0);
             const double inv = 1.0 / diag;
             A.inv_diag[q][c] = inv;
-            nu = max_bits(nu, __double_as_longlong(2.0 * off[q] * inv));
+            nu = max_bits(nu, bound_bits(2.0 * off[q] * inv));
         }
     }
     const int tid = threadIdx.x + blockDim.x * threadIdx.y;

@@ -52,3 +52,35 @@ def test_jacobi_loop_ends(n):
         m.solve(bad, u, rtol=1e-8, max_iters=3)
     assert all(np.array_equal(a.cpu().numpy(), v) for a, v in zip(u, u0))
     m.close()
+
+
+def _nan(negative):
+    return np.array([0xFFF8000000000000 if negative else 0x7FF8000000000000], dtype=np.uint64).view(np.float64)[0]
+
+
+@pytest.mark.parametrize("grid", ["2d", "axi", "3d"])
+def test_coefficients_that_are_not_finite(grid):
+    """One NaN of either sign in rho or mu, or an infinite mu, among cells whose row bound is far below the limit of the
+    point-Jacobi corrections: the set-up reports it, from an inner cell and from one at the boundary."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2206_11294_gb300.binding import MG_ERR_INVALID_COEFF, MgError, Momentum
+    n = (12, 10, 8) if grid == "3d" else (40, 36, 1)
+    bc = ((I.BC_AXIS if grid == "axi" else W, D), (W, W), (D, W) if grid == "3d" else (0, 0))
+    g = I.Grid(dim=3 if grid == "3d" else 2, axisym=int(grid == "axi"), n=n, h=1e-2, bc=bc)
+    rng = np.random.default_rng(5)
+    shape = (n[2], n[1], n[0])
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a, dtype=np.float64)).cuda()
+    rho, mu, dt = rng.uniform(1.0, 1000.0, shape), 1e-4 * rng.uniform(1e-3, 1.0, shape), 1e-4
+    m = Momentum(g)
+    for field, value in (("rho", _nan(False)), ("rho", _nan(True)), ("mu", _nan(False)), ("mu", _nan(True)),
+                         ("mu", np.inf)):
+        for cell in ((n[2] // 2, 5, 7), (0, 0, n[0] - 1)):
+            f = dict(rho=rho.copy(), mu=mu.copy())
+            f[field][cell] = value
+            with pytest.raises(MgError) as e:
+                m.set_coeffs(dt, dev(f["rho"]), dev(f["mu"]))
+            assert e.value.status == MG_ERR_INVALID_COEFF, (field, value, cell)
+    m.set_coeffs(dt, dev(rho), dev(mu))
+    m.close()
