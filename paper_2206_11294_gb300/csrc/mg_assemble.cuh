@@ -53,10 +53,27 @@ __device__ __forceinline__ long long face_index(const int n[3], int a, int i, in
     return (long long)i + n0 * ((long long)j + n1 * k);
 }
 
+// Whether a product of denominators is far from both ends of the double range, so that its reciprocal times its other
+// factors neither overflows nor loses a factor to underflow (zero, infinity and NaN are not).  On the integer pipe.
+__device__ __forceinline__ bool shared_ok(double product) {
+    const unsigned e = (unsigned)__double2hiint(product) & 0x7ff00000u;
+    return e - (323u << 20) < (1401u << 20);                             // 2^-700 <= |product| < 2^701
+}
+
+// Three quotients by a division each.
+struct Three {
+    double a, b, c;
+};
+__device__ __noinline__ Three divide_apart(Three num, Three den) {
+    return Three{num.a / den.a, num.b / den.b, num.c / den.c};
+}
+
 // One phase's share of the lambda averages at (T, p): beta C_i, the bracket of
 // Eq. 8 times C_i, and beta / (rho c_p) times C_i.  free = C_i - m_i b_i.  One
 // reciprocal serves the three denominators (each the product's reciprocal times
-// the others).
+// the others) while their product is in the middle of the double range; a phase
+// with a vanishing mass takes three divisions, each as exact as its own
+// denominator allows.
 __device__ __forceinline__ void phase_terms(const PhaseK &P, double Ci, double mi, double free, double T, double p,
                                             double &beta_c, double &bracket_c, double &bover_c) {
     if (!(Ci > 0.0)) {      // most warps are pure in one phase and skip the other's division
@@ -64,14 +81,18 @@ __device__ __forceinline__ void phase_terms(const PhaseK &P, double Ci, double m
         return;
     }
     const double pp = p + P.Pi, db = P.g1cv * T + P.b * pp;
-    const double dbp = db * pp, r = 1.0 / (dbp * mi), rm = r * mi;
-    const double beta = P.g1cv * (rm * pp);                              // Eq. 10
-    // C_i gamma / (rho_i c_i^2) with c_i^2 of Eq. 11: gamma (C_i - m_i b_i) / (Gamma (p + Pi))
-    const double comp = P.gam_over_G * free * (rm * db);
-    const double c_over_rho = Ci * Ci * (r * dbp);                       // C_i / rho_i
-    const double bcp = beta * c_over_rho * P.inv_cp;                     // C_i beta / (rho_i c_p)
-    beta_c = Ci * beta;
-    bracket_c = comp - beta * T * bcp;
+    const double dbp = db * pp, d = dbp * mi;
+    // beta (Eq. 10); C_i gamma / (rho_i c_i^2) with c_i^2 of Eq. 11, gamma (C_i - m_i b_i) / (Gamma (p + Pi)); C_i / rho_i
+    Three q;
+    if (shared_ok(d)) {
+        const double r = 1.0 / d, rm = r * mi;
+        q = Three{P.g1cv * (rm * pp), P.gam_over_G * free * (rm * db), Ci * Ci * (r * dbp)};
+    } else {
+        q = divide_apart(Three{P.g1cv, P.gam_over_G * free, Ci * Ci}, Three{db, pp, mi});
+    }
+    const double bcp = q.a * q.c * P.inv_cp;                             // C_i beta / (rho_i c_p)
+    beta_c = Ci * q.a;
+    bracket_c = q.b - q.a * T * bcp;
     bover_c = bcp;
 }
 
@@ -103,10 +124,17 @@ __global__ void __launch_bounds__(256) k_assemble(const __grid_constant__ Assemb
     const double shift = (P1.shift * free1 + m1 * P1.q) + (P2.shift * free2 + m2 * P2.q);
     const double dp = rho * (free1 * P1.inv_g1 + free2 * P2.inv_g1), dT = m1 * P1.cpcv + m2 * P2.cpcv;
     const double ri = AXI ? A.r0 + (i + 0.5) * A.h : 0.0, dr = ri * A.h;
-    const double r = 1.0 / (AXI ? dp * dT * dr : dp * dT), rr = AXI ? r * dr : r;
-    const double p = (rho * (E - shift) - 0.5 * mm) * (rr * dT);
+    const double dpT = dp * dT, all = AXI ? dpT * dr : dpT;
+    Three r;                                             // the reciprocals of dp, dT and dr
+    if (shared_ok(all)) {
+        const double ra = 1.0 / all, rr = AXI ? ra * dr : ra;
+        r = Three{rr * dT, rr * dp, AXI ? ra * dpT : 0.0};
+    } else {
+        r = divide_apart(Three{1.0, 1.0, 1.0}, Three{dp, dT, dr});
+    }
+    const double p = (rho * (E - shift) - 0.5 * mm) * r.a;
     // Eq. 23
-    const double T = ((free1 + free2) * p + (P1.Pi * free1 + P2.Pi * free2)) * (rr * dp);
+    const double T = ((free1 + free2) * p + (P1.Pi * free1 + P2.Pi * free2)) * r.b;
     double b1, k1, o1, b2, k2, o2;
     phase_terms(P1, C, m1, free1, T, p, b1, k1, o1);
     phase_terms(P2, C2, m2, free2, T, p, b2, k2, o2);
@@ -119,7 +147,7 @@ __global__ void __launch_bounds__(256) k_assemble(const __grid_constant__ Assemb
         const long long flo = face_index(A.n, a, i, j, k);
         const long long fhi = face_index(A.n, a, pos[0] + (a == 0), pos[1] + (a == 1), pos[2] + (a == 2));
         const double ulo = A.uf[a][flo], uhi = A.uf[a][fhi];
-        if (AXI && a == 0) div = ((ri + 0.5 * A.h) * uhi - (ri - 0.5 * A.h) * ulo) * (r * (dp * dT));
+        if (AXI && a == 0) div = ((ri + 0.5 * A.h) * uhi - (ri - 0.5 * A.h) * ulo) * r.c;
         else diff = a == (AXI ? 1 : 0) ? uhi - ulo : diff + (uhi - ulo);
     }
     div = AXI ? diff * A.inv_h + div : diff * A.inv_h;

@@ -418,3 +418,28 @@ def test_energy_of_an_absent_phase_is_unchanged(torch_cuda, orc):
     np.testing.assert_array_equal(got1[C == 0.0], E1[C == 0.0])
     np.testing.assert_array_equal(got2[C == 1.0], E2[C == 1.0])
     assert np.any(got1[C == 1.0] != E1[C == 1.0]) and np.any(got2[C == 0.0] != E2[C == 0.0])
+
+
+@pytest.mark.parametrize("grid", ["2d_walls", "axi", "3d"])
+def test_phases_with_vanishing_mass(torch_cuda, orc, grid):
+    """A phase's volume fraction of 1e-312 with a subnormal partial density adds nothing to a cell's coefficients, as in
+    the oracle (the usual tolerances); one with no mass at all leaves lambda_1 and lambda_2 finite (its beta does not
+    depend on its density)."""
+    s = _state(GRIDS[grid])
+    s.C, s.m1, s.m2 = np.array(s.C), np.array(s.m1), np.array(s.m2)
+    flat = lambda a: a.reshape(-1)
+    gas = np.argsort(flat(s.C), kind="stable")[:64]
+    flat(s.m2)[gas] = flat(s.m2)[gas] / (1.0 - flat(s.C)[gas])
+    flat(s.C)[gas], flat(s.m1)[gas] = 1e-312, 1e-309
+    got, _, _ = _gpu_assemble(torch_cuda, s)
+    g = s.grid
+    ref = orc.assemble(g, s.ph1, s.ph2, s.dt, s.C, s.m1, s.m2, s.E, s.mom, s.uf)
+    assert all(np.isfinite(v[k]).all() for v in (got, ref) for k in ("lam", "b", "x0"))
+    _compare(g, s, got, ref)
+    flat(s.C)[gas[:8]], flat(s.m1)[gas[:8]] = 1e-3, 0.0
+    got, _, _ = _gpu_assemble(torch_cuda, s)
+    with np.errstate(all="ignore"):
+        ref = orc.assemble(g, s.ph1, s.ph2, s.dt, s.C, s.m1, s.m2, s.E, s.mom, s.uf)
+    for q in (0, 1):
+        assert np.isfinite(got["lam"][gas[:8], q]).all()
+        _close(got["lam"][gas[:8], q], ref["lam"][gas[:8], q], 1e-12, what=f"lambda_{q + 1}")
