@@ -72,8 +72,6 @@ struct BState {                 // per-problem solve state, device side
 };
 
 constexpr int kBatchThreads = 256;
-// Rows per thread of the norm tiles: the other problems fill the SMs, so large tiles with few reductions.
-constexpr int kBatchNormRows = 4;
 constexpr int kBatchBlocksPerSM = 8;    // default persistent blocks per SM
 
 template <typename R> __device__ __forceinline__ const Level<R> &pick(const BLevel &L);
@@ -479,7 +477,11 @@ __device__ __forceinline__ void batch_finish(const BProb &P, BState &S, int loca
     }
 }
 
-// Stopping norm of every (active) problem's finest level (FP64 path).
+template <int R> using Rows = std::integral_constant<int, R>;
+
+// Stopping norm of every (active) problem's finest level (FP64 path).  Each
+// problem's tiles are those of its solo solve (norm_rows), so that the norms, and
+// with them the cycle count, are the ones mg_solve gets, bit for bit.
 template <int DIM>
 __global__ void __launch_bounds__(kBatchThreads) kb_norm(const BLevel *__restrict__ lv, const BProb *__restrict__ pr,
                                                          BState *__restrict__ st, const int2 *__restrict__ tab, int n,
@@ -494,9 +496,12 @@ __global__ void __launch_bounds__(kBatchThreads) kb_norm(const BLevel *__restric
         if (!initial && !st[p].active) continue;
         const Level<double> L = B.d;
         int bx, by, bz;
-        block_coords(e.y, norm_gx(L.n0), norm_gy(L.n1, kBatchNormRows), bx, by, bz);
-        const double2 s = (red && !initial) ? norm_block<DIM, true, kBatchNormRows>(L, bx, by, bz)
-                                               : norm_block<DIM, false, kBatchNormRows>(L, bx, by, bz);
+        const int rows = norm_rows(L.N);
+        block_coords(e.y, norm_gx(L.n0), norm_gy(L.n1, rows), bx, by, bz);
+        auto tile = [&](auto R) {
+            return (red && !initial) ? norm_block<DIM, true, R.value>(L, bx, by, bz) : norm_block<DIM, false, R.value>(L, bx, by, bz);
+        };
+        const double2 s = rows == 1 ? tile(Rows<1>()) : rows == 2 ? tile(Rows<2>()) : tile(Rows<4>());
         batch_finish(pr[p], st[p], e.y, s, initial, rtol, max_cycles, host + p);
     }
 }
@@ -517,12 +522,16 @@ __global__ void __launch_bounds__(kBatchThreads) kb_residual64(const BLevel *__r
         if (!initial && !st[p].active) continue;
         Level<double> L = B.d;
         int bx, by, bz;
-        block_coords(e.y, norm_gx(L.n0), norm_gy(L.n1, kBatchNormRows), bx, by, bz);
+        const int rows = norm_rows(L.N);
+        block_coords(e.y, norm_gx(L.n0), norm_gy(L.n1, rows), bx, by, bz);
         // defect correction: the initial call stores r0 = b - A x0 over b and sets delta = 0; later calls
         // form r0 - A delta
         if (!initial) L.x = B.delta;
-        const double2 s = residual64_to32_block<DIM, kBatchNormRows>(L, B.f.b, B.f.bt, B.f.x, initial ? L.b : nullptr,
-                                                     initial ? B.delta : nullptr, red_start, bx, by, bz);
+        auto tile = [&](auto R) {
+            return residual64_to32_block<DIM, R.value>(L, B.f.b, B.f.bt, B.f.x, initial ? L.b : nullptr,
+                                                       initial ? B.delta : nullptr, red_start, bx, by, bz);
+        };
+        const double2 s = rows == 1 ? tile(Rows<1>()) : rows == 2 ? tile(Rows<2>()) : tile(Rows<4>());
         batch_finish(pr[p], st[p], e.y, s, initial, rtol, max_cycles, host + p);
     }
 }
@@ -879,8 +888,7 @@ mg_status mg_batch_create(int count, mg_handle *const *handles, mg_batch **out) 
         pr[p].kl = h->coarse_kl;
         pr[p].nc = h->nc;
         pr[p].coarse = base[p] + h->nlev - 1;
-        const LevelBuf &l0 = h->L[0];            // at most the handle's own count (norm_rows is smaller)
-        pr[p].npartial = norm_gx(l0.n[0]) * norm_gy(l0.n[1], kBatchNormRows) * l0.n[2];
+        pr[p].npartial = h->npartial;
         pr[p].x32_0 = h->L[0].x32;
     }
     std::vector<int2> tabs;

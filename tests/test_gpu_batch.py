@@ -369,3 +369,22 @@ def test_batch_sample_of_32_vs_oracle(torch_cuda, orc):
     b.close()
     for s in solvers:
         s.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_batch_norms_equal_the_solo_solves(torch_cuda, precision):
+    """The norms that the stop test reads are summed alike in a batch and alone: equal statistics, bit for bit, for sizes
+    on either side of every tile rule of the norm kernels."""
+    from paper_2206_11294_gb300.binding import Batch
+    probs = [I.bubble_2d(n=n, ny=m, seed=500 + n, n_bubbles=2, rmin=0.05, rmax=0.15, centred=False)
+             for n, m in ((64, 96), (992, 512), (1024, 512), (1024, 1024), (2048, 2048))]
+    solvers = _solvers(probs, precision=precision, rtol=0.0, max_cycles=2)
+    solo = [s.solve(p.b, p.x0.copy()) for s, p in zip(solvers, probs)]
+    b = Batch(solvers)
+    st = b.solve([p.b for p in probs], [p.x0.copy() for p in probs])
+    for p, one, mix in zip(probs, solo, st):
+        for key in ("r0", "rfinal"):
+            assert tuple(one[key]) == tuple(mix[key]), (p.grid.n, key, one[key], mix[key])
+    b.close()
+    for s in solvers:
+        s.close()
