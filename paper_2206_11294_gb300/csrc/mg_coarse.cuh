@@ -27,7 +27,7 @@
 // sub-partition whatever its lanes hold, a reciprocal 360, a cluster barrier
 // 400.
 // Both end with a check: a known vector is multiplied by the assembled matrix
-// and solved for.  If an entry comes back further off than kCoarseTol (a zero
+// and solved for.  If an entry comes back further off than coarse_tol (a zero
 // or tiny pivot block, growth, not-finite input), err[3] stays 0 and the banded
 // LU with partial pivoting that follows runs as the fallback, and reports a
 // singular matrix; otherwise err[3] = 1 and those kernels return at once.
@@ -43,7 +43,12 @@ constexpr int kGjThreads = 256;
 constexpr int kGjMax = 128;            // unknowns of one inverted block
 constexpr int kBcrMaxStages = 12;
 constexpr int kBcrThreads = 512;       // threads per CTA of a solve
-constexpr double kCoarseTol = 1e-9;    // forward error of the check (a stable factorisation leaves cond * 1e-16)
+// Largest relative error of an entry in the check.  Both eliminations leave about cond * 1e-16, as the pivoted LU does
+// (4e-16 to 1e-14 for time steps up to 1e-3 on a unit domain, 1e-10 where cond is 1e7); a pivot block delta away from
+// singular leaves 1e-16 / delta more.  Below the finest level the solve is part of a cycle whose residual is taken
+// anew, and 1e-9 of it changes nothing.  A grid that is its own coarsest level has no such residual in FP64: its one
+// solve is the answer, so what the LU could do better falls back to it from 1e-13 on.
+constexpr double kCoarseTol = 1e-9, kCoarseTolOnly = 1e-13;
 enum { kBcrV = 0, kBcrL, kBcrU, kBcrP, kBcrQ, kBcrX, kBcrY, kBcrB, kBcrArrays };
 
 // One coarsest matrix.  Matrices of the reduction are q x q, column-major, in
@@ -51,6 +56,7 @@ enum { kBcrV = 0, kBcrL, kBcrU, kBcrP, kBcrQ, kBcrX, kBcrY, kBcrB, kBcrArrays };
 // blocks of the assembled matrix (a 2x2 block [[x, 0], [y, z]] per cell).
 struct CoarseProb {
     int nc;                // unknowns
+    int only;              // the hierarchy's only level, solved in FP64: kCoarseTolOnly
     int q, m, stages;      // unknowns per block, blocks, elimination stages (q = 0: not this path)
     int n[3];              // cells per axis
     int sb, wa, s1, s2;    // cell of (block, w): block * sb + (w % wa) * s1 + (w / wa) * s2
@@ -60,6 +66,8 @@ struct CoarseProb {
     float *Minv32;
     int *err;              // the handle's flags: [0] errors, [3] this path's factors are good
 };
+
+__device__ __forceinline__ double coarse_tol(bool only) { return only ? kCoarseTolOnly : kCoarseTol; }
 
 __host__ __device__ inline long long bcr_work_doubles(int q, int m) {
     return (long long)kBcrArrays * m * q * q + 4LL * q * m;
@@ -126,7 +134,8 @@ inline size_t gj_smem(int q) {
 // about 64, then by the FP64 pipe (q^2 / 8 FMA per step, CTA and clock pair).
 // With `M` set (the whole coarsest matrix) the check follows.
 template <typename Load, typename Store>
-__device__ __forceinline__ void gj_invert(int q, Load load, Store store, double *sm, const double *M, int *flag) {
+__device__ __forceinline__ void gj_invert(int q, Load load, Store store, double *sm, const double *M, int *flag,
+                                          double tol) {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
@@ -231,7 +240,7 @@ __device__ __forceinline__ void gj_invert(int q, Load load, Store store, double 
                 double t = 0.0;
                 for (int r = 0; r < kGjCtas; r++) t += part[r * q + i];
                 const double z = bcr_known(i);
-                if (!(fabs(t - z) <= kCoarseTol * z)) *flag = 0;
+                if (!(fabs(t - z) <= tol * z)) *flag = 0;
             }
     }
     cl.sync();                                      // no CTA leaves while another may still store into it
@@ -246,7 +255,7 @@ __device__ __forceinline__ void coarse_invert(const CoarseProb &P, double *sm) {
             P.Minv[(long long)i * n + c] = v;
             if (P.Minv32) P.Minv32[(long long)i * n + c] = (float)v;
         },
-        sm, P.M, P.err + 3);
+        sm, P.M, P.err + 3, coarse_tol(P.only));
 }
 
 // The e-th block of stage s.
@@ -262,7 +271,7 @@ __device__ __forceinline__ void bcr_invert(const CoarseProb &P, int s, int e, do
             if (s > 0) return B[(long long)c * q + i];
             return P.M[(2LL * bcr_cell(P, blk, i >> 1) + (i & 1)) * P.nc + 2 * bcr_cell(P, blk, c >> 1) + (c & 1)];
         },
-        [&](int i, int c, double v) { V[(long long)c * q + i] = v; }, sm, nullptr, nullptr);
+        [&](int i, int c, double v) { V[(long long)c * q + i] = v; }, sm, nullptr, nullptr, 0.0);
 }
 
 // Couplings of the assembled matrix between neighbouring blocks (thread t of nt over both sides).
@@ -565,7 +574,7 @@ __device__ __forceinline__ void bcr_check(const CoarseProb &P, double *sm) {
         },
         [&](int c, int a, double v) {
             const double z = bcr_known(2 * c + a);
-            if (!(fabs(v - z) <= kCoarseTol * z)) P.err[3] = 0;
+            if (!(fabs(v - z) <= coarse_tol(P.only) * z)) P.err[3] = 0;
         },
         sm);
 }

@@ -110,3 +110,53 @@ def test_singular_matrix_is_still_refused(binding):
                 s.set_coeffs(lam, ones, fk)
                 s.solve(np.zeros((g.N, 2)), np.zeros((g.N, 2)))
         s.close()
+
+
+@pytest.mark.parametrize("delta", [1e-2, 1e-4, 1e-6, 1e-8, 1e-10, 1e-12, 1e-14])
+@pytest.mark.parametrize("n", [(7, 7, 1), (9, 13, 1)], ids=["inverse", "reduction"])
+def test_nearly_singular_pivot_block(binding, n, delta):
+    """The second pivot block after the first one's elimination is delta away from singular: elimination without row
+    exchanges loses a factor 1 / delta.  A grid that is its own coarsest level is solved from these factors alone, so
+    its error stays within the bound of a backward stable solve, 16 eps cond(A) (test above)."""
+    g, lam, ones = _singular_pivot(n)
+    lam[1, 0] += delta
+    A = paper_operator(g, lam, ones, ones)
+    A = np.asarray((A[0] if isinstance(A, tuple) else A).todense())
+    xs = np.random.default_rng(3).normal(size=(g.N, 2))
+    b = (A @ xs.reshape(-1)).reshape(-1, 2)
+    for batched in (False, True):
+        s = binding.Solver(g, rtol=0.0, max_cycles=1)
+        x = np.zeros((g.N, 2))
+        if batched:
+            batch = binding.Batch([s])
+            batch.set_coeffs([lam], [ones], [ones])
+            batch.solve([b], [x])
+            batch.close()
+        else:
+            s.set_coeffs(lam, ones, ones)
+            s.solve(b, x)
+        s.close()
+        assert np.abs(x - xs).max() <= 16 * np.finfo(float).eps * np.linalg.cond(A) * np.abs(xs).max()
+
+
+def test_long_thin_coarsest_grid(binding):
+    """300 blocks of 4 unknowns: nine elimination stages."""
+    test_single_level_solve_is_the_dense_solution(binding, (2, 300, 1), "fp64")
+
+
+def test_blocks_above_the_inverse_beside_smaller_ones(binding):
+    """9 x 9 x 9 cells have blocks of 162 unknowns, too large for the cluster inverse (kGjMax): in a batch they keep the
+    banded LU while 5 x 5 x 5 and 7 x 6 x 7 take the reduction."""
+    import oracle
+    probs = [I.random_coeff_problem(_grid(n), seed=sum(n)) for n in ((5, 5, 5), (9, 9, 9), (7, 6, 7))]
+    solvers = [binding.Solver(p.grid, rtol=0.0, max_cycles=1) for p in probs]
+    batch = binding.Batch(solvers)
+    batch.set_coeffs([p.lam for p in probs], [p.fa for p in probs], [p.fk for p in probs])
+    xs = [p.x0.copy() for p in probs]
+    batch.solve([p.b for p in probs], xs)
+    for p, x in zip(probs, xs):
+        ref = oracle.dense_solve(p.grid.as_dict(), p.lam, p.fa, p.fk, p.b)
+        assert _rel(x, ref, p.x0) <= 1e-12, p.grid.n
+    batch.close()
+    for s in solvers:
+        s.close()
