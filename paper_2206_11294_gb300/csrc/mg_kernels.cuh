@@ -2101,7 +2101,8 @@ __device__ __forceinline__ void band_lu_blocked_block(const double *__restrict__
                     break;
                 }
                 const int pp = s_p;
-                if (tid < k1 - p) {                         // swap rows p and pp in the panel's columns p..k1-1
+                const int reach = min(k1 - p - 1, ur);      // the panel's columns after p that row p reaches
+                if (tid <= reach) {                         // swap rows p and pp in them and in column p
                     const int j = p + tid;
                     double *cj = colp(j);
                     const int ia = p - j + ur, ib = pp - j + ur;
@@ -2123,14 +2124,14 @@ __device__ __forceinline__ void band_lu_blocked_block(const double *__restrict__
                     bs[(p - k0) * kl + q] = l;
                     Lb[(long long)p * kl + q] = l;
                 }
-                if (tid < k1 - p - 1) {                     // row p of U in the panel's columns p+1..k1-1
+                if (tid < reach) {                          // row p of U in them
                     const int j = p + 1 + tid;
                     const double u = colp(j)[p - j + ur];
                     urow[tid] = u;
                     Uc[(long long)j * C + (j - p)] = u;
                 }
                 __syncthreads();
-                for (int c = warp; c < k1 - p - 1; c += nw) {   // the panel's columns by warp, rows by lane
+                for (int c = warp; c < reach; c += nw) {    // a column per warp, rows by lane
                     const int j = p + 1 + c;
                     double *cj = colp(j);
                     const double u = urow[c];

@@ -160,3 +160,32 @@ def test_blocks_above_the_inverse_beside_smaller_ones(binding):
     batch.close()
     for s in solvers:
         s.close()
+
+
+@pytest.mark.parametrize("n", [(1, 90, 1), (2, 40, 1), (3, 50, 1), (2, 300, 1)], ids=lambda n: "x".join(map(str, n)))
+def test_banded_factors_of_narrow_grids(binding, n):
+    """Bands narrower than a panel of the blocked LU (three columns and less along the fast axis), by the inverse it
+    forms and, with a nearly singular pivot block, as the reduction's fallback.  The tolerances are the ones above."""
+    import oracle
+    p = I.random_coeff_problem(_grid(n), seed=sum(n))
+    ref = oracle.dense_solve(p.grid.as_dict(), p.lam, p.fa, p.fk, p.b)
+    s = binding.Solver(p.grid, rtol=0.0, max_cycles=1, coarse="inverse")
+    assert len(s.levels()) == 1
+    s.set_coeffs(p.lam, p.fa, p.fk)
+    x = p.x0.copy()
+    s.solve(p.b, x)
+    s.close()
+    assert _rel(x, ref, p.x0) <= 1e-12
+    g, lam, ones = _singular_pivot(n)
+    if n[0] < 3:
+        lam[0, 0], lam[1, 0] = 1.0 + n[0], 1.0 + 2.0         # one or two interior faces, and two
+    A = paper_operator(g, lam, ones, ones)
+    A = np.asarray((A[0] if isinstance(A, tuple) else A).todense())
+    xs = np.random.default_rng(3).normal(size=(g.N, 2))
+    b = (A @ xs.reshape(-1)).reshape(-1, 2)
+    x = np.zeros((g.N, 2))
+    s = binding.Solver(g, rtol=0.0, max_cycles=1)
+    s.set_coeffs(lam, ones, ones)
+    s.solve(b, x)
+    s.close()
+    assert np.abs(x - xs).max() <= 16 * np.finfo(float).eps * np.linalg.cond(A) * np.abs(xs).max()

@@ -253,3 +253,25 @@ def test_tma_sweep_on_ragged_grid(torch_cuda, precision):
         assert e.value.status == MG_ERR_INVALID_ARG and "does not fit" in str(e.value)
         assert s0.tuning() == base
     s0.close()
+
+
+def test_tail_whose_padded_state_exceeds_shared_memory(torch_cuda):
+    """Rows of one cell take two slots in the tail's colour-split state: a 2 x 1600 first tail level over a 1 x 800
+    coarsest one is a tail the rules allow (192 KB) and its kernel cannot hold (230 KB).  Such a tail runs as separate
+    launches, with the same result."""
+    g = I.Grid(dim=2, axisym=0, n=(4, 3200, 1), h=1e-4, bc=((I.BC_WALL, I.BC_DIRICHLET), (I.BC_WALL, I.BC_WALL), (0, 0)),
+               bcT=((0, 300), (0, 0), (0, 0)), bcp=((0, 1e5), (0, 0), (0, 0)))
+    p = I.random_coeff_problem(g, seed=9, dt=1e-5)
+    from paper_2206_11294_gb300.binding import Solver
+    out = []
+    for tail in (False, True):
+        s = Solver(g, rtol=0.0, max_cycles=3, coarse="inverse", coarse_min=1)
+        s.set_coeffs(p.lam, p.fa, p.fk)
+        n = s.tuning()["levels"]
+        assert n == 3 and s.levels()[-1][:2] == (1, 800)
+        s.set_tuning(dict(s.tuning(), tail_level=1 if tail else n, tail_ctas=1))
+        x = p.x0.copy()
+        s.solve(p.b, x)
+        out.append(x)
+        s.close()
+    assert np.isfinite(out[0]).all() and np.array_equal(out[0], out[1])
