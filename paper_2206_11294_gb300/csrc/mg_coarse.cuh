@@ -30,7 +30,9 @@
 // and solved for.  If an entry comes back further off than coarse_tol (a zero
 // or tiny pivot block, growth, not-finite input), err[3] stays 0 and the banded
 // LU with partial pivoting that follows runs as the fallback, and reports a
-// singular matrix; otherwise err[3] = 1 and those kernels return at once.
+// singular matrix; otherwise err[3] = 1 and those kernels return at once.  A
+// matrix that falls back pays for both: set-up and two cycles of 992 x 736 take
+// 4.72 ms, 4.52 by the LU alone, 0.94 where the check passes.
 #pragma once
 #include <cooperative_groups.h>
 
@@ -593,7 +595,7 @@ __device__ __forceinline__ void coarse_solve_cluster(const CoarseProb &P, const 
                     f[u] = (double)b[2 * bcr_cell(P, u / P.q, (u % P.q) >> 1) + (u & 1)];
             },
             [&](int c, int a, double v) { x[2 * c + a] = (R)v; }, sm);
-    } else if (blockIdx.x % kGjCtas == 0) {
+    } else if (blockIdx.x % kGjCtas == 0 && threadIdx.x < kLuSolveThreads) {
         coarse_lu_solve_block<R>(Lb, Uc, piv, dinv, P.nc, kl, kl, b, x, P.err, sm);
     }
 }

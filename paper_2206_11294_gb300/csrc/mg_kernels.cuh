@@ -2287,9 +2287,11 @@ __global__ void __launch_bounds__(256) k_band_inv_block(const double *__restrict
 // is.  The steps are those of one column of k_band_inv_block with b in place
 // of e_j: the row swaps and multipliers in the order the factorisation
 // applied them, then U from the last row up.  A step's multiply-adds are
-// spread over the block's warps and so over the SM's sub-partitions: GB300's FP64
-// pipe issues a warp's FMA over many cycles, so one warp would take four
-// times as long per step.  One barrier per step, two for a forward step that
+// spread over four warps, one per SM sub-partition: GB300's FP64 pipe issues a
+// warp's FMA over many cycles, so one warp would take four times as long per
+// step, and more than four only make the barrier longer (a cycle of 992 x 736
+// with a 31 x 23 coarsest grid on the fallback: 719 us with 16 warps, 685 with
+// 4).  One barrier per step, two for a forward step that
 // swaps rows: every thread reads the pivot row's value itself (and, for a
 // swap, y_k, before thread 0 overwrites it); the thread that updates the
 // pivot row starts from the value swapped out of row k.  In the backward
@@ -2301,6 +2303,7 @@ __global__ void __launch_bounds__(256) k_band_inv_block(const double *__restrict
 // the solve) x is set to 0.
 // ---------------------------------------------------------------------------
 constexpr int kLuSolveRows = 16;
+constexpr int kLuSolveThreads = 128;
 
 // Shared memory of that solve (bytes): y, then two chunks each of Lb rows,
 // Uc rows and piv.
@@ -2347,12 +2350,17 @@ __global__ void k_scale_uc(double *__restrict__ Uc, const double *__restrict__ d
              (long long)gridDim.x * blockDim.x);
 }
 
+// Barrier of the threads that solve (the rest of the block is not in it).
+__device__ __forceinline__ void lu_solve_sync() { asm volatile("bar.sync 1, %0;\n" ::"n"(kLuSolveThreads) : "memory"); }
+
+// Called by the block's first kLuSolveThreads threads.
 template <typename R>
 __device__ void coarse_lu_solve_block(const double *__restrict__ Lb, const double *__restrict__ Uc,
                                       const int *__restrict__ piv, const double *__restrict__ dinv, int n, int kl,
                                       int ku, const R *__restrict__ b, R *__restrict__ x,
                                       const int *__restrict__ err, double *sm) {
-    const int tid = threadIdx.x, nt = blockDim.x;
+    constexpr int nt = kLuSolveThreads;
+    const int tid = threadIdx.x;
     if (*(volatile const int *)err & 4) {
         for (int i = tid; i < n; i += nt) x[i] = R(0);
         return;
@@ -2376,14 +2384,14 @@ __device__ void coarse_lu_solve_block(const double *__restrict__ Lb, const doubl
     stage_l(0, 0);
     for (int c = 0; c < nch; c++) {
         const int k0 = c * kLuSolveRows, cnt = min(kLuSolveRows, n - k0), buf = c & 1;
-        __syncthreads();                        // chunk c - 1, in the other buffer, is done with
+        lu_solve_sync();                        // chunk c - 1, in the other buffer, is done with
         if (c + 1 < nch) {
             stage_l(k0 + kLuSolveRows, buf ^ 1);
             cp_async_wait<1>();
         } else {
             cp_async_wait<0>();
         }
-        __syncthreads();
+        lu_solve_sync();
         const double *Lc = Lbuf + buf * kLuSolveRows * kl;
         const int *pc = pbuf + buf * kLuSolveRows;
         for (int t = 0; t < cnt; t++) {
@@ -2392,7 +2400,7 @@ __device__ void coarse_lu_solve_block(const double *__restrict__ Lb, const doubl
             double a = 0.0;
             if (p != k) {                          // the same branch in every thread
                 a = y[k];
-                __syncthreads();                   // both read everywhere before either changes
+                lu_solve_sync();                   // both read everywhere before either changes
                 if (tid == 0) y[k] = yk;
             }
             const int m = min(kl, n - 1 - k);
@@ -2401,7 +2409,7 @@ __device__ void coarse_lu_solve_block(const double *__restrict__ Lb, const doubl
                 const double v = r == p ? a : y[r];
                 y[r] = v - Lc[t * kl + q] * yk;
             }
-            __syncthreads();
+            lu_solve_sync();
         }
     }
     // backward: rows hi - cnt + 1 .. hi of the scaled Uc per chunk, from the last row up
@@ -2415,21 +2423,21 @@ __device__ void coarse_lu_solve_block(const double *__restrict__ Lb, const doubl
     stage_u(n - 1, 0);
     for (int c = 0; c < nch; c++) {
         const int hi = n - 1 - c * kLuSolveRows, cnt = min(kLuSolveRows, hi + 1), lo = hi - cnt + 1, buf = c & 1;
-        __syncthreads();
+        lu_solve_sync();
         if (c + 1 < nch) {
             stage_u(hi - kLuSolveRows, buf ^ 1);
             cp_async_wait<1>();
         } else {
             cp_async_wait<0>();
         }
-        __syncthreads();
+        lu_solve_sync();
         const double *Ucc = Ubuf + buf * kLuSolveRows * C;
         for (int t = cnt - 1; t >= 0; t--) {
             const int i = lo + t;
             const double yi = y[i];
             const int m = min(ur, i);
             for (int o = 1 + tid; o <= m; o += nt) y[i - o] -= Ucc[t * C + o] * yi;
-            __syncthreads();
+            lu_solve_sync();
         }
     }
     for (int i = tid; i < n; i += nt) x[i] = (R)(y[i] * dinv[i]);
