@@ -52,11 +52,15 @@ __device__ __forceinline__ void block_coords(int local, int gx, int gy, int &bx,
     } while (0)
 // A 2x2 block by one 256-bit access (sm_100 and later; 32-byte aligned): a
 // lane's block is one sector, which two 128-bit accesses would touch twice.
+// Volatile, so that it stays behind pdl_entry's wait (not volatile, it would be a
+// function of the address to the compiler, free to move); a memory clobber
+// besides, which no caller needs (no kernel reads blocks that it writes), cost
+// the batch of 24 grids 1.2%.
 __device__ __forceinline__ dq ldgq(const dq *p) {
     dq q;
-    asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];\n"
-        : "=d"(q.a), "=d"(q.b), "=d"(q.c), "=d"(q.d)
-        : "l"(__cvta_generic_to_global(p)));
+    asm volatile("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];\n"
+                 : "=d"(q.a), "=d"(q.b), "=d"(q.c), "=d"(q.d)
+                 : "l"(__cvta_generic_to_global(p)));
     return q;
 }
 __device__ __forceinline__ void stq(dq *p, const dq &q) {

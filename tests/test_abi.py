@@ -194,3 +194,16 @@ def test_binding_constants_match_the_header():
         named = k.startswith(("MG_SWEEP_", "MG_ERR_", "MG_ASSEMBLE_", "MG_MOMENTUM_"))
         if named or k in ("MG_OK", "MG_FP64", "MG_MIXED"):
             assert k in bound, k
+
+
+def test_assembly_that_touches_memory_is_volatile():
+    """A load written as plain asm is a function of its address to the compiler, which may move it in front of the wait
+    for the kernel before (griddepcontrol.wait) or a barrier."""
+    root = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2206_11294_gb300", "csrc")
+    plain = []
+    for name in sorted(os.listdir(root)):
+        text = open(os.path.join(root, name)).read()
+        for m in re.finditer(r"\basm\s*(volatile)?\s*\(\s*\"([^\"]*)", text):
+            if not m.group(1) and "[" in m.group(2):
+                plain.append((name, m.group(2)))
+    assert not plain
