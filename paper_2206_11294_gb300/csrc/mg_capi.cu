@@ -283,7 +283,8 @@ void plan(mg_handle *h, char *base, size_t *bytes) {
         const bool pingpong = g.dim == 2 || h->opt.smoother == MG_SMOOTH_WJAC;
         if (pingpong) l.xalt = P.take<double2>(l.N);
         for (int a = 0; a < g.dim; a++) l.G[a] = P.take<double2>(l.nf[a]);
-        l.S = P.take<dq>(l.N);
+        // (the finest level's S is lambda itself on Cartesian grids: SetupFine::lam)
+        if (h->nlev > 0 || g.axisym) l.S = P.take<dq>(l.N);
         l.D = P.take<dq>(l.N);
         l.Dinv = P.take<dq>(l.N);
         l.W = P.take<dq>(l.N);
@@ -1555,10 +1556,8 @@ mg_status solve_mixed(mg_handle *h, mg_stats *st) {
     }
     // r0 = b - A x0 once, delta from A delta = r0 by FP32 cycles with the
     // FP64 residual r0 - A delta after each outer step; solve_out adds x0
-    const LevelBuf &f = h->L[0];
-    const mg_status e = run_loop(h, st, h->g32, h->graph_kernels32, h->opt.inner_cycles,
-                                 [&](cudaStream_t s) { enqueue_residual_to32<DIM>(h, s, true, h->norms_h + 2); });
-    return e;
+    return run_loop(h, st, h->g32, h->graph_kernels32, h->opt.inner_cycles,
+                    [&](cudaStream_t s) { enqueue_residual_to32<DIM>(h, s, true, h->norms_h + 2); });
 }
 
 // opt.max_cycles FP64 cycles from x = 0 with no stopping norms and no host wait: a fixed linear map of rhs, the
@@ -1590,7 +1589,7 @@ mg_status enqueue_correction(mg_handle *h, cudaStream_t s, const double2 *rhs) {
     if (h->opt.precision == MG_MIXED) {
         enqueue_residual_to32<DIM>(h, s, true, nullptr);        // x = 0: b32 = b, bt32 = Dinv b, e32 = 0
         for (int q = 0; q < h->opt.max_cycles; q++)
-        enqueue_vcycle<float, DIM>(h, s, 0, h->opt.cycle, q == 0 && red_start(h));
+            enqueue_vcycle<float, DIM>(h, s, 0, h->opt.cycle, q == 0 && red_start(h));
         launch_k(h, k_add_correction, lin_blocks(f.N), 256, 0, s, 0, f.x, f.x32, f.N);
         counted(h);
     } else {

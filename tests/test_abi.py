@@ -178,6 +178,18 @@ def test_factored_coarse_solve_needs_no_inverse(lib):
     assert st == st2 == 0 and a == b
 
 
+def test_no_finest_row_blocks_on_cartesian_grids(lib):
+    """The set-up coarsens the caller's lambda on Cartesian grids, so the workspace holds the finest level's scaled rows
+    (32 bytes a cell) on axisymmetric grids only."""
+    n = (512, 256, 1)
+    st, plane = _size(lib, _grid(n=n, h=1 / 512))
+    g = _grid(n=n, h=1 / 512)
+    g.axisym, g.bc[0][0] = 1, 2
+    st2, axi = _size(lib, g)
+    assert st == st2 == 0
+    assert axi - plane == 32 * n[0] * n[1]
+
+
 def test_binding_constants_match_the_header():
     """Every MG_* enum value the binding defines equals the header's, and the
     header's sweep kinds, status codes and flags all have a binding name."""
