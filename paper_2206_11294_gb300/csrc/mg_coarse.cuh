@@ -58,7 +58,6 @@ enum { kBcrV = 0, kBcrL, kBcrU, kBcrP, kBcrQ, kBcrX, kBcrY, kBcrB, kBcrArrays };
 // blocks of the assembled matrix (a 2x2 block [[x, 0], [y, z]] per cell).
 struct CoarseProb {
     int nc;                // unknowns
-    int only;              // the hierarchy's only level, solved in FP64: kCoarseTolOnly
     int q, m, stages;      // unknowns per block, blocks, elimination stages (q = 0: not this path)
     int n[3];              // cells per axis
     int sb, wa, s1, s2;    // cell of (block, w): block * sb + (w % wa) * s1 + (w / wa) * s2
@@ -67,6 +66,7 @@ struct CoarseProb {
     double *Minv;          // nc <= kBandSmemMax: the inverse, row-major
     float *Minv32;
     int *err;              // the handle's flags: [0] errors, [3] this path's factors are good
+    int only;              // the hierarchy's only level, solved in FP64: kCoarseTolOnly
 };
 
 __device__ __forceinline__ double coarse_tol(bool only) { return only ? kCoarseTolOnly : kCoarseTol; }
