@@ -41,7 +41,7 @@ struct BProb {                  // one problem, device side
     int kl;
     int nc;
     int coarse;                 // index of its coarsest level in the BLevel table
-    int npartial;
+    int npartial, nitems;       // tiles of the stopping norm, and work items they are summed in
     float2 *x32_0;              // finest-level FP32 correction (mixed)
 };
 
@@ -72,6 +72,8 @@ struct BState {                 // per-problem solve state, device side
 };
 
 constexpr int kBatchThreads = 256;
+// Rows per thread of the norm kernels' work items: the other problems fill the SMs, so large items.
+constexpr int kBatchNormRows = 4;
 constexpr int kBatchBlocksPerSM = 8;    // default persistent blocks per SM
 
 template <typename R> __device__ __forceinline__ const Level<R> &pick(const BLevel &L);
@@ -431,20 +433,47 @@ __device__ __forceinline__ bool batch_converged(const double n0[2], const double
     return true;
 }
 
-// After a block stored its partial: the problem's last block sums them (in
-// order), updates that problem's state with mg_solve's stopping rule and
+// One work item of the norm kernels, kBatchNormRows x kBY rows of a tile column:
+// row(j, zT2, zp2) adds row j's squares.  The item holds one, two or four tiles
+// of the problem's solo solve (norm_rows), each summed and stored as a solo block
+// would (block_sum2), a warp per sum, so that the norms and with them the cycle
+// count are the ones mg_solve gets, bit for bit; the loads and the ticket are
+// those of one large tile (a set-up and solve of 24 to 30 uneven grids within
+// 0.6% of one sum per item; an item per tile 0.5 to 2% slower).  The problem's
+// last item sums its tiles (in order),
+// updates that problem's state with mg_solve's stopping rule and
 // leaves a copy in page-locked host memory, where the host counts the problems
 // that continue (a counter with its memset and copy nodes cost 9 us a cycle).
-__device__ __forceinline__ void batch_finish(const BProb &P, BState &S, int local, double2 s, int initial,
-                                             double rtol, int max_cycles, BState *host) {
+template <typename Row>
+__device__ __forceinline__ void batch_norms(const BProb &P, BState &S, const Level<double> &L, int bx, int by, int bz,
+                                            Row row, int initial, double rtol, int max_cycles, BState *host) {
     __shared__ bool last;
+    __shared__ double sv[2 * kBatchNormRows][kBatchThreads];
     const int tid = threadIdx.x + blockDim.x * threadIdx.y;
     const int nthr = blockDim.x * blockDim.y;
-    if (tid == 0) {
-        P.partial[local] = s;
-        __threadfence();
-        last = atomicAdd(P.ticket, 1u) == (unsigned)P.npartial - 1u;
+    const int shift = norm_rows(L.N) >> 1, tiles = kBatchNormRows >> shift;      // rows 1, 2, 4: 1 << shift
+    double zT2 = 0.0, zp2 = 0.0;
+#pragma unroll
+    for (int r = 0; r < kBatchNormRows; r++) {
+        row((by * kBatchNormRows + r) * kBY + (int)threadIdx.y, zT2, zp2);
+        if (((r + 1) & ((1 << shift) - 1)) == 0) {       // a tile ends (the same branch in every thread)
+            const int t = r >> shift;
+            sv[2 * t][tid] = zT2;
+            sv[2 * t + 1][tid] = zp2;
+            zT2 = zp2 = 0.0;
+        }
     }
+    __syncthreads();
+    const int w = tid >> 5, gx = norm_gx(L.n0), gy = norm_gy(L.n1, 1 << shift), tile = by * tiles + (w >> 1);
+    if (w < 2 * tiles) {
+        const double v = warp_sum(sv[w], tid & 31);
+        if ((tid & 31) == 0 && tile < gy) {
+            reinterpret_cast<double *>(P.partial + bx + (long long)gx * (tile + (long long)gy * bz))[w & 1] = v;
+            __threadfence();
+        }
+    }
+    __syncthreads();
+    if (tid == 0) last = atomicAdd(P.ticket, 1u) == (unsigned)P.nitems - 1u;
     __syncthreads();
     if (!last) return;
     __threadfence();
@@ -477,11 +506,7 @@ __device__ __forceinline__ void batch_finish(const BProb &P, BState &S, int loca
     }
 }
 
-template <int R> using Rows = std::integral_constant<int, R>;
-
-// Stopping norm of every (active) problem's finest level (FP64 path).  Each
-// problem's tiles are those of its solo solve (norm_rows), so that the norms, and
-// with them the cycle count, are the ones mg_solve gets, bit for bit.
+// Stopping norm of every (active) problem's finest level (FP64 path).
 template <int DIM>
 __global__ void __launch_bounds__(kBatchThreads) kb_norm(const BLevel *__restrict__ lv, const BProb *__restrict__ pr,
                                                          BState *__restrict__ st, const int2 *__restrict__ tab, int n,
@@ -496,13 +521,15 @@ __global__ void __launch_bounds__(kBatchThreads) kb_norm(const BLevel *__restric
         if (!initial && !st[p].active) continue;
         const Level<double> L = B.d;
         int bx, by, bz;
-        const int rows = norm_rows(L.N);
-        block_coords(e.y, norm_gx(L.n0), norm_gy(L.n1, rows), bx, by, bz);
-        auto tile = [&](auto R) {
-            return (red && !initial) ? norm_block<DIM, true, R.value>(L, bx, by, bz) : norm_block<DIM, false, R.value>(L, bx, by, bz);
-        };
-        const double2 s = rows == 1 ? tile(Rows<1>()) : rows == 2 ? tile(Rows<2>()) : tile(Rows<4>());
-        batch_finish(pr[p], st[p], e.y, s, initial, rtol, max_cycles, host + p);
+        block_coords(e.y, norm_gx(L.n0), norm_gy(L.n1, kBatchNormRows), bx, by, bz);
+        const int k = DIM == 3 ? bz : 0;
+        batch_norms(
+            pr[p], st[p], L, bx, by, bz,
+            [&](int j, double &zT2, double &zp2) {
+                if (red && !initial) norm_row<DIM, true>(L, bx, j, k, zT2, zp2);
+                else norm_row<DIM, false>(L, bx, j, k, zT2, zp2);
+            },
+            initial, rtol, max_cycles, host + p);
     }
 }
 
@@ -522,17 +549,18 @@ __global__ void __launch_bounds__(kBatchThreads) kb_residual64(const BLevel *__r
         if (!initial && !st[p].active) continue;
         Level<double> L = B.d;
         int bx, by, bz;
-        const int rows = norm_rows(L.N);
-        block_coords(e.y, norm_gx(L.n0), norm_gy(L.n1, rows), bx, by, bz);
+        block_coords(e.y, norm_gx(L.n0), norm_gy(L.n1, kBatchNormRows), bx, by, bz);
         // defect correction: the initial call stores r0 = b - A x0 over b and sets delta = 0; later calls
         // form r0 - A delta
         if (!initial) L.x = B.delta;
-        auto tile = [&](auto R) {
-            return residual64_to32_block<DIM, R.value>(L, B.f.b, B.f.bt, B.f.x, initial ? L.b : nullptr,
-                                                       initial ? B.delta : nullptr, red_start, bx, by, bz);
-        };
-        const double2 s = rows == 1 ? tile(Rows<1>()) : rows == 2 ? tile(Rows<2>()) : tile(Rows<4>());
-        batch_finish(pr[p], st[p], e.y, s, initial, rtol, max_cycles, host + p);
+        double2 *r_out = initial ? L.b : nullptr, *r_out2 = initial ? B.delta : nullptr;
+        batch_norms(
+            pr[p], st[p], L, bx, by, bz,
+            [&](int j, double &zT2, double &zp2) {
+                residual64_to32_row<DIM>(L, B.f.b, B.f.bt, B.f.x, r_out, r_out2, red_start, bx, j, DIM == 3 ? bz : 0, zT2,
+                                         zp2);
+            },
+            initial, rtol, max_cycles, host + p);
     }
 }
 
@@ -888,7 +916,9 @@ mg_status mg_batch_create(int count, mg_handle *const *handles, mg_batch **out) 
         pr[p].kl = h->coarse_kl;
         pr[p].nc = h->nc;
         pr[p].coarse = base[p] + h->nlev - 1;
-        pr[p].npartial = h->npartial;
+        pr[p].npartial = h->npartial;            // the solo solve's tiles
+        const LevelBuf &l0 = h->L[0];
+        pr[p].nitems = norm_gx(l0.n[0]) * norm_gy(l0.n[1], kBatchNormRows) * l0.n[2];
         pr[p].x32_0 = h->L[0].x32;
     }
     std::vector<int2> tabs;
@@ -926,7 +956,7 @@ mg_status mg_batch_create(int count, mg_handle *const *handles, mg_batch **out) 
         const mg_handle *h = handles[p];
         const dim3 g0 = cell_grid(h->L[0], dim, h->L[0].n[0]);
         add_blocks(tn, base[p], (long long)g0.x * g0.y * g0.z);
-        add_blocks(tnorm, base[p], pr[p].npartial);
+        add_blocks(tnorm, base[p], pr[p].nitems);
         if (!h->coarse_factors)
             for (int r = 0; r * coarse_rows_per_block(h->nc) < h->nc; r++) tco.push_back(make_int2(p, r));
         add_blocks(tcell, base[p], (h->L[0].N + kBatchThreads - 1) / kBatchThreads);

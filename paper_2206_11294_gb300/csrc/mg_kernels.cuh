@@ -616,6 +616,16 @@ __global__ void __launch_bounds__(kReduceThreads) k_coarse_matvec(const R *__res
 // trees in every warp (ten additions each) would be the larger part of a small
 // tile's work: the values meet in shared memory, warp 0 sums a and warp 1 b, one
 // column of eight per lane and then one tree each.
+// warp_sum: one warp's part of it, the sum in lane 0.
+__device__ __forceinline__ double warp_sum(const double *v, int lane) {
+    double a = v[lane];
+#pragma unroll
+    for (int r = 1; r < kReduceThreads / 32; r++) a += v[32 * r + lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+    return a;
+}
+
 __device__ __forceinline__ void block_sum2(double &a, double &b) {
     __shared__ double sv[2][kReduceThreads];
     __shared__ double res[2];
@@ -625,11 +635,7 @@ __device__ __forceinline__ void block_sum2(double &a, double &b) {
     __syncthreads();
     const int w = tid >> 5, lane = tid & 31;
     if (w < 2) {
-        double v = sv[w][lane];
-#pragma unroll
-        for (int r = 1; r < kReduceThreads / 32; r++) v += sv[w][32 * r + lane];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        const double v = warp_sum(sv[w], lane);
         if (lane == 0) res[w] = v;
     }
     __syncthreads();
@@ -682,7 +688,7 @@ __device__ __forceinline__ void finish_norms(double2 *partial, int nblocks, unsi
 // cells over more SMs (64^2: 8 tiles instead of 2, 15.4 -> 8.1 us; the residual
 // of 256 x 512 cells: 256 tiles instead of 64, 22.7 -> 12.3 us).  Each thread
 // accumulates its cells' squares with FMAs; a persistent block reduces once.
-// (The batched kernels reduce per tile.)
+// (The batched kernels reduce per tile, batch_norms.)
 constexpr int kNormCols = 64;
 __host__ __device__ __forceinline__ int norm_rows(long long N) { return N >= (1LL << 22) ? 4 : N >= (1LL << 19) ? 2 : 1; }
 __host__ __device__ __forceinline__ int norm_gx(int n0) { return (n0 + kNormCols - 1) / kNormCols; }
@@ -701,40 +707,34 @@ __device__ __forceinline__ void norm_cell(const Level<double> &L, int i, int j, 
     zp2 = fma(zp, zp, zp2);
 }
 
-// Sums of (Dinv r)_T^2 and (Dinv r)_p^2 over tile (bx, by, bz) of the norm
-// grid (norm_gx, norm_gy, n2), added to zT2, zp2 (norm_block: reduced over the
-// block).
+// Sums of (Dinv r)_T^2 and (Dinv r)_p^2 over row j of tile column bx (norm_tile:
+// over tile (bx, by, bz) of the norm grid, norm_gx x norm_gy x n2), added to zT2,
+// zp2.
 //
 // RED: x has just come out of a red-black sweep, so the block residual of
 // the black cells is exactly zero (z = gs_update - x recomputes the very
 // update that produced x, bit for bit) and each thread visits the one red
 // cell of its column pair per row.
-template <int DIM, bool RED, int ROWS>
-__device__ __forceinline__ void norm_tile(const Level<double> &L, int bx, int by, int bz, double &zT2, double &zp2) {
-    const int k = DIM == 3 ? bz : 0;
+template <int DIM, bool RED>
+__device__ __forceinline__ void norm_row(const Level<double> &L, int bx, int j, int k, double &zT2, double &zp2) {
+    if (j >= L.n1) return;
+    if (RED) {
+        const int i = bx * kNormCols + 2 * threadIdx.x + ((j + k) & 1);
+        if (i < L.n0) norm_cell<DIM>(L, i, j, k, zT2, zp2);
+    } else {
 #pragma unroll
-    for (int r = 0; r < ROWS; r++) {
-        const int j = (by * ROWS + r) * kBY + threadIdx.y;
-        if (j >= L.n1) continue;
-        if (RED) {
-            const int i = bx * kNormCols + 2 * threadIdx.x + ((j + k) & 1);
+        for (int e = 0; e < 2; e++) {
+            const int i = bx * kNormCols + e * kBX + threadIdx.x;
             if (i < L.n0) norm_cell<DIM>(L, i, j, k, zT2, zp2);
-        } else {
-#pragma unroll
-            for (int e = 0; e < 2; e++) {
-                const int i = bx * kNormCols + e * kBX + threadIdx.x;
-                if (i < L.n0) norm_cell<DIM>(L, i, j, k, zT2, zp2);
-            }
         }
     }
 }
 
 template <int DIM, bool RED, int ROWS>
-__device__ __forceinline__ double2 norm_block(const Level<double> &L, int bx, int by, int bz) {
-    double zT2 = 0.0, zp2 = 0.0;
-    norm_tile<DIM, RED, ROWS>(L, bx, by, bz, zT2, zp2);
-    block_sum2(zT2, zp2);
-    return make_double2(zT2, zp2);
+__device__ __forceinline__ void norm_tile(const Level<double> &L, int bx, int by, int bz, double &zT2, double &zp2) {
+    const int k = DIM == 3 ? bz : 0;
+#pragma unroll
+    for (int r = 0; r < ROWS; r++) norm_row<DIM, RED>(L, bx, (by * ROWS + r) * kBY + threadIdx.y, k, zT2, zp2);
 }
 
 template <int DIM, bool RED, bool P, int ROWS>
@@ -784,7 +784,20 @@ __device__ __forceinline__ void residual64_to32_cell(const Level<double> &L, flo
     }
 }
 
-// Block (bx, by, bz) of the norm grid.
+// Row j of tile column bx, and block (bx, by, bz), of the norm grid.
+template <int DIM>
+__device__ __forceinline__ void residual64_to32_row(const Level<double> &L, float2 *__restrict__ b32,
+                                                    float2 *__restrict__ bt32, float2 *__restrict__ e32,
+                                                    double2 *__restrict__ r_out, double2 *__restrict__ r_out2,
+                                                    int red_start, int bx, int j, int k, double &zT2, double &zp2) {
+    if (j >= L.n1) return;
+#pragma unroll
+    for (int e = 0; e < 2; e++) {
+        const int i = bx * kNormCols + e * kBX + threadIdx.x;
+        if (i < L.n0) residual64_to32_cell<DIM>(L, b32, bt32, e32, r_out, r_out2, red_start, i, j, k, zT2, zp2);
+    }
+}
+
 template <int DIM, int ROWS>
 __device__ __forceinline__ void residual64_to32_tile(const Level<double> &L, float2 *__restrict__ b32,
                                                      float2 *__restrict__ bt32, float2 *__restrict__ e32,
@@ -792,26 +805,9 @@ __device__ __forceinline__ void residual64_to32_tile(const Level<double> &L, flo
                                                      int red_start, int bx, int by, int bz, double &zT2, double &zp2) {
     const int k = DIM == 3 ? bz : 0;
 #pragma unroll
-    for (int r = 0; r < ROWS; r++) {
-        const int j = (by * ROWS + r) * kBY + threadIdx.y;
-        if (j >= L.n1) continue;
-#pragma unroll
-        for (int e = 0; e < 2; e++) {
-            const int i = bx * kNormCols + e * kBX + threadIdx.x;
-            if (i < L.n0) residual64_to32_cell<DIM>(L, b32, bt32, e32, r_out, r_out2, red_start, i, j, k, zT2, zp2);
-        }
-    }
-}
-
-template <int DIM, int ROWS>
-__device__ __forceinline__ double2 residual64_to32_block(const Level<double> &L, float2 *__restrict__ b32,
-                                                         float2 *__restrict__ bt32, float2 *__restrict__ e32,
-                                                         double2 *__restrict__ r_out, double2 *__restrict__ r_out2,
-                                                         int red_start, int bx, int by, int bz) {
-    double zT2 = 0.0, zp2 = 0.0;
-    residual64_to32_tile<DIM, ROWS>(L, b32, bt32, e32, r_out, r_out2, red_start, bx, by, bz, zT2, zp2);
-    block_sum2(zT2, zp2);
-    return make_double2(zT2, zp2);
+    for (int r = 0; r < ROWS; r++)
+        residual64_to32_row<DIM>(L, b32, bt32, e32, r_out, r_out2, red_start, bx, (by * ROWS + r) * kBY + threadIdx.y, k,
+                                 zT2, zp2);
 }
 
 template <int DIM, bool P, int ROWS>
