@@ -350,7 +350,7 @@ void plan(mg_handle *h, char *base, size_t *bytes) {
     CoarseProb &cp = h->cprob;
     std::memset(&cp, 0, sizeof(cp));
     cp.nc = h->nc;
-    cp.only = h->nlev == 1 && !mixed ? 1 : 0;
+    cp.tol = h->nlev == 1 && !mixed ? kCoarseTolOnly : kCoarseTol;
     for (int a = 0; a < 3; a++) cp.n[a] = c.n[a];
     if (h->coarse_factors) {
         bcr_shape(cp);

@@ -27,7 +27,7 @@
 // sub-partition whatever its lanes hold, a reciprocal 360, a cluster barrier
 // 400.
 // Both end with a check: a known vector is multiplied by the assembled matrix
-// and solved for.  If an entry comes back further off than coarse_tol (a zero
+// and solved for.  If an entry comes back further off than the tolerance (a zero
 // or tiny pivot block, growth, not-finite input), err[3] stays 0 and the banded
 // LU with partial pivoting that follows runs as the fallback, and reports a
 // singular matrix; otherwise err[3] = 1 and those kernels return at once.  A
@@ -66,10 +66,8 @@ struct CoarseProb {
     double *Minv;          // nc <= kBandSmemMax: the inverse, row-major
     float *Minv32;
     int *err;              // the handle's flags: [0] errors, [3] this path's factors are good
-    int only;              // the hierarchy's only level, solved in FP64: kCoarseTolOnly
+    double tol;            // of the check: kCoarseTol, or kCoarseTolOnly
 };
-
-__device__ __forceinline__ double coarse_tol(bool only) { return only ? kCoarseTolOnly : kCoarseTol; }
 
 __host__ __device__ inline long long bcr_work_doubles(int q, int m) {
     return (long long)kBcrArrays * m * q * q + 4LL * q * m;
@@ -257,7 +255,7 @@ __device__ __forceinline__ void coarse_invert(const CoarseProb &P, double *sm) {
             P.Minv[(long long)i * n + c] = v;
             if (P.Minv32) P.Minv32[(long long)i * n + c] = (float)v;
         },
-        sm, P.M, P.err + 3, coarse_tol(P.only));
+        sm, P.M, P.err + 3, P.tol);
 }
 
 // The e-th block of stage s.
@@ -576,7 +574,7 @@ __device__ __forceinline__ void bcr_check(const CoarseProb &P, double *sm) {
         },
         [&](int c, int a, double v) {
             const double z = bcr_known(2 * c + a);
-            if (!(fabs(v - z) <= coarse_tol(P.only) * z)) P.err[3] = 0;
+            if (!(fabs(v - z) <= P.tol * z)) P.err[3] = 0;
         },
         sm);
 }
