@@ -919,6 +919,8 @@ __device__ __forceinline__ void prep_rhs_cells(const Level<double> &L, const dou
     if (i >= L.n0 || j >= L.n1) return;
     const long long c = cell_id(i, j, k, L.n0, L.n1);
     const double2 q = rhs[c];
+    dq Di;
+    if (DIM == 2) Di = ldgq(L.Dinv + c);        // in flight with the right-hand side; in 3D the registers cost more
     double bT = q.x, bp = q.y;
     if (AXI) {
         const double s = r0 + (i + 0.5) * h;
@@ -931,7 +933,7 @@ __device__ __forceinline__ void prep_rhs_cells(const Level<double> &L, const dou
         bp -= g.y;
     }
     L.b[c] = make_double2(bT, bp);
-    const dq Di = ldgq(L.Dinv + c);
+    if (DIM == 3) Di = ldgq(L.Dinv + c);
     L.bt[c] = make_double2(Di.a * bT + Di.b * bp, Di.c * bT + Di.d * bp);
     if (xin) L.x[c] = xin[c];
     else if (zero) L.x[c] = make_double2(0.0, 0.0);
