@@ -60,3 +60,24 @@ def test_first_sweep_from_zero(torch_cuda, nu1, nu2):
         total = np.hypot(norms[:, f], norms[:, 2 + f])
         assert np.isfinite(total).all() and total[3] <= 0.5 * total[0], (nu1, nu2, total)
     c.close()
+
+
+@pytest.mark.parametrize("cycles", [1, 2])
+@pytest.mark.parametrize("nu1,nu2", [(0, 2), (1, 1), (2, 0), (3, 1)])
+def test_sweep_counts_match_the_oracle(torch_cuda, nu1, nu2, cycles):
+    """The cycle from a cleared correction (nu1 = 0), from its first colour, and without post-sweeps, within 1e-12 of the
+    oracle's in the deviation from the guess (the tolerance of the default counts)."""
+    from oracle import composite as cf
+    from paper_2206_11294_gb300.binding import Composite
+    b, p, box = I.composite_bubble(48, box=((0, 20), (0, 24)), seed=23, n_bubbles=1, rmin=0.08, rmax=0.12)
+    c = Composite(b.grid, box, nu1=nu1, nu2=nu2)
+    c.set_coeffs(b.lam, b.fa, b.fk, p.lam, p.fa, p.fk)
+    x = [_dev(torch_cuda, a) for a in (b.x0, p.x0)]
+    c.solve(_dev(torch_cuda, b.b), _dev(torch_cuda, p.b), *x, cycles=cycles, norms=False)
+    ref = cf.fac_solve(b.grid.as_dict(), box, b.lam, b.fa, b.fk, p.lam, p.fa, p.fk, b.b, p.b, b.x0, p.x0, cycles, nu1=nu1,
+                       nu2=nu2)
+    for got, want, start in zip(x, ref, (b.x0, p.x0)):
+        got = got.cpu().numpy().reshape(-1, 2)
+        for f in range(2):
+            assert np.abs(got[:, f] - want[:, f]).max() <= 1e-12 * np.abs(want[:, f] - start[:, f]).max()
+    c.close()
