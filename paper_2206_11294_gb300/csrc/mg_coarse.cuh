@@ -13,8 +13,8 @@
 //     pivot cell's columns are sent to all of them by distributed
 //     shared-memory stores, one cluster barrier per step);
 //   - above, the cells along the longest axis are the blocks of a block
-//     tridiagonal matrix (q unknowns per block, m blocks, m <= 31 x 2 for the
-//     grids served).  Stage s eliminates the blocks i with i + 1 = 2^s (mod
+//     tridiagonal matrix (q <= kGjMax unknowns per block, m blocks, q m at most
+//     2048, stages <= kBcrMaxStages; 31 x 31 cells: q 62, m 31).  Stage s eliminates the blocks i with i + 1 = 2^s (mod
 //     2^(s+1)): their diagonal blocks are inverted (the Gauss-Jordan clusters),
 //     and the remaining blocks' diagonals and couplings take dense products.
 //     A solve visits the stages down and up again: 2 log2(m) + 1 dependent
@@ -131,7 +131,8 @@ inline size_t gj_smem(int q) {
 // out at once, so that the chain of a step is: pivot rows, one update, the
 // determinant's reciprocal, the stores into the other CTAs, one cluster barrier;
 // the rest of the update runs beside it.  Bound by that chain while q is below
-// about 64, then by the FP64 pipe (q^2 / 8 FMA per step, CTA and clock pair).
+// about 64, then by the FP64 pipe (a CTA's q / 8 columns take q^2 / 4 FMA per
+// step, q^2 / 8 clocks at two a clock).
 // With `M` set (the whole coarsest matrix) the check follows.
 template <typename Load, typename Store>
 __device__ __forceinline__ void gj_invert(int q, Load load, Store store, double *sm, const double *M, int *flag,
@@ -333,7 +334,7 @@ __device__ __forceinline__ void bcr_update0(const CoarseProb &P, int job, int t,
 
 // 16 x 16 tile of base - sum of up to two products (sign -1) or of one product
 // (sign +1): one output per thread, the operands' rows and columns staged whole.
-// The FP64 pipe bounds it (a tile is 256 q FMA, 8 q clocks of an SM), so the
+// The FP64 pipe bounds it (a tile is 256 q FMA, 128 q clocks of an SM), so the
 // tile is small: the late stages have few products and need many tiles to fill
 // the chip.
 constexpr int kBcrTile = 16;

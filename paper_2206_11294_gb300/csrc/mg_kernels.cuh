@@ -78,7 +78,10 @@ __device__ __forceinline__ fq ldgq(const fq *p) {
 // while the kernel before it in the stream drains: its blocks are scheduled
 // as that kernel's last blocks exit, and pdl_entry() (griddepcontrol.wait)
 // returns once that kernel has completed and its writes are visible.  Every
-// such kernel calls it before it reads or writes anything.  Launched without
+// such kernel calls it before it reads or writes anything; k_vcycle_tail alone
+// stages coefficients and the coarsest inverse first, which are complete long
+// before: the host waits for the set-up's kernels, and the inverse's event is a
+// full dependency.  Launched without
 // the attribute it returns at once.  No kernel triggers its dependents early
 // (griddepcontrol.launch_dependents): blocks of the next grid scheduled while
 // this one still runs land on the SMs that free first, and small FP64 grids
