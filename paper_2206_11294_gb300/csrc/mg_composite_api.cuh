@@ -220,6 +220,7 @@ mg_status mg_composite_create(const mg_grid *grid, const int box[2][2], const mg
         delete m;
         return st;
     }
+    m->hb->cprob.tol = kCoarseTol;      // a correction, whose residual is taken anew, on a single level too
     m->Nb = (long long)g.n0 * g.n1;
     m->Nf = (long long)g.m0 * g.m1;
     m->nfb[0] = (long long)(g.n0 + 1) * g.n1;

@@ -288,6 +288,8 @@ mg_status mg_momentum_create(const mg_grid *grid, int flags, const mg_options *i
         mg_momentum_destroy(m);
         return fail(st, msg);
     }
+    m->hA->cprob.tol = kCoarseTol;      // a correction, whose residual is taken anew, on a single level too
+    if (dim == 3) m->hB->cprob.tol = kCoarseTol;
     m->N = (long long)grid->n[0] * grid->n[1] * grid->n[2];
     const dim3 gr = cell_grid(*grid);
     m->nblocks = (long long)gr.x * gr.y * gr.z;
